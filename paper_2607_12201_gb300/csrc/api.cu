@@ -572,9 +572,8 @@ collo_status collo_problem_create_conditions(const collo_network* net,
   pr->dz = A.alloc<double>(2 * (size_t)p);
   pr->thx = A.alloc<double>(8 * (size_t)p + 8);
   pr->fails = A.alloc<int>(1);
-  const size_t sweep_dim = (size_t)P.K * n;
-  const bool sweep_global = sweep_dim * (sweep_dim + 1) * sizeof(float) > 160 * 1024;
-  if (sweep_global) pr->sweep_work = A.alloc<float>(sweep_dim * (sweep_dim + 1));
+  const size_t sweep_floats = sweep_work_floats(P);
+  if (sweep_floats) pr->sweep_work = A.alloc<float>(sweep_floats);
   bool ok = P.react && P.prod && P.pidx && P.kfix && P.x0 && P.theta_lo && P.theta_hi &&
             (pr->host.cond_scale.empty() || P.kscale) &&
             P.nu_ptr && P.nu_r && P.nu_v && P.rs_ptr && P.rs_r && P.pr_ptr && P.pr_r && pat_ok &&
@@ -583,7 +582,7 @@ collo_status collo_problem_create_conditions(const collo_network* net,
             E.red && E.wtt && S.S && S.Sd && S.xth && S.inertia && S.diag && pr->sigma &&
             pr->kvec_a && pr->kvec_b && pr->kvec_r && pr->kvec_c && pr->thpart && pr->npart &&
             pr->scal && pr->red_parts && pr->x && pr->lam && pr->zl && pr->zu && pr->dz && pr->thx && pr->fails &&
-            (!sweep_global || pr->sweep_work);
+            (!sweep_floats || pr->sweep_work);
   if (!ok) { set_error("device allocation failed"); return COLLO_ERR_OOM; }
   if (cudaMallocHost(&pr->hscal, 64 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();

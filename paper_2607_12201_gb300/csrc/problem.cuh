@@ -39,13 +39,9 @@ cudaError_t launch_solve(const DevProb& P, const DevFactor<T>& F, const DevSchur
 
 // launchers (ipm.cu)
 cudaError_t launch_axpy(double* y, const double* x, double a, size_t n, cudaStream_t st);
-cudaError_t launch_forward_sweep(collo_problem* pr);
 
 cudaError_t launch_init_point_b(const DevInst* insts, const int* act, int A, double k1, double k2,
                                 cudaStream_t st);
-cudaError_t launch_sweep_b(const DevInst* insts, const int* act_warp, int A_warp,
-                           size_t smem_warp, const int* act_cta, int A_cta, size_t smem_cta,
-                           cudaStream_t st);
 cudaError_t launch_theta_prep_b(const DevInst* insts, const int* act, int A, const InstParams* prm,
                                 cudaStream_t st);
 cudaError_t launch_vec_reduce_b(const DevInst* insts, const int* act, int A, int which,
@@ -56,8 +52,13 @@ cudaError_t launch_trial_barrier_b(const DevInst* insts, const int* act, int A,
                                    const InstParams* prm, cudaStream_t st);
 cudaError_t launch_update_b(const DevInst* insts, const int* act, int A, const long long* pre,
                             long long total, const InstParams* prm, int mode, cudaStream_t st);
-size_t sweep_smem_bytes(const DevProb& P, bool jm_in_smem);
-size_t sweep_warp_smem_bytes(const DevProb& P);
+// forward sweep (sweep.cu): threads and dynamic shared memory of the largest
+// problem of the launch; floats of a problem's matrix in global memory (0: none)
+cudaError_t launch_sweep_b(const DevInst* insts, const int* act, int A, int threads, size_t smem,
+                           cudaStream_t st);
+size_t sweep_smem_bytes(const DevProb& P);
+int sweep_block_threads(const DevProb& P);
+size_t sweep_work_floats(const DevProb& P);
 // batched launchers (eval.cu, factor.cu); `reserve`: SMs the cooperative
 // grids leave to kernels of another stream
 cudaError_t launch_eval_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
@@ -248,7 +249,7 @@ struct collo_problem {
   double* dz = nullptr;       // [2p] bound-dual steps
   double* thx = nullptr;      // [2p] parameter-space helper vectors
   int* fails = nullptr;       // [1]
-  float* sweep_work = nullptr;   // forward-sweep FP32 Newton matrix when too big for smem
+  float* sweep_work = nullptr;   // forward-sweep FP32 matrix when too big for smem
   int64_t n_x = 0, n_c = 0;
   // grid-barrier wait settings of this problem's own runner
   // (collo_problem_set_wait_limit): polls before a wait gives up (0: default)

@@ -97,7 +97,7 @@ collo_status collo_time_phase(collo_problem* prob, int phase, int precision, int
     set_error("phase 2 (solve) needs a factorization in this precision");
     return COLLO_ERR_NOT_FACTORED;
   }
-  if (phase >= 1 && phase <= 3) return runner_time_phase(prob, phase, precision, reps, ms_per_launch);
+  if (phase >= 1 && phase <= 4) return runner_time_phase(prob, phase, precision, reps, ms_per_launch);
   auto launch = [&]() -> cudaError_t {
     switch (phase) {
       case 0:
@@ -105,8 +105,6 @@ collo_status collo_time_phase(collo_problem* prob, int phase, int precision, int
                                                  prob->fac_dc, prob->f32.F, st)
                      : launch_elem_factor<double>(prob->P, prob->E, prob->sigma, prob->fac_dw,
                                                   prob->fac_dc, prob->f64.F, st);
-      case 4:
-        return launch_forward_sweep(prob);
       default:
         return cudaErrorInvalidValue;
     }

@@ -44,9 +44,9 @@ struct Plan {
   cudaEvent_t ev_int = nullptr, ev_prm = nullptr;
   bool int_pending = false, prm_pending = false;
   size_t off_act = 0, off_elem = 0, off_lv = 0, off_cs_s = 0, off_cs_r = 0, off_f32 = 0,
-         off_f64 = 0, off_sw_w = 0, off_sw_c = 0;
-  int n_sw_w = 0, n_sw_c = 0;
-  size_t smem_eval = 0, smem_f[2] = {0, 0}, smem_sw_w = 0, smem_sw_c = 0;
+         off_f64 = 0;
+  int sweep_threads = 0;
+  size_t smem_eval = 0, smem_f[2] = {0, 0}, smem_sweep = 0;
   int cap_f[2] = {1 << 30, 1 << 30};
   int per_warp[2] = {0, 0};
   int rt_threads[2] = {0, 0};   // block size of the register-tiled element kernel
@@ -210,7 +210,7 @@ struct Runner {
     pl.max_p = maxp;
     pl.max_n = 0;
     for (int s : slots) pl.max_n = std::max(pl.max_n, P(s).np * P(s).n);
-    const size_t n_int = (size_t)A + (A + 1) * (size_t)(4 + maxL + 1) + 2 * (size_t)A + 2 * (size_t)A;
+    const size_t n_int = (size_t)A + (A + 1) * (size_t)(4 + maxL + 1) + 2 * (size_t)A;
     cudaError_t e = grow(&pl.d_int, &pl.h_int, &pl.cap_int, n_int);
     if (e == cudaSuccess) e = grow(&pl.d_ll, &pl.h_ll, &pl.cap_ll, (size_t)A + 1);
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return COLLO_ERR_OOM; }
@@ -307,24 +307,13 @@ struct Runner {
       pl.bcr_tpt = btpt;
       pl.bcr_full = bfull;
     }
-    // forward-sweep lists and eval shared memory
-    pl.off_sw_w = o;
-    pl.n_sw_w = 0; pl.smem_sw_w = 0;
-    for (int k = 0; k < A; ++k)
-      if (P(slots[k]).K * P(slots[k]).n <= 32) {
-        h[o + pl.n_sw_w++] = slots[k];
-        pl.smem_sw_w = std::max(pl.smem_sw_w, sweep_warp_smem_bytes(P(slots[k])));
-      }
-    o += A;
-    pl.off_sw_c = o;
-    pl.n_sw_c = 0; pl.smem_sw_c = 0;
-    for (int k = 0; k < A; ++k)
-      if (P(slots[k]).K * P(slots[k]).n > 32) {
-        h[o + pl.n_sw_c++] = slots[k];
-        pl.smem_sw_c = std::max(pl.smem_sw_c,
-                                sweep_smem_bytes(P(slots[k]), probs[slots[k]]->sweep_work == nullptr));
-      }
-    o += A;
+    // forward sweep: block size and shared memory of the largest problem
+    pl.sweep_threads = 0;
+    pl.smem_sweep = 0;
+    for (int k = 0; k < A; ++k) {
+      pl.sweep_threads = std::max(pl.sweep_threads, sweep_block_threads(P(slots[k])));
+      pl.smem_sweep = std::max(pl.smem_sweep, sweep_smem_bytes(P(slots[k])));
+    }
     pl.smem_eval = 0;
     for (int k = 0; k < A; ++k) pl.smem_eval = std::max(pl.smem_eval, eval_smem_bytes(P(slots[k])));
     pl.h_ll[0] = 0;
@@ -645,8 +634,7 @@ struct IpmInst {
 static collo_status ipm_begin_sweep(Runner& R, int which, const Opt& o, cudaStream_t st) {
   const Plan& pl = R.plans[which];
   COLLO_CUDA(launch_init_point_b(R.d_insts, pl.act(), pl.A, o.kappa1, o.kappa2, st));
-  COLLO_CUDA(launch_sweep_b(R.d_insts, pl.d_int + pl.off_sw_w, pl.n_sw_w, pl.smem_sw_w,
-                            pl.d_int + pl.off_sw_c, pl.n_sw_c, pl.smem_sw_c, st));
+  COLLO_CUDA(launch_sweep_b(R.d_insts, pl.act(), pl.A, pl.sweep_threads, pl.smem_sweep, st));
   return COLLO_OK;
 }
 
@@ -1148,7 +1136,8 @@ collo_status runner_solve(collo_problem* pr, int refine_max, double refine_tol, 
 }
 
 // CUDA-event timing of one batched phase of this problem (batch of one):
-// 1 factorization, 2 solve (no refinement), 3 evaluation with derivatives.
+// 1 factorization, 2 solve (no refinement), 3 evaluation with derivatives,
+// 4 forward sweep.
 collo_status runner_time_phase(collo_problem* pr, int phase, int prec, int reps, double* ms) {
   collo_status s = ensure_factor_storage(pr, prec);
   if (s != COLLO_OK) return s;
@@ -1160,6 +1149,12 @@ collo_status runner_time_phase(collo_problem* pr, int phase, int prec, int reps,
   auto run = [&]() -> collo_status {
     if (phase == 1) return R->factor(0, prec);
     if (phase == 2) return R->solve(0, prec, 0);
+    if (phase == 4) {
+      const Plan& pl = R->plans[0];
+      COLLO_CUDA(launch_sweep_b(R->d_insts, pl.act(), pl.A, pl.sweep_threads, pl.smem_sweep,
+                                R->stream));
+      return COLLO_OK;
+    }
     return R->eval(0, 1 /* V_X */, 0, 2 /* V_LAM */, true);
   };
   if ((s = run()) != COLLO_OK) return s;
@@ -1255,8 +1250,8 @@ collo_status collo_initial_states(collo_problem* prob, const double* theta, doub
                                R->stream));
   if ((s = R->set_plan(3, {0})) != COLLO_OK) return s;
   const Plan& pl = R->plans[3];
-  COLLO_CUDA(launch_sweep_b(R->d_insts, pl.d_int + pl.off_sw_w, pl.n_sw_w, pl.smem_sw_w,
-                            pl.d_int + pl.off_sw_c, pl.n_sw_c, pl.smem_sw_c, R->stream));
+  COLLO_CUDA(launch_sweep_b(R->d_insts, pl.act(), pl.A, pl.sweep_threads, pl.smem_sweep,
+                            R->stream));
   int f = 0;
   COLLO_CUDA(cudaMemcpyAsync(&f, prob->fails, sizeof(int), cudaMemcpyDeviceToHost, R->stream));
   if (x_out)
