@@ -55,12 +55,13 @@ __device__ inline void tri_tile(int t, int& ti, int& tj) {
   tj = t - i * (i + 1) / 2;
 }
 
-// Panel buffer leading dimension: odd (the per-row and per-column accesses of
-// the panel eliminations spread over the banks) and PANEL_PAD rows past msz, so
-// that every warp tile of trailing_update (rows below msz + 4 TR, columns below
-// msz + 4 TR + 8 TC) reads inside the buffer.
-constexpr int PANEL_PAD = 96;
-__host__ __device__ inline int panel_ld(int msz) { return (msz + PANEL_PAD) | 1; }
+// Panel buffer leading dimension: at least PANEL_PAD rows past msz, so that every
+// warp tile of trailing_update reads inside the buffer; a multiple of 4 (16-byte
+// loads of consecutive rows in trailing_update, of a column's diagonal part in
+// the panel eliminations) but not of 8, so that the column copies into it meet
+// at most four ways in a bank.
+constexpr int PANEL_PAD = 89;
+__host__ __device__ inline int panel_ld(int msz) { return (((msz + 92) >> 3) << 3) + 4; }
 
 // Trailing update of pair_eliminate_packed for kernels with a small register
 // budget (the cyclic-reduction blocks inside the cooperative factorization
@@ -122,89 +123,265 @@ __device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* 
   }
 }
 
+// Two FP32 values in one 64-bit register, and the packed multiply-add on them
+// (each half rounded like fmaf): half the issue slots of two scalar ones.
+__device__ inline unsigned long long pack2(float a, float b) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ inline void unpack2(unsigned long long d, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
+}
+__device__ inline unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                          unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// Accumulators of a register tile of TR consecutive rows and TC columns:
+// acc[u][v] += l[u] w[v].  FP32 rows go in packed pairs.
+template <typename T, int TR, int TC>
+struct TileAcc {
+  T a[TR][TC];
+  __device__ void clear() {
+#pragma unroll
+    for (int u = 0; u < TR; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) a[u][v] = T(0);
+  }
+  // l: TR consecutive entries (16-byte aligned), w: columns 8 entries apart
+  __device__ void add(const T* __restrict__ l, const T* __restrict__ w) {
+    T lr[TR], uc[TC];
+#pragma unroll
+    for (int u = 0; u < TR; u += 2) {
+      const double2 q = *reinterpret_cast<const double2*>(l + u);
+      lr[u] = q.x;
+      lr[u + 1] = q.y;
+    }
+#pragma unroll
+    for (int v = 0; v < TC; ++v) uc[v] = w[8 * v];
+#pragma unroll
+    for (int u = 0; u < TR; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) a[u][v] = fma(lr[u], uc[v], a[u][v]);
+  }
+  __device__ T get(int u, int v) const { return a[u][v]; }
+};
+template <int TR, int TC>
+struct TileAcc<float, TR, TC> {
+  unsigned long long a[TR / 2][TC];
+  __device__ void clear() {
+#pragma unroll
+    for (int u = 0; u < TR / 2; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) a[u][v] = 0ull;
+  }
+  __device__ void add(const float* __restrict__ l, const float* __restrict__ w) {
+    ulonglong2 lr[TR / 4];
+    unsigned long long uc[TC];
+#pragma unroll
+    for (int u = 0; u < TR / 4; ++u) lr[u] = reinterpret_cast<const ulonglong2*>(l)[u];
+#pragma unroll
+    for (int v = 0; v < TC; ++v) uc[v] = pack2(w[8 * v], w[8 * v]);
+#pragma unroll
+    for (int u = 0; u < TR / 4; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) {
+        a[2 * u][v] = fma2(lr[u].x, uc[v], a[2 * u][v]);
+        a[2 * u + 1][v] = fma2(lr[u].y, uc[v], a[2 * u + 1][v]);
+      }
+  }
+  __device__ float get(int u, int v) const {
+    float x, y;
+    unpack2(a[u >> 1][v], x, y);
+    return (u & 1) ? y : x;
+  }
+};
+
 // Trailing update of pair_eliminate_packed: A[r][c] -= sum_k Lp[k][r] W[k][c]
 // for cend <= c <= r < msz (packed lower triangle, shared or global memory),
 // the sum over k = 0..K-1 in ascending order, subtracted once.  Warp-blocked
 // register tiles: a warp owns 4 TR rows x 8 TC columns of the trailing
-// matrix, lane (ty, tx) = (lane / 8, lane % 8) the rows r0 + ty + 4u (u < TR)
-// and the columns c0 + tx + 8v (v < TC), so that for every k the warp reads
-// 4 TR entries of Lp[k] in runs of 4 and 8 TC entries of W[k] in runs of 8
-// (no bank conflicts), and each thread does TR TC multiply-adds per TR + TC
-// shared loads at fixed offsets from one address per k.  TR x TC is set by
+// matrix, lane (ty, tx) = (lane / 8, lane % 8) the TR consecutive rows r0 + TR
+// ty and the columns c0 + tx + 8v (v < TC): per k a thread's rows arrive in
+// 16-byte loads (broadcast over its eight lanes) and its columns in runs of
+// eight, and A is read and written in full 32-byte sectors.  Tiles start at a
+// multiple of four rows for those loads.  TR x TC is set by
 // the register budget of the calling kernel; out of line, so that the tile
 // gets the kernel's whole register budget.  Rows and columns past msz are
 // computed from the panel buffers' padding and never stored.
+// Bound: FP32 multiply-adds against shared-memory loads and issue slots.  In
+// isolation (K = 32, 16 warps) scalar multiply-adds with scalar loads reach 69 of
+// the SM's 128 lanes per clock, packed ones with 16-byte loads 88.
 template <typename T, int TR, int TC>
 __device__ __noinline__ void trailing_update(T* A, int msz, int cend, int K,
                                              const T* __restrict__ Lp, const T* __restrict__ W,
                                              int ldw) {
   constexpr int WR = 4 * TR, WC = 8 * TC;
-  static_assert(WR + WC <= PANEL_PAD, "panel buffers padded for the warp tile");
+  static_assert(WR <= PANEL_PAD && WC <= PANEL_PAD, "panel buffers padded for the warp tile");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int ty = lane >> 3, tx = lane & 7;
-  const int Tn = msz - cend;
-  if (Tn <= 0) return;
-  const int nbr = (Tn + WR - 1) / WR;
+  if (msz <= cend) return;
+  const int rbase = cend & ~3;
+  const int nbr = (msz - rbase + WR - 1) / WR;
   int blk = 0;
   for (int bi = 0; bi < nbr; ++bi) {
-    const int nbc = ((bi + 1) * WR + WC - 1) / WC;   // blocks meeting the lower triangle
+    // blocks meeting the lower triangle
+    const int nbc = (min(msz, rbase + (bi + 1) * WR) - cend + WC - 1) / WC;
     for (int bj = 0; bj < nbc; ++bj, ++blk) {
       if (blk % nw != warp) continue;
-      const int r0 = cend + bi * WR + ty, c0 = cend + bj * WC + tx;
-      // rows / columns past msz (fewer than WR + WC) read the padding of the
-      // panel buffers: indeterminate values in entries never stored
+      const int r0 = rbase + bi * WR + TR * ty, c0 = cend + bj * WC + tx;
       const T* lb = Lp + r0;
       const T* wb = W + c0;
       // the tile's entries are loaded first, so that their latency (the
       // triangle may be in global memory) overlaps the products
-      T cur[TR][TC], acc[TR][TC];
+      T cur[TR][TC];
 #pragma unroll
       for (int u = 0; u < TR; ++u)
 #pragma unroll
         for (int v = 0; v < TC; ++v) {
-          const int r = r0 + 4 * u, c = c0 + 8 * v;
+          const int r = r0 + u, c = c0 + 8 * v;
           cur[u][v] = (r < msz && c <= r) ? A[tri_at(r, c)] : T(0);
-          acc[u][v] = T(0);
         }
+      TileAcc<T, TR, TC> acc;
+      acc.clear();
 #pragma unroll 2
-      for (int k = 0; k < K; ++k) {
-        const T* lk = lb + k * ldw;
-        const T* wk = wb + k * ldw;
-        T lr[TR], uc[TC];
-#pragma unroll
-        for (int u = 0; u < TR; ++u) lr[u] = lk[4 * u];
-#pragma unroll
-        for (int v = 0; v < TC; ++v) uc[v] = wk[8 * v];
-#pragma unroll
-        for (int u = 0; u < TR; ++u)
-#pragma unroll
-          for (int v = 0; v < TC; ++v) acc[u][v] = fma(lr[u], uc[v], acc[u][v]);
-      }
+      for (int k = 0; k < K; ++k) acc.add(lb + k * ldw, wb + k * ldw);
 #pragma unroll
       for (int u = 0; u < TR; ++u) {
-        const int r = r0 + 4 * u;
+        const int r = r0 + u;
         if (r >= msz) continue;
 #pragma unroll
         for (int v = 0; v < TC; ++v) {
           const int c = c0 + 8 * v;
-          if (c <= r) A[tri_at(r, c)] = cur[u][v] - acc[u][v];
+          if (c <= r) A[tri_at(r, c)] = cur[u][v] - acc.get(u, v);
         }
       }
     }
   }
 }
 
+// Four (FP32) or two (FP64) consecutive entries at a 16-byte boundary.
+template <typename T>
+struct alignas(16) Quad {
+  T v[16 / sizeof(T)];
+};
+
+// One pair's update of a row's remaining panel columns: x[j] -= l0 U0[j] +
+// l1 U1[j] for j = kk + 2 .. 2 PB - 1, each by two multiply-adds.  U0, U1: the
+// pair's unscaled columns at the panel's own rows (the same for every row, read
+// as shared-memory broadcasts).  Entries past the panel's last column are
+// updated from whatever the buffer holds and not used.
+template <typename T, int PB>
+__device__ inline void pair_row_update(T (&x)[2 * PB], int kk, const T* __restrict__ U0,
+                                       const T* __restrict__ U1, T l0, T l1) {
+  constexpr int Q = 16 / sizeof(T);
+#pragma unroll
+  for (int g = 0; g < 2 * PB / Q; ++g) {
+    if (Q * g + Q - 1 < kk + 2) continue;
+    const Quad<T> u0 = reinterpret_cast<const Quad<T>*>(U0)[g];
+    const Quad<T> u1 = reinterpret_cast<const Quad<T>*>(U1)[g];
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+      if (Q * g + i >= kk + 2)
+        x[Q * g + i] = fma(-l1, u1.v[i], fma(-l0, u0.v[i], x[Q * g + i]));
+  }
+}
+
+// Pivot inverse (ia, ib, id) of the pair (a, b, d); zero where it has none.
+template <typename T>
+__device__ inline void pivot_inverse(T a, T b, T d, T& ia, T& ib, T& id) {
+  const T det = fma(a, d, -(b * b));
+  if (det != T(0) && isfinite(det)) {
+    const T inv = T(1) / det;
+    ia = d * inv; ib = -b * inv; id = a * inv;
+  } else {
+    ia = ib = id = T(0);
+  }
+}
+
+// The panel's diagonal block (rows and columns cp .. cp + K - 1, in W) by one
+// warp: lane r holds row cp + r in registers; a pair's two columns, final once
+// the earlier pairs are applied, go back to W, from where every lane reads them
+// and the pivot.  L columns of these rows to Lout, pivots to piv (shared).
+// Bound: the chain of pivots (a shared-memory round trip and a reciprocal per
+// pair).
+template <typename T, int PB>
+__device__ __noinline__ void panel_diag(T* W, int ldw, int cp, int K, T* __restrict__ Lout,
+                                        int lds, T (*piv)[3]) {
+  const int lane = threadIdx.x & 31;
+  T* Wr = W + cp + lane;
+  T x[2 * PB];
+#pragma unroll
+  for (int j = 0; j < 2 * PB; ++j) x[j] = (j <= lane && lane < K) ? Wr[j * ldw] : T(0);
+#pragma unroll
+  for (int kk = 0; kk < 2 * PB; kk += 2) {
+    if (kk >= K) break;
+    if (lane >= kk && lane < K) {
+      Wr[kk * ldw] = x[kk];
+      Wr[(kk + 1) * ldw] = x[kk + 1];
+    }
+    __syncwarp();
+    const T* U0 = W + kk * ldw + cp;
+    const T* U1 = U0 + ldw;
+    const T a = U0[kk], b = U0[kk + 1], d = U1[kk + 1];
+    T ia, ib, id;
+    pivot_inverse(a, b, d, ia, ib, id);
+    if (lane == 0) {
+      piv[kk >> 1][0] = a; piv[kk >> 1][1] = b; piv[kk >> 1][2] = d;
+    }
+    const T l0 = fma(x[kk], ia, x[kk + 1] * ib);
+    const T l1 = fma(x[kk], ib, x[kk + 1] * id);
+    if (lane > kk + 1 && lane < K) {
+      Lout[(size_t)(cp + kk) * lds + cp + lane] = l0;
+      Lout[(size_t)(cp + kk + 1) * lds + cp + lane] = l1;
+    }
+    pair_row_update<T, PB>(x, kk, U0, U1, l0, l1);
+  }
+}
+
+// The panel's eliminations on the rows below it (cp + K .. msz - 1), one thread
+// per row, the row's panel entries in registers: final unscaled entries back to
+// W, multipliers to Lp and Lout.  pinv: the pairs' pivot inverses.
+template <typename T, int PB>
+__device__ __noinline__ void panel_rows(T* W, T* Lp, int ldw, int msz, int cp, int K,
+                                        T* __restrict__ Lout, int lds, const T (*pinv)[3]) {
+  for (int r = cp + K + threadIdx.x; r < msz; r += blockDim.x) {
+    T x[2 * PB];
+#pragma unroll
+    for (int j = 0; j < 2 * PB; ++j) x[j] = j < K ? W[j * ldw + r] : T(0);
+    T* lo = Lout + (size_t)cp * lds + r;
+#pragma unroll
+    for (int kk = 0; kk < 2 * PB; kk += 2) {
+      if (kk >= K) break;
+      const T ia = pinv[kk >> 1][0], ib = pinv[kk >> 1][1], id = pinv[kk >> 1][2];
+      const T l0 = fma(x[kk], ia, x[kk + 1] * ib);
+      const T l1 = fma(x[kk], ib, x[kk + 1] * id);
+      if (kk > 0) {
+        W[kk * ldw + r] = x[kk];
+        W[(kk + 1) * ldw + r] = x[kk + 1];
+      }
+      Lp[kk * ldw + r] = l0;
+      Lp[(kk + 1) * ldw + r] = l1;
+      lo[(size_t)kk * lds] = l0;
+      lo[(size_t)(kk + 1) * lds] = l1;
+      pair_row_update<T, PB>(x, kk, W + kk * ldw + cp, W + (kk + 1) * ldw + cp, l0, l1);
+    }
+  }
+}
 
 // Eliminate the first npairs (state, multiplier) pairs of the symmetric msz x
 // msz matrix A, stored as a packed lower triangle (shared or global memory),
 // blocked right-looking: pairs are taken in panels of PB.  A panel's 2 PB
 // columns (rows >= the panel) are copied into W[j][r] (leading dimension
-// ldw = panel_ld(msz)).  One warp eliminates the panel's pairs on its own 2 PB rows
-// (the diagonal block), recording each pair's pivot inverse; then every
-// thread replays the same eliminations on the rows below, one row at a time
-// in registers (a row's multipliers depend only on the diagonal block), with
-// no barrier between pairs; then the trailing matrix receives one rank-2PB
-// update, in register tiles of TR x TC (4 x 4 per thread at a time for TR = 0),
+// ldw = panel_ld(msz)), those of the panel's own rows by warp 0, which
+// eliminates the panel's pairs on them (panel_diag) while the other warps copy
+// the rows below; then every thread replays the same eliminations on its rows
+// below (panel_rows; a row's multipliers depend only on the diagonal block);
+// then the trailing matrix receives one rank-2PB update, in register tiles of
+// TR x TC (4 x 4 per thread at a time for TR = 0),
 // from the multipliers Lp[j][r] and the unscaled columns W.  Every entry sees the arithmetic, in the order, of the
 // pair-by-pair elimination: the pivot inverse ia = d / det, ib = -b / det,
 // id = a / det; multipliers l0 = x0 ia + x1 ib, l1 = x0 ib + x1 id; the
@@ -212,83 +389,62 @@ __device__ __noinline__ void trailing_update(T* A, int msz, int cend, int K,
 // over the panel's 2 PB columns in ascending order, subtracted once
 // (trailing_update for TR x TC > 0, trailing_update_tiles4 for TR = 0).
 // L columns go to Lout[c * lds + r] (rows r > pair), pivots (a, b, d) to
-// Dout[3 q]; pivot inertia is counted by thread 0.  The trailing block (rows
-// and columns >= 2 npairs) is left in A.
+// Dout[3 q]; inert[0..2] receives the pivots' inertia (counted off the
+// elimination's path, by the last warp: its FP64 sign tests are slow).  The
+// trailing block (rows and columns >= 2 npairs) is left in A.
 // PB is 8 for blocks held in shared memory and 16 for blocks in the global
 // slab (half the trailing passes over global memory, twice the arithmetic per
 // entry read and written).
 template <typename T, int PB, int TR, int TC>
 __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__ Lout, int lds,
-                                      T* __restrict__ Dout, T* Lp, T* W, int& pos, int& neg,
-                                      int& zero) {
+                                      T* __restrict__ Dout, T* Lp, T* W,
+                                      int* __restrict__ inert) {
   const int tid = threadIdx.x, nt = blockDim.x, ldw = panel_ld(msz);
-  __shared__ T pinv[PB][3];   // pivot inverse (ia, ib, id) of the panel's pairs
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  __shared__ T piv[PB][3], pinv[PB][3];   // pivots and their inverses of the panel's pairs
+  int pos = 0, neg = 0, zero = 0;
   for (int q0 = 0; q0 < npairs; q0 += PB) {
     const int pe = min(q0 + PB, npairs);
-    const int cp = 2 * q0, cend = 2 * pe, K = cend - cp, rows = msz - cp;
-    // panel columns cp .. cend-1 for rows >= cp (the lower triangle; the
-    // entries above the diagonal are never read)
-    for (int idx = tid; idx < K * rows; idx += nt) {
-      const int r = cp + idx / K, j = idx - (r - cp) * K, c = cp + j;
-      if (c <= r) W[j * ldw + r] = A[tri_at(r, c)];
-    }
-    __syncthreads();
-    // 1. the diagonal block (rows cp .. cend-1), pair by pair, by warp 0
-    if (tid < 32) {
-      const int lane = tid;
-      for (int q = q0; q < pe; ++q) {
-        const int c0 = 2 * q, c1 = c0 + 1, kk = 2 * (q - q0);
-        const T a = W[kk * ldw + c0], b = W[kk * ldw + c1], d = W[(kk + 1) * ldw + c1];
-        const T det = fma(a, d, -(b * b));
-        T ia, ib, id;
-        if (det != T(0) && isfinite(det)) {
-          const T inv = T(1) / det;
-          ia = d * inv; ib = -b * inv; id = a * inv;
-        } else {
-          ia = ib = id = T(0);
+    const int cp = 2 * q0, cend = 2 * pe, K = cend - cp;
+    // panel columns cp .. cend-1 (the lower triangle; the entries above the
+    // diagonal are never used), 32 / (2 PB) rows per warp at a time
+    constexpr int RW = 32 / (2 * PB);
+    const int j = lane % (2 * PB), sub = lane / (2 * PB);
+    auto copy_rows = [&](int lo, int hi, int first, int step) {
+      constexpr int B = 8;   // loads in flight per lane
+      for (int r = lo + first * RW + sub; r < hi; r += B * step * RW) {
+        T v[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          const int ri = r + i * step * RW;
+          v[i] = (j < K && ri < hi && cp + j <= ri) ? A[tri_at(ri, cp + j)] : T(0);
         }
-        if (lane == 0) {
-          Dout[3 * q + 0] = a; Dout[3 * q + 1] = b; Dout[3 * q + 2] = d;
-          pinv[q - q0][0] = ia; pinv[q - q0][1] = ib; pinv[q - q0][2] = id;
-          pivot_inertia((double)a, (double)b, (double)d, pos, neg, zero);
-        }
-        const int r = c1 + 1 + lane;
-        if (r < cend) {
-          const T x0 = W[kk * ldw + r], x1 = W[(kk + 1) * ldw + r];
-          const T l0 = fma(x0, ia, x1 * ib);
-          const T l1 = fma(x0, ib, x1 * id);
-          Lout[(size_t)c0 * lds + r] = l0;
-          Lout[(size_t)c1 * lds + r] = l1;
-          for (int c = c1 + 1; c <= r; ++c) {   // remaining panel columns, c <= r
-            T& w = W[(c - cp) * ldw + r];
-            w = fma(-l1, W[(kk + 1) * ldw + c], fma(-l0, W[kk * ldw + c], w));
-          }
-        }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    // 2. rows below the panel: the same eliminations, each thread on its own
-    // rows (entries of row r are updated in place in W; the diagonal block's
-    // columns are read through a volatile view, loaded where used)
-    const volatile T* U = W;
-    for (int r = cend + tid; r < msz; r += nt) {
-      for (int kk = 0; kk < K; kk += 2) {
-        const T ia = pinv[kk >> 1][0], ib = pinv[kk >> 1][1], id = pinv[kk >> 1][2];
-        const T x0 = W[kk * ldw + r], x1 = W[(kk + 1) * ldw + r];
-        const T l0 = fma(x0, ia, x1 * ib);
-        const T l1 = fma(x0, ib, x1 * id);
-        Lp[kk * ldw + r] = l0;
-        Lp[(kk + 1) * ldw + r] = l1;
-        Lout[(size_t)(cp + kk) * lds + r] = l0;
-        Lout[(size_t)(cp + kk + 1) * lds + r] = l1;
-        for (int j = kk + 2; j < K; ++j) {
-          const int c = cp + j;
-          T& w = W[j * ldw + r];
-          w = fma(-l1, U[(kk + 1) * ldw + c], fma(-l0, U[kk * ldw + c], w));
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          const int ri = r + i * step * RW;
+          if (j < K && ri < hi && cp + j <= ri) W[j * ldw + ri] = v[i];
         }
       }
+    };
+    if (warp == 0) {
+      copy_rows(cp, cend, 0, 1);
+      __syncwarp();
+      panel_diag<T, PB>(W, ldw, cp, K, Lout, lds, piv);
+      __syncwarp();
+      if (lane < K / 2) {
+        pivot_inverse(piv[lane][0], piv[lane][1], piv[lane][2], pinv[lane][0], pinv[lane][1],
+                      pinv[lane][2]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) Dout[3 * (q0 + lane) + i] = piv[lane][i];
+      }
+    } else {
+      copy_rows(cend, msz, warp - 1, nw - 1);
     }
+    __syncthreads();
+    panel_rows<T, PB>(W, Lp, ldw, msz, cp, K, Lout, lds, pinv);
+    if (warp == nw - 1 && lane < K / 2)
+      pivot_inertia((double)piv[lane][0], (double)piv[lane][1], (double)piv[lane][2], pos, neg,
+                    zero);
     __syncthreads();
     // trailing rank-K update of rows / columns >= cend (lower part)
     if constexpr (TR == 0)
@@ -296,6 +452,12 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
     else
       trailing_update<T, TR, TC>(A, msz, cend, K, Lp, W, ldw);
     __syncthreads();
+  }
+  if (warp == nw - 1) {
+    pos = __reduce_add_sync(0xffffffffu, pos);
+    neg = __reduce_add_sync(0xffffffffu, neg);
+    zero = __reduce_add_sync(0xffffffffu, zero);
+    if (lane == 0) { inert[0] = pos; inert[1] = neg; inert[2] = zero; }
   }
 }
 
@@ -306,7 +468,7 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
 // global slab (L2-resident) and the panel buffers in shared memory, or, when
 // even they do not fit, in the slab behind the triangle.
 __host__ __device__ inline size_t big_tri_elems(int msz) {
-  return ((size_t)msz * (msz + 1) / 2 + 1) & ~size_t(1);
+  return ((size_t)msz * (msz + 1) / 2 + 3) & ~size_t(3);   // a multiple of 16 bytes
 }
 template <typename T>
 __host__ __device__ inline int big_pb(int msz) {
@@ -321,12 +483,12 @@ __host__ __device__ inline size_t big_panel_elems(int msz) {
 // whose panel buffers are sized for 16)
 template <typename T, int TR, int TC>
 __device__ inline void pair_eliminate_big(T* A, int msz, int npairs, T* __restrict__ Lout,
-                                          int lds, T* __restrict__ Dout, T* Lp, T* W, int& pos,
-                                          int& neg, int& zero, int pb) {
+                                          int lds, T* __restrict__ Dout, T* Lp, T* W,
+                                          int* __restrict__ inert, int pb) {
   if (pb == 16)
-    pair_eliminate_packed<T, 16, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, pos, neg, zero);
+    pair_eliminate_packed<T, 16, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
   else
-    pair_eliminate_packed<T, 8, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, pos, neg, zero);
+    pair_eliminate_packed<T, 8, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
 }
 template <typename T>
 __host__ __device__ inline bool panel_in_global(int msz) {
@@ -394,12 +556,9 @@ __device__ void elem_factor_big(const DevProb& P, const DevEval& E,
                   E.Wzt + (size_t)e * K * np, E.JT + (size_t)e * K * np,
                   E.Wobj + (size_t)e * npt * npt * n,
                   sigma ? sigma + (size_t)e * npt * n : nullptr, dw, dc, A);
-  int pos = 0, neg = 0, zero = 0;
   pair_eliminate_big<T, TR, TC>(A, ext, nint, F.Lel + (size_t)e * (2 * nint) * ext, ext,
-                        F.Del + (size_t)e * nint * 3, pl.Lp, pl.W, pos, neg, zero, pb);
-  if (tid == 0) {
-    F.inert[e * 3 + 0] = pos; F.inert[e * 3 + 1] = neg; F.inert[e * 3 + 2] = zero;
-  }
+                                F.Del + (size_t)e * nint * 3, pl.Lp, pl.W,
+                                F.inert + (size_t)e * 3, pb);
   const int n2 = 2 * n;
   auto tr = [&](int a, int b) { return a >= b ? A[tri_at(a, b)] : A[tri_at(b, a)]; };
   double* Sc = F.Scon + (size_t)e * p * p;
@@ -434,7 +593,7 @@ template <typename T>
 __global__ void __launch_bounds__(FBS)
 k_elem_factor(DevProb P, DevEval E, const double* __restrict__ sigma, double dw, double dc,
               DevFactor<T> F, int use_smem, int slab_pb) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const BigPlace<T> pl = big_place<T>(smraw, F.work, P.ext, use_smem != 0);
   for (int e = blockIdx.x; e < P.N; e += gridDim.x)
     elem_factor_big<T, 8, sizeof(T) == 4 ? 8 : 4>(P, E, sigma, dw, dc, F, e, pl,
@@ -1040,13 +1199,9 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
       A[tri_at(a, b)] = v;
     }
   __syncthreads();
-  int pos = 0, neg = 0, zero = 0;
   pair_eliminate_big<T, TR, TC>(A, bext, n, F.Lb + (size_t)i * n2 * bext, bext,
-                        F.Db + (size_t)i * n * 3, pl.Lp, pl.W, pos, neg, zero, pb);
-  if (tid == 0) {
-    int* in = F.inert + (size_t)(N + i) * 3;
-    in[0] = pos; in[1] = neg; in[2] = zero;
-  }
+                                F.Db + (size_t)i * n * 3, pl.Lp, pl.W,
+                                F.inert + (size_t)(N + i) * 3, pb);
   // scatter the trailing (Schur) block into the neighbours
   auto tr = [&](int a, int b) { return a >= b ? A[tri_at(a, b)] : A[tri_at(b, a)]; };
   if (L >= 0) {
@@ -1223,7 +1378,7 @@ __host__ __device__ inline int bcr_level_blocks(int N, int stride) {
 template <typename T, int BT>
 __global__ void __launch_bounds__(FBS)
 k_bcr_factor(DevProb P, DevFactor<T> F, int stride, int final_level, int use_smem, int slab_pb) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
   if constexpr (BT > 0) {
     // two blocks of the level per CUDA block, one per half
@@ -1716,7 +1871,7 @@ __device__ void elem_bwd_one(const DevProb& P, const DevFactor<T>& F, const DevS
 template <typename T>
 __global__ void __launch_bounds__(32 * SOLVE_WARPS)
 k_elem_fwd(DevProb P, DevFactor<T> F, const double* __restrict__ b) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int warp = threadIdx.x >> 5;
   const int e = blockIdx.x * SOLVE_WARPS + warp;
   if (e >= P.N) return;
@@ -1726,7 +1881,7 @@ k_elem_fwd(DevProb P, DevFactor<T> F, const double* __restrict__ b) {
 template <typename T>
 __global__ void __launch_bounds__(32 * SOLVE_WARPS)
 k_bcr_fwd(DevProb P, DevFactor<T> F, int stride, int final_level) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int warp = threadIdx.x >> 5;
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
   const int bi = blockIdx.x * SOLVE_WARPS + warp;
@@ -1738,7 +1893,7 @@ template <typename T>
 __global__ void __launch_bounds__(32 * SOLVE_WARPS)
 k_bcr_bwd(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int stride,
           int final_level) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int warp = threadIdx.x >> 5;
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
   const int bi = blockIdx.x * SOLVE_WARPS + warp;
@@ -1750,7 +1905,7 @@ k_bcr_bwd(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int s
 template <typename T>
 __global__ void __launch_bounds__(32 * SOLVE_WARPS)
 k_elem_bwd(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int warp = threadIdx.x >> 5;
   const int e = blockIdx.x * SOLVE_WARPS + warp;
   if (e >= P.N) return;
@@ -1855,7 +2010,7 @@ __global__ void __launch_bounds__(BS, BS == 256 ? 2 : 1)
 k_elem_factor_big_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
                     const int* __restrict__ pre_elem, const InstParams* __restrict__ prm,
                     const int* __restrict__ flags, int slab_pb) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   for (int t = blockIdx.x; t < pre_elem[A]; t += gridDim.x) {
     const int k = find_item(pre_elem, A, t);
     if (flags[k] & 4) continue;   // condensed by k_elem_factor_rt_b
@@ -1882,7 +2037,7 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
            const int* __restrict__ pre_cs, const InstParams* __restrict__ prm,
            const int* __restrict__ flags, GridBar* gb, size_t smem_bytes, int bcr_full,
            int slab_pb) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   unsigned int ep = 0;
   // 1. element condensation: done by k_elem_factor_rt_b / k_elem_factor_big_b
   // before this launch
@@ -1987,7 +2142,7 @@ __global__ void __launch_bounds__(FBS)
 k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
           const int* __restrict__ pre_elem, const int* __restrict__ pre_lv, int maxL, int lsplit,
           const int* __restrict__ pre_cs, int ir, int per_warp, GridBar* gb) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   unsigned int ep = 0;
   const int warp = threadIdx.x >> 5, wpb = FBS / 32;
   const int gw = blockIdx.x * wpb + warp, nw = gridDim.x * wpb;
