@@ -80,12 +80,12 @@ template <typename T, class Fn>
 static void factor_layout(const DevProb& P, int n_slabs, DevFactor<T>& F, Fn&& fn) {
   const size_t N = P.N, n = P.n, p = P.p;
   const size_t K = P.K;
-  fn(F.Lel, N * 2 * K * n * P.ext);
+  fn(F.Lel, N * 2 * K * n * factor_ld<T>(P.ext));
   fn(F.Del, N * K * n * 3);
   fn(F.Aif, N * 4 * n * n);
   fn(F.Cpl, N * n * n);
   fn(F.Bif, N * 2 * n * p);
-  fn(F.Lb, N * 2 * n * P.bext);
+  fn(F.Lb, N * 2 * n * factor_ld<T>(P.bext));
   fn(F.Db, N * n * 3);
   fn(F.Scon, 2 * N * p * p);
   fn(F.inert, 2 * N * 3);

@@ -123,15 +123,22 @@ struct GridBar {
   long long spin_limit; // polls before a wait gives up (0: GRID_SPIN_LIMIT)
 };
 
+// Leading dimension of L columns of m rows: whole 16-byte quantities.
+template <typename T>
+__host__ __device__ inline int factor_ld(int m) {
+  constexpr int Q = 16 / sizeof(T);
+  return (m + Q - 1) / Q * Q;
+}
+
 // Factorization storage (T = double or float).
 template <typename T>
 struct DevFactor {
-  T* Lel;        // [N][2Kn][ext]  element interior L columns (column-major)
+  T* Lel;        // [N][2Kn][factor_ld(ext)]  element interior L columns (column-major)
   T* Del;        // [N][Kn][3]     element interior 2x2 pivots (a, b, d)
   T* Aif;        // [N][2n][2n]    chain blocks (full symmetric)
   T* Cpl;        // [N][n][n]      coupling K[c0 of block, chain state of left neighbour]
   T* Bif;        // [N][2n][p]     interface border
-  T* Lb;         // [N][2n][bext]  cyclic-reduction L columns
+  T* Lb;         // [N][2n][factor_ld(bext)]  cyclic-reduction L columns
   T* Db;         // [N][n][3]      cyclic-reduction 2x2 pivots
   double* Scon;  // [2N][p][p]     parameter Schur contributions
   int* inert;    // [2N][3]        (pos, neg, zero) per factored block
@@ -155,18 +162,22 @@ constexpr int CHUNKS = 64;
 __host__ __device__ inline int n_chunks(int C) { return C < CHUNKS ? (C > 0 ? C : 1) : CHUNKS; }
 
 struct DevSchur {
-  double* S;       // [p][p] assembled, then overwritten by L (unit lower) and D;
-                   // followed by [p] of scratch (schur_doubles), the multiplier
-                   // row of the factorization when it runs in global memory
+  double* S;       // L (unit lower), entry (r, c) at c schur_ld(p) + r; the matrix
+                   // itself and scratch behind it (schur_doubles) when it is
+                   // factored in global memory
   double* Sd;      // [p] pivots
   double* xth;     // [p] parameter solution
   long long* inertia;  // [3] total inertia
   double* diag;    // [p] W_thth + sigma_theta + delta_w (assembled by host-side launch)
 };
 
-// Doubles of DevSchur::S: the p x p block and the p-entry multiplier row the
-// factorization uses when the block does not fit in shared memory.
-inline size_t schur_doubles(int p) { return (size_t)p * p + (size_t)p; }
+// Leading dimension of the parameter factor: whole 16-byte quantities.
+__host__ __device__ inline int schur_ld(int p) { return factor_ld<double>(p); }
+// Doubles of DevSchur::S: the factor, and three columns of multipliers for the
+// factorization when it does not fit in shared memory.
+__host__ __device__ inline size_t schur_doubles(int p) {
+  return (size_t)p * schur_ld(p) + 3 * (size_t)p;
+}
 
 // ---- batched execution ------------------------------------------------------------
 // Everything one instance owns on the device, gathered for batched kernels.

@@ -25,11 +25,14 @@
 // Inertia is counted from every pivot block (Sylvester's law of inertia).
 // T = double (plain path) or float (mixed path; residuals and refinement
 // are FP64 elsewhere).
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "collo_internal.cuh"
+#include "subst.cuh"
 
 namespace collo {
 
@@ -556,7 +559,8 @@ __device__ void elem_factor_big(const DevProb& P, const DevEval& E,
                   E.Wzt + (size_t)e * K * np, E.JT + (size_t)e * K * np,
                   E.Wobj + (size_t)e * npt * npt * n,
                   sigma ? sigma + (size_t)e * npt * n : nullptr, dw, dc, A);
-  pair_eliminate_big<T, TR, TC>(A, ext, nint, F.Lel + (size_t)e * (2 * nint) * ext, ext,
+  const int ldl = factor_ld<T>(ext);
+  pair_eliminate_big<T, TR, TC>(A, ext, nint, F.Lel + (size_t)e * (2 * nint) * ldl, ldl,
                                 F.Del + (size_t)e * nint * 3, pl.Lp, pl.W,
                                 F.inert + (size_t)e * 3, pb);
   const int n2 = 2 * n;
@@ -656,18 +660,6 @@ struct Pivot {
 __device__ inline float recip_rn(float x) { return __frcp_rn(x); }
 __device__ inline double recip_rn(double x) { return __drcp_rn(x); }
 
-// Asynchronous copies (cp.async, completed by cp_async_wait_all) of single
-// elements from global to shared memory.
-template <typename T>
-__device__ inline void cp_async_elem(T* dst, const T* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 constexpr int RT_MAX_PAIRS = 2 * RT_MAX_TR + 2;   // pairs of a block of <= 124 rows
 constexpr int RT_MAX_THREADS = 512;               // threads of a register-tiled block
 
@@ -1091,7 +1083,9 @@ __device__ void elem_factor_rt(const DevProb& P, const DevEval& E,
   auto sink = [&](int r, int c, T val) { blk[tri_at(r, c)] = val; };
   __shared__ Pivot<T> pivs[RT_MAX_PAIRS];
   __shared__ int cnt[3];
-  pair_eliminate_rt<T, TPT, true>(tid, nt, ext, nint, entry, F.Lel + (size_t)e * (2 * nint) * ext, ext,
+  const int ldl = factor_ld<T>(ext);
+  pair_eliminate_rt<T, TPT, true>(tid, nt, ext, nint, entry,
+                            F.Lel + (size_t)e * (2 * nint) * ldl, ldl,
                             F.Del + (size_t)e * nint * 3, sink, CtaBar{}, ub, pivs, cnt);
   if (tid == 0) {
     F.inert[e * 3 + 0] = cnt[0]; F.inert[e * 3 + 1] = cnt[1]; F.inert[e * 3 + 2] = cnt[2];
@@ -1199,7 +1193,8 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
       A[tri_at(a, b)] = v;
     }
   __syncthreads();
-  pair_eliminate_big<T, TR, TC>(A, bext, n, F.Lb + (size_t)i * n2 * bext, bext,
+  const int ldl = factor_ld<T>(bext);
+  pair_eliminate_big<T, TR, TC>(A, bext, n, F.Lb + (size_t)i * n2 * ldl, ldl,
                                 F.Db + (size_t)i * n * 3, pl.Lp, pl.W,
                                 F.inert + (size_t)(N + i) * 3, pb);
   // scatter the trailing (Schur) block into the neighbours
@@ -1306,7 +1301,8 @@ __device__ void bcr_factor_staged(const DevProb& P, const DevFactor<T>& F, int s
   // is collected in the staging buffer (the inputs are in registers by now) ...
   const int b2 = 2 * n;
   auto sink = [&](int r, int c, T val) { stage[tri_at(r - b2, c - b2)] = val; };
-  pair_eliminate_rt<T, TPT, false>(tid, 128, bext, n, entry, F.Lb + (size_t)i * n2 * bext, bext,
+  const int ldl = factor_ld<T>(bext);
+  pair_eliminate_rt<T, TPT, false>(tid, 128, bext, n, entry, F.Lb + (size_t)i * n2 * ldl, ldl,
                             F.Db + (size_t)i * n * 3, sink, bar, ub, pivs, cnt);
   if (tid == 0) {
     int* in = F.inert + (size_t)(N + i) * 3;
@@ -1432,38 +1428,83 @@ cudaError_t launch_chunk_sums(const double* X, int C, int L, double* part, cudaS
   return cudaGetLastError();
 }
 
+// Sum of the chunk sums of entry l, by one thread: four interleaved partial sums,
+// sixteen loads in flight.
 __device__ inline double sum_chunks(const double* __restrict__ part, int G, int L, int l) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int g = 0;
-  for (; g + 3 < G; g += 4) {
-    a0 += part[(size_t)g * L + l];
-    a1 += part[(size_t)(g + 1) * L + l];
-    a2 += part[(size_t)(g + 2) * L + l];
-    a3 += part[(size_t)(g + 3) * L + l];
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  const int G4 = G & ~3;
+  for (int g0 = 0; g0 < G4; g0 += 16) {
+    double v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = g0 + i < G4 ? part[(size_t)(g0 + i) * L + l] : 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (g0 + i < G4) a[i & 3] += v[i];
   }
-  for (; g < G; ++g) a0 += part[(size_t)g * L + l];
-  return (a0 + a1) + (a2 + a3);
+  for (int g = G4; g < G; ++g) a[0] += part[(size_t)g * L + l];
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+// Total of entry idx of the p x p contributions, left in its first chunk's place
+// (by the one thread that handles the entry); only the lower triangle is used.
+__device__ inline void schur_total(double* chunkS, int N, int p, int idx) {
+  const int q = idx / p, q2 = idx - q * p;
+  if (q2 <= q) chunkS[idx] = sum_chunks(chunkS, n_chunks(2 * N), p * p, idx);
+}
+__global__ void __launch_bounds__(CS_BS) k_schur_total(double* chunkS, int N, int p) {
+  const int idx = blockIdx.x * CS_BS + threadIdx.x;
+  if (idx < p * p) schur_total(chunkS, N, p, idx);
+}
+
+// The same sum by four neighbouring lanes (part 0 .. 3 of a quad, the whole warp
+// calling): the four partial sums of sum_chunks, each with its loads in flight
+// at once, added in its order; every lane of the quad returns it.
+__device__ inline double sum_chunks4(const double* __restrict__ part, int G, int L, int l,
+                                     int quarter) {
+  const int G4 = G & ~3;
+  double a = 0.0;
+  for (int g0 = quarter; g0 < G4; g0 += 32) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = g0 + 4 * i < G4 ? part[(size_t)(g0 + 4 * i) * L + l] : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (g0 + 4 * i < G4) a += v[i];
+  }
+  if (quarter == 0)
+    for (int g = G4; g < G; ++g) a += part[(size_t)g * L + l];
+  const unsigned m = __activemask();
+  a += __shfl_xor_sync(m, a, 1);
+  return a + __shfl_xor_sync(m, a, 2);
 }
 
 constexpr int SBS = 256;
-// One block: S = (chunk sums of all contributions) + diag(W_thth + sigma + dw),
-// FP64 LDL^T with 1x1 pivots, total inertia.  sS: [p][p] followed by a
-// p-entry multiplier row, in dynamic shared memory, or S.S itself when that
-// does not fit (S.S holds p p + p doubles for this).
+// One block: S = (total of all contributions, schur_total) + diag(W_thth + sigma +
+// dw), FP64 LDL^T with 1x1 pivots, total inertia.  work: schur_doubles(p) doubles
+// in dynamic shared memory, or S.S itself when that does not fit: the matrix,
+// lower triangle column-major (entry (r, c) at c ld + r, the layout of the
+// factor left in S.S), and three columns of multipliers.
+// Bound: the chain of pivots, each a reciprocal (some 400 cycles in FP64) behind
+// the update of its column.  Warp 0 updates column k + 1 first and inverts its
+// pivot while the other warps apply column k to the columns beyond: one barrier
+// per column, and the reciprocal is off the other warps' path.
 __device__ void schur_block(const DevProb& P, const int* __restrict__ inert,
-                            const double* __restrict__ chunkS, const double* __restrict__ wtt,
+                            const double* __restrict__ total, const double* __restrict__ wtt,
                             const double* __restrict__ sigma, double dw, const DevSchur& S,
-                            double* sS) {
+                            double* work) {
   __shared__ long long cnt[3];
   __shared__ long long red[3][SBS];
-  const int p = P.p, N = P.N, tid = threadIdx.x;
+  const int p = P.p, N = P.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ld = schur_ld(p);
   const size_t nz = (size_t)N * P.np * P.n;
-  double* l = sS + (size_t)p * p;
+  double* A = work;
+  double* lbuf = A + (size_t)p * ld;
   for (int idx = tid; idx < p * p; idx += SBS) {
     const int q = idx / p, q2 = idx - q * p;
-    double v = sum_chunks(chunkS, n_chunks(2 * N), p * p, idx);
+    if (q2 > q) continue;
+    double v = total[idx];
     if (q == q2) v += wtt[q] + (sigma ? sigma[nz + q] : 0.0) + dw;
-    sS[idx] = v;
+    A[(size_t)q2 * ld + q] = v;
   }
   {
     long long a = 0, b = 0, c = 0;
@@ -1477,26 +1518,46 @@ __device__ void schur_block(const DevProb& P, const int* __restrict__ inert,
     if (tid == 0) { cnt[0] = red[0][0]; cnt[1] = red[1][0]; cnt[2] = red[2][0]; }
   }
   __syncthreads();
-  for (int k = 0; k < p; ++k) {
-    const double d = sS[k * p + k];
+  // multipliers of column k (final) into buffer k % 3, its pivot counted; warp 0
+  auto finish = [&](int k) {
+    const double d = A[(size_t)k * ld + k];
     const bool ok = (d != 0.0) && isfinite(d);
     const double inv = ok ? 1.0 / d : 0.0;
-    for (int r = k + 1 + tid; r < p; r += SBS) l[r] = sS[r * p + k] * inv;
-    if (tid == 0) {
+    double* l = lbuf + (size_t)(k % 3) * p;
+    for (int r = k + 1 + lane; r < p; r += 32) l[r] = A[(size_t)k * ld + r] * inv;
+    if (lane == 0) {
       if (!ok) cnt[2] += 1; else if (d > 0) cnt[0] += 1; else cnt[1] += 1;
       S.Sd[k] = d;
     }
-    __syncthreads();
-    const int w = p - k - 1;
-    for (int idx = tid; idx < w * w; idx += SBS) {
-      const int r = k + 1 + idx / w, c = k + 1 + idx % w;
-      if (c <= r) sS[r * p + c] -= l[r] * sS[c * p + k];
+  };
+  // column c -= l u[c], rows c .. p - 1
+  auto apply = [&](int c, const double* l, const double* u) {
+    const double uc = u[c];
+    double* col = A + (size_t)c * ld;
+    for (int r = c + lane; r < p; r += 32) col[r] = fma(-l[r], uc, col[r]);
+  };
+  if (warp == 0 && p > 0) finish(0);
+  __syncthreads();
+  for (int k = 0; k < p; ++k) {
+    const double* l = lbuf + (size_t)(k % 3) * p;
+    const double* u = A + (size_t)k * ld;
+    if (warp == 0) {
+      if (k + 1 < p) {
+        apply(k + 1, l, u);
+        __syncwarp();
+        finish(k + 1);
+      }
+    } else {
+      // the multipliers of the column before leave for S.S (where they may
+      // replace the column itself, which nobody reads any more)
+      if (warp == 1 && k > 0) {
+        const double* lp = lbuf + (size_t)((k - 1) % 3) * p;
+        for (int r = k + lane; r < p; r += 32) S.S[(size_t)(k - 1) * ld + r] = lp[r];
+      }
+      for (int c = k + 1 + warp; c < p; c += SBS / 32 - 1) apply(c, l, u);
     }
     __syncthreads();
-    for (int r = k + 1 + tid; r < p; r += SBS) sS[r * p + k] = l[r];
-    __syncthreads();
   }
-  for (int idx = tid; idx < p * p; idx += SBS) S.S[idx] = sS[idx];
   if (tid == 0) { S.inertia[0] = cnt[0]; S.inertia[1] = cnt[1]; S.inertia[2] = cnt[2]; }
   __syncthreads();
 }
@@ -1509,8 +1570,68 @@ k_schur(DevProb P, const int* __restrict__ inert, const double* __restrict__ chu
   schur_block(P, inert, chunkS, wtt, sigma, dw, S, in_global ? S.S : sS);
 }
 
-// ---- solves: one warp per block ----------------------------------------------------
-constexpr int SOLVE_WARPS = 4;
+// ---- solves: one warp or one CUDA block per block ------------------------------------
+// Blocks of at most SOLVE_NARROW rows are solved by one warp each, eight at a
+// time in a CUDA block; larger ones by the whole CUDA block (subst.cuh).  One
+// solve against one warp per block throughout, two columns loaded per step: 10
+// species, 400 elements 148 -> 128 us; 27 species, 415 elements 483 -> 206 us; 50
+// species, 2000 elements 1743 -> 969 us.
+constexpr int SOLVE_NARROW = 128;
+constexpr int SOLVE_G = FBS / 32;   // warps of a wide block's group
+__host__ __device__ inline bool elem_solve_wide(const DevProb& P) { return P.ext > SOLVE_NARROW; }
+__host__ __device__ inline bool bcr_solve_wide(const DevProb& P) { return P.bext > SOLVE_NARROW; }
+// Dynamic shared memory of a solve kernel: narrow blocks of at most pn rows, wide
+// ones of at most pw, a parameter block of max_p (each 0: none).  Three panels in
+// flight per group (two, one), if two CUDA blocks then still fit an SM; else as
+// many as one block has room for.  With many narrow blocks (several for each warp
+// the device holds) one panel: twice the warps hide the latency better than
+// the second panel does (32 problems of 10 species: 362 against 302 us a solve).
+template <typename T, int G>
+static size_t group_smem(int msz, int groups, int most = SUB_STAGES) {
+  const size_t v = sizeof(T) * sub_vec_elems(msz), pn = sub_slot_bytes<T, G>(msz);
+  auto bytes = [&](int st) { return groups * ((v + st * pn + 15) & ~size_t(15)); };
+  for (size_t cap : {size_t(110), size_t(200)})
+    for (int st = most; st > 1; --st)
+      if (bytes(st) <= cap * 1024) return bytes(st);
+  return bytes(1);
+}
+template <typename T>
+size_t solve_smem(int pn, bool many, int pw, int max_p) {
+  size_t b = max_p > 0 ? group_smem<double, SOLVE_G>(max_p, 1) : 0;
+  if (pn > 0) b = std::max(b, group_smem<T, 1>(pn, SOLVE_G, many ? 1 : SUB_STAGES));
+  if (pw > 0) b = std::max(b, group_smem<T, SOLVE_G>(pw, 1));
+  return b;
+}
+// The part of the `bytes` of dynamic shared memory of this thread's group: all for
+// G > 1 (blocks of up to msz rows), this warp's share for G = 1.
+template <typename T, int G>
+__device__ inline SubMem<T, G> sub_mem(unsigned char* sm, size_t bytes, int msz,
+                                       unsigned long long* bars, int* err) {
+  if constexpr (G > 1) {
+    return sub_carve<T, G>(sm, bytes, msz, bars, err);
+  } else {
+    const int warp = threadIdx.x >> 5;
+    const size_t share = (bytes / SOLVE_G) & ~size_t(15);
+    return sub_carve<T, 1>(sm + warp * share, share, msz, bars + warp * SUB_STAGES, err);
+  }
+}
+constexpr int SOLVE_BARS = SOLVE_G * SUB_STAGES;   // barriers of a kernel's narrow groups
+
+// The L columns of element e and of reduction block i.
+template <typename T>
+__device__ inline FactorCols<T> elem_cols(const DevProb& P, const DevFactor<T>& F, int e) {
+  const int ld = factor_ld<T>(P.ext), nc = 2 * P.K * P.n;
+  return {F.Lel + (size_t)e * nc * ld, ld, P.ext, nc};
+}
+template <typename T>
+__device__ inline FactorCols<T> bcr_cols(const DevProb& P, const DevFactor<T>& F, int i) {
+  const int ld = factor_ld<T>(P.bext), nc = 2 * P.n;
+  return {F.Lb + (size_t)i * nc * ld, ld, P.bext, nc};
+}
+// Block bi of the level with this stride (final_level: the last block).
+__device__ inline int bcr_block(int stride, int final_level, int bi) {
+  return final_level ? 0 : stride * (2 * bi + 1);
+}
 
 template <typename T>
 __device__ inline void pair_solve_d(T a, T b, T d, T w0, T w1, T& v0, T& v1) {
@@ -1524,138 +1645,12 @@ __device__ inline void pair_solve_d(T a, T b, T d, T w0, T w1, T& v0, T& v1) {
   }
 }
 
-// Substitutions through a block's eliminated pairs, one warp per block.  The
-// work is a sequence of items: pair q (columns 2q, 2q+1 of L, stored as
-// Lc[c * lds + r]) restricted to one chunk of SUB_J * 32 of its rows below the
-// pair.  The L values of an item do not depend on the vector being solved, so
-// they are loaded SUB_D items ahead into a register ring: each warp keeps
-// several loads in flight instead of waiting a memory latency per pair.  Per
-// row, the arithmetic and its order are those of the plain column loop.
-constexpr int SUB_J = 4;   // rows per lane in one item (chunks of 128 rows)
-constexpr int SUB_D = 2;   // items loaded ahead
-
-__device__ inline int sub_chunks(int msz, int q) {
-  const int rows = msz - 2 * q - 2;
-  return rows > 0 ? (rows + 32 * SUB_J - 1) / (32 * SUB_J) : 0;
-}
-
-template <typename T>
-__device__ inline void sub_fetch(const T* __restrict__ Lc, int lds, int msz, int q, int k, bool ok,
-                                 T (&a)[SUB_J], T (&b)[SUB_J]) {
-  const int lane = threadIdx.x & 31;
-  const T* L0 = Lc + (size_t)(2 * q) * lds;
-  const T* L1 = L0 + lds;
-  const int r0 = 2 * q + 2 + 32 * SUB_J * k + lane;
-#pragma unroll
-  for (int j = 0; j < SUB_J; ++j) {
-    const int r = r0 + 32 * j;
-    const bool in = ok && r < msz;
-    a[j] = in ? L0[r] : T(0);
-    b[j] = in ? L1[r] : T(0);
-  }
-}
-
-// Forward substitution: w (length msz) in shared memory; after the call w
-// holds L^{-1} w.  Items run over pairs ascending, chunks ascending.
-template <typename T>
-__device__ void warp_forward(T* w, int msz, int npairs, const T* __restrict__ Lc, int lds) {
-  const int lane = threadIdx.x & 31;
-  // consumer and prefetch cursors (pair, chunk); a pair without rows below
-  // it ends the sequence, since every later pair has fewer rows
-  int cq = 0, ck = 0, fq = 0, fk = 0;
-  auto valid = [&](int q) { return q < npairs && sub_chunks(msz, q) > 0; };
-  auto advance = [&](int& q, int& k) {
-    if (++k >= sub_chunks(msz, q)) { ++q; k = 0; }
-  };
-  T a[SUB_D][SUB_J], b[SUB_D][SUB_J];
-#pragma unroll
-  for (int s = 0; s < SUB_D; ++s) {
-    const bool ok = valid(fq);
-    sub_fetch<T>(Lc, lds, msz, fq, fk, ok, a[s], b[s]);
-    if (ok) advance(fq, fk);
-  }
-  while (valid(cq)) {
-#pragma unroll
-    for (int s = 0; s < SUB_D; ++s) {
-      if (valid(cq)) {
-        __syncwarp();
-        const T w0 = w[2 * cq], w1 = w[2 * cq + 1];
-        const int r0 = 2 * cq + 2 + 32 * SUB_J * ck + lane;
-#pragma unroll
-        for (int j = 0; j < SUB_J; ++j) {
-          const int r = r0 + 32 * j;
-          if (r < msz) w[r] = fma(-b[s][j], w1, fma(-a[s][j], w0, w[r]));
-        }
-        const bool ok = valid(fq);
-        sub_fetch<T>(Lc, lds, msz, fq, fk, ok, a[s], b[s]);
-        if (ok) advance(fq, fk);
-        advance(cq, ck);
-      }
-    }
-  }
-  __syncwarp();
-}
-
-// Back substitution: x (length msz) holds the known tail values; pairs are
-// solved from the last to the first: x_q = v_q - sum_{r > q} L[r][q] x_r.
-// Every pair is at least one item, so that pairs without rows below them
-// are solved too.
-template <typename T>
-__device__ void warp_backward(T* x, const T* v, int msz, int npairs, const T* __restrict__ Lc,
-                              int lds) {
-  const int lane = threadIdx.x & 31;
-  auto nitems = [&](int q) { return max(1, sub_chunks(msz, q)); };
-  int cq = npairs - 1, ck = 0, fq = npairs - 1, fk = 0;
-  auto advance = [&](int& q, int& k) {
-    if (++k >= nitems(q)) { --q; k = 0; }
-  };
-  T a[SUB_D][SUB_J], b[SUB_D][SUB_J];
-#pragma unroll
-  for (int s = 0; s < SUB_D; ++s) {
-    const bool ok = fq >= 0;
-    sub_fetch<T>(Lc, lds, msz, ok ? fq : 0, fk, ok, a[s], b[s]);
-    if (ok) advance(fq, fk);
-  }
-  T s0 = T(0), s1 = T(0);
-  while (cq >= 0) {
-#pragma unroll
-    for (int s = 0; s < SUB_D; ++s) {
-      if (cq >= 0) {
-        const int r0 = 2 * cq + 2 + 32 * SUB_J * ck + lane;
-#pragma unroll
-        for (int j = 0; j < SUB_J; ++j) {
-          const int r = r0 + 32 * j;
-          if (r < msz) {
-            const T xr = x[r];
-            s0 = fma(a[s][j], xr, s0);
-            s1 = fma(b[s][j], xr, s1);
-          }
-        }
-        const bool ok = fq >= 0;
-        sub_fetch<T>(Lc, lds, msz, ok ? fq : 0, fk, ok, a[s], b[s]);
-        if (ok) advance(fq, fk);
-        if (ck + 1 >= nitems(cq)) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-          }
-          if (lane == 0) { x[2 * cq] = v[2 * cq] - s0; x[2 * cq + 1] = v[2 * cq + 1] - s1; }
-          s0 = T(0); s1 = T(0);
-          __syncwarp();
-        }
-        advance(cq, ck);
-      }
-    }
-  }
-}
-
 // local index a < m -> position in the API-layout KKT vector of element e.
 // Radau: every local row is an unknown of the element.
 __device__ inline size_t elem_global(const DevProb& P, int e, int a) {
   const int n = P.n;
   const size_t nx = (size_t)P.N * 4 * n + P.p;
-  const int pr = a >> 1, g = pr / n, s = pr - g * n;
+  const int pr = a >> 1, g = (pr >= n) + (pr >= 2 * n) + (pr >= 3 * n), s = pr - g * n;
   if (a & 1) return nx + ((size_t)e * 4 + grp_con(0, 3, g)) * n + s;
   return ((size_t)e * 4 + grp_point(0, 3, g)) * n + s;
 }
@@ -1673,19 +1668,19 @@ __device__ inline long long elem_global_gauss(const DevProb& P, int e, int a) {
   return (long long)(((size_t)e * np + (g < P.K ? g + 1 : 0)) * n + s);
 }
 // w[a] = v[global index of a] (0 where there is none) for a in [lo, hi), or
-// the reverse when store (Gauss elements, one warp; out of line).
+// the reverse when store (Gauss elements, by thread tid of nt; out of line).
 template <typename T>
 __device__ __noinline__ void gauss_elem_gather(const DevProb& P, int e, const double* v, T* w,
-                                               int lo, int hi) {
-  for (int a = lo + (threadIdx.x & 31); a < hi; a += 32) {
+                                               int lo, int hi, int tid, int nt) {
+  for (int a = lo + tid; a < hi; a += nt) {
     const long long gi = elem_global_gauss(P, e, a);
     w[a] = gi >= 0 ? (T)v[gi] : T(0);
   }
 }
 template <typename T>
 __device__ __noinline__ void gauss_elem_scatter(const DevProb& P, int e, const T* w, double* v,
-                                                int lo, int hi) {
-  for (int a = lo + (threadIdx.x & 31); a < hi; a += 32) {
+                                                int lo, int hi, int tid, int nt) {
+  for (int a = lo + tid; a < hi; a += nt) {
     const long long gi = elem_global_gauss(P, e, a);
     if (gi >= 0) v[gi] = (double)w[a];
   }
@@ -1695,221 +1690,238 @@ __device__ __noinline__ void gauss_elem_scatter(const DevProb& P, int e, const T
 // elimination (wt: the trailing rows (z_e0, c_(e+1)0) interleaved): the z part
 // of chain block e and the c part of chain block e + 1 (the rhs of c_(e+1)0
 // updated by this element's elimination); a chain's first element also sets
-// its own c part, the rhs of its initial condition.  One warp.
+// its own c part, the rhs of its initial condition.  Thread tid of nt.
 template <typename T>
 __device__ __noinline__ void gauss_chain_rhs(const DevProb& P, const DevFactor<T>& F,
-                                             const double* __restrict__ b, int e, const T* wt) {
-  const int lane = threadIdx.x & 31, n = P.n;
+                                             const double* __restrict__ b, int e, const T* wt,
+                                             int tid, int nt) {
+  const int n = P.n;
   const size_t nx = (size_t)P.N * P.np * n + P.p;
   T* Rif = F.Rif + (size_t)e * 2 * n;
   const bool start = chain_start(P, e), next = chain_next(P, e);
-  for (int s2 = lane; s2 < n; s2 += 32) {
+  for (int s2 = tid; s2 < n; s2 += nt) {
     Rif[2 * s2] = wt[2 * s2];
     if (start) Rif[2 * s2 + 1] = (T)b[nx + (size_t)e * P.np * n + s2];
     if (next) F.Rif[(size_t)(e + 1) * 2 * n + 2 * s2 + 1] = wt[2 * s2 + 1];
   }
 }
 
-template <typename T>
+// Forward substitution of element e by a group of G warps: V, the chain rows'
+// right-hand side and the parameter rows' contribution.  Here and below, the
+// block's first panels have been asked for (sub_start), and next() asks for
+// those of the group's next block once this one's substitution is done.
+template <typename T, int G, class Next>
 __device__ void elem_fwd_one(const DevProb& P, const DevFactor<T>& F, const double* __restrict__ b,
-                             int e, T* w) {
-  const int lane = threadIdx.x & 31;
-  const int n = P.n, ext = P.ext, m = P.m, p = P.p;
+                             int e, SubMem<T, G>& sm, Next next) {
+  constexpr int NT = 32 * G;
+  const int tid = group_tid<G>();
+  const int n = P.n, ext = P.ext, m = P.m, p = P.p, nint = P.K * n;
+  T* w = sm.w;
   if (!P.gauss) {
-    for (int a = lane; a < ext; a += 32) w[a] = a < m ? (T)b[elem_global(P, e, a)] : T(0);
+    for (int a = tid; a < ext; a += NT) w[a] = a < m ? (T)b[elem_global(P, e, a)] : T(0);
   } else {
-    gauss_elem_gather<T>(P, e, b, w, 0, m);
-    for (int a = m + lane; a < ext; a += 32) w[a] = T(0);
+    gauss_elem_gather<T>(P, e, b, w, 0, m, tid, NT);
+    for (int a = m + tid; a < ext; a += NT) w[a] = T(0);
   }
-  __syncwarp();
-  const int nint = P.K * n;
-  const T* Lc = F.Lel + (size_t)e * (2 * nint) * ext;
-  warp_forward<T>(w, ext, nint, Lc, ext);
-  const T* D = F.Del + (size_t)e * nint * 3;
+  group_sync<G>();
+  const T* D = F.Del + (size_t)e * nint * 3;   // asked for before the substitution
+  T d0 = T(0), d1 = T(0), d2 = T(0);
+  if (tid < nint) { d0 = D[3 * tid]; d1 = D[3 * tid + 1]; d2 = D[3 * tid + 2]; }
+  sub_set(sm.ring, group_forward<G, true>(w, sm.ring, elem_cols(P, F, e)));
+  next();
   T* V = F.Vint + (size_t)e * 2 * nint;
-  for (int q = lane; q < nint; q += 32) {
+  for (int q = tid; q < nint; q += NT) {
+    if (q >= NT) { d0 = D[3 * q]; d1 = D[3 * q + 1]; d2 = D[3 * q + 2]; }
     T v0, v1;
-    pair_solve_d<T>(D[3 * q], D[3 * q + 1], D[3 * q + 2], w[2 * q], w[2 * q + 1], v0, v1);
+    pair_solve_d<T>(d0, d1, d2, w[2 * q], w[2 * q + 1], v0, v1);
     V[2 * q] = v0; V[2 * q + 1] = v1;
   }
   T* Rif = F.Rif + (size_t)e * 2 * n;
   if (!P.gauss) {
-    for (int u = lane; u < 2 * n; u += 32) Rif[u] = w[2 * nint + u];
+    for (int u = tid; u < 2 * n; u += NT) Rif[u] = w[2 * nint + u];
   } else {
-    gauss_chain_rhs<T>(P, F, b, e, w + 2 * nint);
+    gauss_chain_rhs<T>(P, F, b, e, w + 2 * nint, tid, NT);
   }
   double* Rth = F.Rth + (size_t)e * p;
-  for (int q = lane; q < p; q += 32) Rth[q] = (double)w[m + q];
-  __syncwarp();
+  for (int q = tid; q < p; q += NT) Rth[q] = (double)w[m + q];
+  group_sync<G>();
 }
 
-template <typename T>
+template <typename T, int G, class Next>
 __device__ void bcr_fwd_one(const DevProb& P, const DevFactor<T>& F, int stride, int final_level,
-                            int bi, T* w) {
-  const int lane = threadIdx.x & 31;
+                            int bi, SubMem<T, G>& sm, Next next) {
+  constexpr int NT = 32 * G;
+  const int tid = group_tid<G>();
   const int n = P.n, p = P.p, N = P.N, bext = P.bext, n2 = 2 * n;
-  const int i = final_level ? 0 : stride * (2 * bi + 1);
+  const int i = bcr_block(stride, final_level, bi);
   const int L = final_level ? -1 : i - stride;
   const int R = (!final_level && i + stride < N) ? i + stride : -1;
   const T* Rii = F.Rif + (size_t)i * n2;
-  for (int a = lane; a < bext; a += 32) w[a] = a < n2 ? Rii[a] : T(0);
-  __syncwarp();
-  warp_forward<T>(w, bext, n, F.Lb + (size_t)i * n2 * bext, bext);
+  T* w = sm.w;
+  for (int a = tid; a < bext; a += NT) w[a] = a < n2 ? Rii[a] : T(0);
+  // what the end needs from memory, asked for before the substitution: pivots
+  // and the neighbours' right-hand sides (this block alone adds to these entries)
   const T* D = F.Db + (size_t)i * n * 3;
+  T* RL = F.Rif + (size_t)(L >= 0 ? L : 0) * n2;
+  T* RR = F.Rif + (size_t)(R >= 0 ? R : 0) * n2;
+  T d0 = T(0), d1 = T(0), d2 = T(0), rl = T(0), rr = T(0);
+  if (tid < n) {
+    d0 = D[3 * tid]; d1 = D[3 * tid + 1]; d2 = D[3 * tid + 2];
+    if (L >= 0) rl = RL[2 * tid];
+    if (R >= 0) rr = RR[2 * tid + 1];
+  }
+  group_sync<G>();
+  sub_set(sm.ring, group_forward<G, true>(w, sm.ring, bcr_cols(P, F, i)));
+  next();
   T* V = F.Vb + (size_t)i * n2;
-  for (int q = lane; q < n; q += 32) {
+  for (int q = tid; q < n; q += NT) {
+    if (q >= NT) {
+      d0 = D[3 * q]; d1 = D[3 * q + 1]; d2 = D[3 * q + 2];
+      if (L >= 0) rl = RL[2 * q];
+      if (R >= 0) rr = RR[2 * q + 1];
+    }
     T v0, v1;
-    pair_solve_d<T>(D[3 * q], D[3 * q + 1], D[3 * q + 2], w[2 * q], w[2 * q + 1], v0, v1);
+    pair_solve_d<T>(d0, d1, d2, w[2 * q], w[2 * q + 1], v0, v1);
     V[2 * q] = v0; V[2 * q + 1] = v1;
-  }
-  if (L >= 0) {
-    T* RL = F.Rif + (size_t)L * n2;
-    for (int t = lane; t < n; t += 32) RL[2 * t] += w[n2 + t];
-  }
-  if (R >= 0) {
-    T* RR = F.Rif + (size_t)R * n2;
-    for (int s = lane; s < n; s += 32) RR[2 * s + 1] += w[3 * n + s];
+    if (L >= 0) RL[2 * q] = rl + w[n2 + q];
+    if (R >= 0) RR[2 * q + 1] = rr + w[3 * n + q];
   }
   double* Rth = F.Rth + (size_t)(N + i) * p;
-  for (int q = lane; q < p; q += 32) Rth[q] = (double)w[4 * n + q];
-  __syncwarp();
+  for (int q = tid; q < p; q += NT) Rth[q] = (double)w[4 * n + q];
+  group_sync<G>();
 }
 
-// Parameter solve by one block: rhs = b_theta + chunk sums of the
-// contributions, then the FP64 LDL^T of the Schur complement (column-oriented
-// substitutions, one barrier per column).  sv: dynamic shared [p].
+// Parameter solve by one block of FBS threads: rhs = b_theta + chunk sums of the
+// contributions, then the FP64 LDL^T of the Schur complement.
 __device__ void theta_solve_block(const DevProb& P, const double* __restrict__ chunkR,
                                   const double* __restrict__ b, const DevSchur& S,
-                                  double* __restrict__ sol, double* sv) {
+                                  double* __restrict__ sol, SubMem<double, SOLVE_G>& sm) {
   const int p = P.p, N = P.N, tid = threadIdx.x;
   const size_t nz = (size_t)N * P.np * P.n;
-  for (int q = tid; q < p; q += blockDim.x) sv[q] = b[nz + q] + sum_chunks(chunkR, n_chunks(2 * N), p, q);
-  __syncthreads();
-  for (int k = 0; k < p; ++k) {
-    const double xk = sv[k];
-    for (int r = k + 1 + tid; r < p; r += blockDim.x) sv[r] -= S.S[r * p + k] * xk;
-    __syncthreads();
+  double* sv = sm.w;
+  const FactorCols<double> L{S.S, factor_ld<double>(p), p, p};
+  sub_start<SOLVE_G>(sm.ring, L, true);
+  for (int q = tid >> 2; q < p; q += FBS / 4) {
+    const double v = sum_chunks4(chunkR, n_chunks(2 * N), p, q, tid & 3);
+    if ((tid & 3) == 0) sv[q] = b[nz + q] + v;
   }
-  for (int k = tid; k < p; k += blockDim.x) {
+  __syncthreads();
+  sub_set(sm.ring, group_forward<SOLVE_G, false>(sv, sm.ring, L));
+  sub_start<SOLVE_G>(sm.ring, L, false);
+  for (int k = tid; k < p; k += FBS) {
     const double d = S.Sd[k];
     sv[k] = (d != 0.0 && isfinite(d)) ? sv[k] / d : 0.0;
   }
   __syncthreads();
-  for (int k = p - 1; k >= 0; --k) {
-    const double xk = sv[k];
-    for (int r = tid; r < k; r += blockDim.x) sv[r] -= S.S[k * p + r] * xk;
-    __syncthreads();
-  }
-  for (int q = tid; q < p; q += blockDim.x) { sol[nz + q] = sv[q]; S.xth[q] = sv[q]; }
+  sub_set(sm.ring, group_backward<SOLVE_G, false>(sv, sm.sums, sm.ring, L));
+  for (int q = tid; q < p; q += FBS) { sol[nz + q] = sv[q]; S.xth[q] = sv[q]; }
+  sub_release();
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(SBS)
+__global__ void __launch_bounds__(FBS)
 k_theta_solve(DevProb P, const double* __restrict__ chunkR, const double* __restrict__ b,
-              DevSchur S, double* __restrict__ sol) {
-  extern __shared__ double sv[];
-  theta_solve_block(P, chunkR, b, S, sol, sv);
+              DevSchur S, double* __restrict__ sol, int* err, size_t smem) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ unsigned long long bars[SUB_STAGES];
+  sub_init(bars, SUB_STAGES);
+  SubMem<double, SOLVE_G> sm = sub_mem<double, SOLVE_G>(smraw, smem, P.p, bars, err);
+  theta_solve_block(P, chunkR, b, S, sol, sm);
 }
 
-template <typename T>
+template <typename T, int G, class Next>
 __device__ void bcr_bwd_one(const DevProb& P, const DevFactor<T>& F, const DevSchur& S,
-                            double* __restrict__ sol, int stride, int final_level, int bi, T* x) {
-  const int lane = threadIdx.x & 31;
+                            double* __restrict__ sol, int stride, int final_level, int bi,
+                            SubMem<T, G>& sm, Next next) {
+  constexpr int NT = 32 * G;
+  const int tid = group_tid<G>();
   const int n = P.n, p = P.p, N = P.N, bext = P.bext, n2 = 2 * n, np = P.np, cpt = P.cpt;
-  const int i = final_level ? 0 : stride * (2 * bi + 1);
+  const int i = bcr_block(stride, final_level, bi);
   const int L = final_level ? -1 : i - stride;
   const int R = (!final_level && i + stride < N) ? i + stride : -1;
   const size_t nx = (size_t)N * np * n + p;
-  for (int a = lane; a < bext; a += 32) {
+  const T* V = F.Vb + (size_t)i * n2;
+  T* x = sm.w;
+  for (int a = tid; a < bext; a += NT) {
     T v = T(0);
-    if (a >= n2 && a < 3 * n) {
+    if (a < n2) {
+      v = V[a];
+    } else if (a < 3 * n) {
       if (L >= 0) v = (T)sol[((size_t)L * np + cpt) * n + (a - n2)];
-    } else if (a >= 3 * n && a < 4 * n) {
+    } else if (a < 4 * n) {
       if (R >= 0) v = (T)sol[nx + (size_t)R * np * n + (a - 3 * n)];
-    } else if (a >= 4 * n) {
+    } else {
       v = (T)S.xth[a - 4 * n];
     }
     x[a] = v;
   }
-  __syncwarp();
-  warp_backward<T>(x, F.Vb + (size_t)i * n2, bext, n, F.Lb + (size_t)i * n2 * bext, bext);
-  for (int s = lane; s < n; s += 32) {
+  group_sync<G>();
+  sub_set(sm.ring, group_backward<G, true>(x, sm.sums, sm.ring, bcr_cols(P, F, i)));
+  next();
+  for (int s = tid; s < n; s += NT) {
     sol[((size_t)i * np + cpt) * n + s] = (double)x[2 * s];
     sol[nx + (size_t)i * np * n + s] = (double)x[2 * s + 1];
   }
-  __syncwarp();
+  group_sync<G>();
 }
 
-template <typename T>
+template <typename T, int G, class Next>
 __device__ void elem_bwd_one(const DevProb& P, const DevFactor<T>& F, const DevSchur& S,
-                             double* __restrict__ sol, int e, T* x) {
-  const int lane = threadIdx.x & 31;
+                             double* __restrict__ sol, int e, SubMem<T, G>& sm, Next next) {
+  constexpr int NT = 32 * G;
+  const int tid = group_tid<G>();
   const int n = P.n, ext = P.ext, m = P.m;
   const int nint = P.K * n;
+  const T* V = F.Vint + (size_t)e * 2 * nint;
+  T* x = sm.w;
+  for (int a = tid; a < 2 * nint; a += NT) x[a] = V[a];
   if (!P.gauss) {
-    for (int a = lane; a < ext; a += 32) {
-      T v = T(0);
-      if (a >= 2 * nint && a < m) v = (T)sol[elem_global(P, e, a)];
-      else if (a >= m) v = (T)S.xth[a - m];
-      x[a] = v;
-    }
+    for (int a = 2 * nint + tid; a < m; a += NT) x[a] = (T)sol[elem_global(P, e, a)];
   } else {
-    for (int a = lane; a < 2 * nint; a += 32) x[a] = T(0);
-    gauss_elem_gather<T>(P, e, sol, x, 2 * nint, m);
-    for (int a = m + lane; a < ext; a += 32) x[a] = (T)S.xth[a - m];
+    gauss_elem_gather<T>(P, e, sol, x, 2 * nint, m, tid, NT);
   }
-  __syncwarp();
-  warp_backward<T>(x, F.Vint + (size_t)e * 2 * nint, ext, nint,
-                   F.Lel + (size_t)e * (2 * nint) * ext, ext);
+  for (int a = m + tid; a < ext; a += NT) x[a] = (T)S.xth[a - m];
+  group_sync<G>();
+  sub_set(sm.ring, group_backward<G, true>(x, sm.sums, sm.ring, elem_cols(P, F, e)));
+  next();
   if (!P.gauss)
-    for (int a = lane; a < 2 * nint; a += 32) sol[elem_global(P, e, a)] = (double)x[a];
+    for (int a = tid; a < 2 * nint; a += NT) sol[elem_global(P, e, a)] = (double)x[a];
   else
-    gauss_elem_scatter<T>(P, e, x, sol, 0, 2 * nint);
-  __syncwarp();
+    gauss_elem_scatter<T>(P, e, x, sol, 0, 2 * nint, tid, NT);
+  group_sync<G>();
 }
 
-template <typename T>
-__global__ void __launch_bounds__(32 * SOLVE_WARPS)
-k_elem_fwd(DevProb P, DevFactor<T> F, const double* __restrict__ b) {
+// One launch per phase: a narrow block per warp or a wide one per CUDA block
+// (G = SOLVE_G).
+template <typename T, int G>
+__global__ void __launch_bounds__(FBS)
+k_elem_solve(DevProb P, DevFactor<T> F, DevSchur S, const double* __restrict__ b,
+             double* __restrict__ sol, int fwd, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int warp = threadIdx.x >> 5;
-  const int e = blockIdx.x * SOLVE_WARPS + warp;
+  __shared__ unsigned long long bars[SOLVE_BARS];
+  sub_init(bars, SOLVE_BARS);
+  SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.ext, bars, &F.gbar->err);
+  const int e = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
   if (e >= P.N) return;
-  elem_fwd_one<T>(P, F, b, e, reinterpret_cast<T*>(smraw) + (size_t)warp * P.ext);
+  sub_start<G>(sm.ring, elem_cols(P, F, e), fwd != 0);
+  if (fwd) elem_fwd_one<T, G>(P, F, b, e, sm, [] {});
+  else elem_bwd_one<T, G>(P, F, S, sol, e, sm, [] {});
 }
 
-template <typename T>
-__global__ void __launch_bounds__(32 * SOLVE_WARPS)
-k_bcr_fwd(DevProb P, DevFactor<T> F, int stride, int final_level) {
+template <typename T, int G>
+__global__ void __launch_bounds__(FBS)
+k_bcr_solve(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int fwd, int stride,
+            int final_level, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int warp = threadIdx.x >> 5;
+  __shared__ unsigned long long bars[SOLVE_BARS];
+  sub_init(bars, SOLVE_BARS);
+  SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.bext, bars, &F.gbar->err);
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
-  const int bi = blockIdx.x * SOLVE_WARPS + warp;
+  const int bi = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
   if (bi >= nblk) return;
-  bcr_fwd_one<T>(P, F, stride, final_level, bi, reinterpret_cast<T*>(smraw) + (size_t)warp * P.bext);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(32 * SOLVE_WARPS)
-k_bcr_bwd(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int stride,
-          int final_level) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int warp = threadIdx.x >> 5;
-  const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
-  const int bi = blockIdx.x * SOLVE_WARPS + warp;
-  if (bi >= nblk) return;
-  bcr_bwd_one<T>(P, F, S, sol, stride, final_level, bi,
-                 reinterpret_cast<T*>(smraw) + (size_t)warp * P.bext);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(32 * SOLVE_WARPS)
-k_elem_bwd(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int warp = threadIdx.x >> 5;
-  const int e = blockIdx.x * SOLVE_WARPS + warp;
-  if (e >= P.N) return;
-  elem_bwd_one<T>(P, F, S, sol, e, reinterpret_cast<T*>(smraw) + (size_t)warp * P.ext);
+  sub_start<G>(sm.ring, bcr_cols(P, F, bcr_block(stride, final_level, bi)), fwd != 0);
+  if (fwd) bcr_fwd_one<T, G>(P, F, stride, final_level, bi, sm, [] {});
+  else bcr_bwd_one<T, G>(P, F, S, sol, stride, final_level, bi, sm, [] {});
 }
 
 // ---- persistent cooperative kernels ------------------------------------------------
@@ -1962,6 +1974,22 @@ __device__ void grid_exit(GridBar* gb) {
       atomicExch(&gb->exits, 0u);
     }
   }
+}
+
+// Descriptor of a lone instance in shared memory.  The acquire of a grid barrier
+// empties the L1 cache, after which every read through the descriptor in global
+// memory waits for the L2 again; with one instance its copy here is used instead.
+struct LoneInst {
+  alignas(16) unsigned char b[sizeof(DevInst)];
+};
+__device__ inline void lone_load(LoneInst& s, const DevInst* insts, const int* act, int A) {
+  static_assert(sizeof(DevInst) % 8 == 0, "copied by 8-byte words");
+  if (A == 1) {
+    const double* src = reinterpret_cast<const double*>(insts + act[0]);
+    double* dst = reinterpret_cast<double*>(s.b);
+    for (int i = threadIdx.x; i < (int)(sizeof(DevInst) / 8); i += blockDim.x) dst[i] = src[i];
+  }
+  __syncthreads();
 }
 
 // ---- batched persistent kernels -------------------------------------------------------
@@ -2116,11 +2144,19 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
     F.chunkS[it] = chunk_sum_item(F.Scon, 2 * I.P.N, L, G, it / L, it % L);
   }
   grid_barrier(gb, ep);
+  // ... their totals
+  for (int t = blockIdx.x * FBS + threadIdx.x; t < pre_cs[A]; t += gridDim.x * FBS) {
+    const int k = find_item(pre_cs, A, t);
+    const DevInst& I = insts[act[k]];
+    if (t - pre_cs[k] < I.P.p * I.P.p)
+      schur_total(inst_factor<T>(I).chunkS, I.P.N, I.P.p, t - pre_cs[k]);
+  }
+  grid_barrier(gb, ep);
   // 4. parameter Schur complement, one block per instance
   for (int k = blockIdx.x; k < A; k += gridDim.x) {
     const DevInst& I = insts[act[k]];
     const DevFactor<T>& F = inst_factor<T>(I);
-    const size_t need = sizeof(double) * ((size_t)I.P.p * I.P.p + I.P.p);
+    const size_t need = sizeof(double) * schur_doubles(I.P.p);
     double* sS = need <= smem_bytes ? reinterpret_cast<double*>(smraw) : I.S.S;
     schur_block(I.P, F.inert, F.chunkS, I.E.wtt, I.sigma, prm[k].dw, I.S, sS);
     if (threadIdx.x == 0) {
@@ -2131,91 +2167,136 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
   grid_exit(gb);
 }
 
+// Work lists of the batched solve: prefix arrays over the active instances of
+// the elements and of the reduction blocks of each level, separately for the
+// instances whose blocks are narrow (one warp each) and wide (one CUDA block).
+struct SolvePlan {
+  const int* elem[2];   // [wide][A + 1]
+  const int* lv[2];     // [wide][level][A + 1]
+};
+
 // Batched solve.  Levels below `lsplit` run over the whole grid, a grid
 // barrier after each; from level `lsplit` up (few blocks per instance) one
 // block owns an instance and separates its levels by block barriers, and the
 // same block then solves the parameter system and substitutes back down to
-// level `lsplit`.  Every block solve is the same per-warp code as in the
+// level `lsplit`.  Every block solve is the same code as in the
 // single-instance launches, so the result does not depend on the split.
 template <typename T>
-__global__ void __launch_bounds__(FBS)
-k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
-          const int* __restrict__ pre_elem, const int* __restrict__ pre_lv, int maxL, int lsplit,
-          const int* __restrict__ pre_cs, int ir, int per_warp, GridBar* gb) {
+__global__ void __launch_bounds__(FBS, sizeof(T) == 4 ? 2 : 1)
+k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A, SolvePlan sp,
+          const int* __restrict__ pre_lv, int maxL, int lsplit,
+          const int* __restrict__ pre_cs, int ir, int pn, int pw, int max_p, size_t smem,
+          GridBar* gb) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ unsigned long long bars[SOLVE_BARS + 2 * SUB_STAGES];
+  __shared__ LoneInst lone;
+  lone_load(lone, insts, act, A);
+  sub_init(bars, SOLVE_BARS + 2 * SUB_STAGES);
+  auto inst = [&](int k) -> const DevInst& {
+    return A == 1 ? *reinterpret_cast<const DevInst*>(lone.b) : insts[act[k]];
+  };
   unsigned int ep = 0;
   const int warp = threadIdx.x >> 5, wpb = FBS / 32;
   const int gw = blockIdx.x * wpb + warp, nw = gridDim.x * wpb;
-  T* wv = reinterpret_cast<T*>(smraw) + (size_t)warp * per_warp;
-  auto level_blocks = [&](int lv, int k) {
-    const int* pre = pre_lv + (size_t)lv * (A + 1);
-    return lv == maxL ? 1 : pre[k + 1] - pre[k];
+  // the three groups use the same shared memory, one at a time
+  SubMem<T, 1> narrow = sub_mem<T, 1>(smraw, smem, max(pn, 1), bars, &gb->err);
+  SubMem<T, SOLVE_G> wide =
+      sub_mem<T, SOLVE_G>(smraw, smem, max(pw, 1), bars + SOLVE_BARS, &gb->err);
+  SubMem<double, SOLVE_G> theta =
+      sub_mem<double, SOLVE_G>(smraw, smem, max(max_p, 1), bars + SOLVE_BARS + SUB_STAGES, &gb->err);
+  auto phase_end = [&]() { sub_release(); grid_barrier(gb, ep); };
+  // Items t0, t0 + step, ... of a list for one group: cols(I, i) are an item's L
+  // columns, run(I, i, next) its substitution.
+  auto list = [&](const int* pre, int t0, int step, auto& sm, bool fwd, auto&& cols, auto&& run) {
+    constexpr int G = std::is_same_v<std::decay_t<decltype(sm)>, SubMem<T, 1>> ? 1 : SOLVE_G;
+    const int tot = pre[A];
+    auto find = [&](int t) { return A == 1 ? 0 : find_item(pre, A, t); };
+    int k = t0 < tot ? find(t0) : 0;
+    if (t0 < tot) sub_start<G>(sm.ring, cols(inst(k), t0 - pre[k]), fwd);
+    for (int t = t0; t < tot; t += step) {
+      const int tn = t + step, kn = tn < tot ? find(tn) : 0;
+      run(inst(k), t - pre[k],
+          [&] { if (tn < tot) sub_start<G>(sm.ring, cols(inst(kn), tn - pre[kn]), fwd); });
+      k = kn;
+    }
   };
-  for (int t = gw; t < pre_elem[A]; t += nw) {
-    const int k = find_item(pre_elem, A, t);
-    const DevInst& I = insts[act[k]];
-    elem_fwd_one<T>(I.P, inst_factor<T>(I), ir ? I.kr : I.ka, t - pre_elem[k], wv);
-  }
-  grid_barrier(gb, ep);
-  for (int lv = 0; lv < lsplit; ++lv) {
+  auto elems = [&](bool fwd) {
+    auto cols = [&](const DevInst& I, int e) { return elem_cols(I.P, inst_factor<T>(I), e); };
+    auto one = [&](auto& sm) {
+      return [&, fwd](const DevInst& I, int e, auto next) {
+        if (fwd) elem_fwd_one(I.P, inst_factor<T>(I), ir ? I.kr : I.ka, e, sm, next);
+        else elem_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, e, sm, next);
+      };
+    };
+    list(sp.elem[1], blockIdx.x, gridDim.x, wide, fwd, cols, one(wide));
+    sub_release();
+    __syncthreads();
+    list(sp.elem[0], gw, nw, narrow, fwd, cols, one(narrow));
+  };
+  auto level = [&](int lv, bool fwd) {
+    const size_t o = (size_t)lv * (A + 1);
+    auto cols = [&](const DevInst& I, int bi) {
+      return bcr_cols(I.P, inst_factor<T>(I), bcr_block(1 << lv, 0, bi));
+    };
+    auto one = [&](auto& sm) {
+      return [&, fwd](const DevInst& I, int bi, auto next) {
+        if (fwd) bcr_fwd_one(I.P, inst_factor<T>(I), 1 << lv, 0, bi, sm, next);
+        else bcr_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, 1 << lv, 0, bi, sm, next);
+      };
+    };
+    list(sp.lv[1] + o, blockIdx.x, gridDim.x, wide, fwd, cols, one(wide));
+    sub_release();
+    __syncthreads();
+    list(sp.lv[0] + o, gw, nw, narrow, fwd, cols, one(narrow));
+  };
+  // the levels from lsplit up of instance k, by this block
+  auto top = [&](const DevInst& I, int k, int lv, bool fwd) {
+    const int fin = lv == maxL, stride = fin ? 1 : 1 << lv;
     const int* pre = pre_lv + (size_t)lv * (A + 1);
-    for (int t = gw; t < pre[A]; t += nw) {
-      const int k = find_item(pre, A, t);
-      const DevInst& I = insts[act[k]];
-      bcr_fwd_one<T>(I.P, inst_factor<T>(I), 1 << lv, 0, t - pre[k], wv);
-    }
-    grid_barrier(gb, ep);
+    const int nb = fin ? 1 : pre[k + 1] - pre[k];
+    auto run = [&](int bi, auto& sm, auto g) {
+      constexpr int G = decltype(g)::value;
+      sub_start<G>(sm.ring, bcr_cols(I.P, inst_factor<T>(I), bcr_block(stride, fin, bi)), fwd);
+      if (fwd) bcr_fwd_one(I.P, inst_factor<T>(I), stride, fin, bi, sm, [] {});
+      else bcr_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, stride, fin, bi, sm, [] {});
+    };
+    if (bcr_solve_wide(I.P))
+      for (int bi = 0; bi < nb; ++bi) run(bi, wide, std::integral_constant<int, SOLVE_G>{});
+    else
+      for (int bi = warp; bi < nb; bi += wpb) run(bi, narrow, std::integral_constant<int, 1>{});
+    sub_release();
+    __syncthreads();
+  };
+  elems(true);
+  phase_end();
+  for (int lv = 0; lv < lsplit; ++lv) {
+    level(lv, true);
+    phase_end();
   }
-  for (int k = blockIdx.x; k < A; k += gridDim.x) {
-    const DevInst& I = insts[act[k]];
-    for (int lv = lsplit; lv <= maxL; ++lv) {
-      const bool fin = lv == maxL;
-      const int nb = level_blocks(lv, k);
-      for (int bi = warp; bi < nb; bi += wpb)
-        bcr_fwd_one<T>(I.P, inst_factor<T>(I), fin ? 1 : 1 << lv, fin ? 1 : 0, bi, wv);
-      __syncthreads();
-    }
-  }
-  grid_barrier(gb, ep);
+  for (int k = blockIdx.x; k < A; k += gridDim.x)
+    for (int lv = lsplit; lv <= maxL; ++lv) top(inst(k), k, lv, true);
+  phase_end();
   for (int t = blockIdx.x * FBS + threadIdx.x; t < pre_cs[A]; t += gridDim.x * FBS) {
     const int k = find_item(pre_cs, A, t);
-    const DevInst& I = insts[act[k]];
+    const DevInst& I = inst(k);
     const DevFactor<T>& F = inst_factor<T>(I);
     const int L = I.P.p, G = n_chunks(2 * I.P.N);
     const int it = t - pre_cs[k];
     F.chunkR[it] = chunk_sum_item(F.Rth, 2 * I.P.N, L, G, it / L, it % L);
   }
-  grid_barrier(gb, ep);
+  phase_end();
   for (int k = blockIdx.x; k < A; k += gridDim.x) {
-    const DevInst& I = insts[act[k]];
-    double* sol = ir ? I.kc : I.kb;
-    // theta_solve_block ends with a block barrier: its shared vector and the
-    // per-warp vectors below may overlap
-    theta_solve_block(I.P, inst_factor<T>(I).chunkR, ir ? I.kr : I.ka, I.S, sol,
-                      reinterpret_cast<double*>(smraw));
-    for (int lv = maxL; lv >= lsplit; --lv) {
-      const bool fin = lv == maxL;
-      const int nb = level_blocks(lv, k);
-      for (int bi = warp; bi < nb; bi += wpb)
-        bcr_bwd_one<T>(I.P, inst_factor<T>(I), I.S, sol, fin ? 1 : 1 << lv, fin ? 1 : 0, bi, wv);
-      __syncthreads();
-    }
+    const DevInst& I = inst(k);
+    theta_solve_block(I.P, inst_factor<T>(I).chunkR, ir ? I.kr : I.ka, I.S, ir ? I.kc : I.kb,
+                      theta);
+    for (int lv = maxL; lv >= lsplit; --lv) top(I, k, lv, false);
   }
-  grid_barrier(gb, ep);
+  phase_end();
   for (int lv = lsplit - 1; lv >= 0; --lv) {
-    const int* pre = pre_lv + (size_t)lv * (A + 1);
-    for (int t = gw; t < pre[A]; t += nw) {
-      const int k = find_item(pre, A, t);
-      const DevInst& I = insts[act[k]];
-      bcr_bwd_one<T>(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, 1 << lv, 0, t - pre[k], wv);
-    }
-    grid_barrier(gb, ep);
+    level(lv, false);
+    phase_end();
   }
-  for (int t = gw; t < pre_elem[A]; t += nw) {
-    const int k = find_item(pre_elem, A, t);
-    const DevInst& I = insts[act[k]];
-    elem_bwd_one<T>(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, t - pre_elem[k], wv);
-  }
+  elems(false);
   grid_exit(gb);
 }
 
@@ -2350,7 +2431,7 @@ cudaError_t launch_factor(const DevProb& P, const DevEval& E, const double* sigm
                           double dc, const DevFactor<T>& F, const DevSchur& S, cudaStream_t st) {
   const bool es = elem_uses_smem<T>(P), bs = bcr_uses_smem<T>(P);
   const size_t sme = elem_factor_smem<T>(P, es), smb = bcr_factor_smem<T>(P, bs);
-  const size_t sms = sizeof(double) * ((size_t)P.p * P.p + P.p);
+  const size_t sms = sizeof(double) * schur_doubles(P.p);
   cudaError_t e;
   if ((e = launch_elem_factor<T>(P, E, sigma, dw, dc, F, st)) != cudaSuccess) return e;
   const int bt = bcr_rt_tiles(P.bext);
@@ -2376,11 +2457,16 @@ cudaError_t launch_factor(const DevProb& P, const DevEval& E, const double* sigm
     if ((e = bcr_level(s, 0)) != cudaSuccess) return e;
   if ((e = bcr_level(1, 1)) != cudaSuccess) return e;
   // the Schur block works in shared memory up to the factorization limit,
-  // otherwise in S.S (p p + p doubles) itself
+  // otherwise in S.S itself
   const bool sg = sms > SMEM_LIMIT;
   if (!sg && sms > SMEM_OPTIN_ABOVE)
     cudaFuncSetAttribute(k_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms);
   if ((e = launch_chunk_sums(F.Scon, 2 * P.N, P.p * P.p, F.chunkS, st)) != cudaSuccess) return e;
+  if (P.p > 0) {
+    count_launch();
+    k_schur_total<<<ceil_div((long long)P.p * P.p, CS_BS), CS_BS, 0, st>>>(F.chunkS, P.N, P.p);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   count_launch();
   k_schur<<<1, SBS, sg ? 0 : sms, st>>>(P, F.inert, F.chunkS, E.wtt, sigma, dw, S, sg ? 1 : 0);
   return cudaGetLastError();
@@ -2389,50 +2475,40 @@ cudaError_t launch_factor(const DevProb& P, const DevEval& E, const double* sigm
 template <typename T>
 cudaError_t launch_solve(const DevProb& P, const DevFactor<T>& F, const DevSchur& S,
                          const double* b, double* sol, cudaStream_t st) {
-  const int tpb = 32 * SOLVE_WARPS;
+  const bool ew = elem_solve_wide(P), bw = bcr_solve_wide(P);
+  const size_t sme = solve_smem<T>(ew ? 0 : P.ext, false, ew ? P.ext : 0, 0);
+  const size_t smb = solve_smem<T>(bw ? 0 : P.bext, false, bw ? P.bext : 0, 0);
+  const size_t smt = solve_smem<T>(0, false, 0, std::max(P.p, 1));
   cudaError_t e;
-  size_t sme = sizeof(T) * (size_t)P.ext * SOLVE_WARPS;
-  size_t smb = sizeof(T) * (size_t)P.bext * SOLVE_WARPS;
-  if (sme > SMEM_OPTIN_ABOVE) {
-    cudaFuncSetAttribute(k_elem_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sme);
-    cudaFuncSetAttribute(k_elem_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sme);
-  }
-  if (smb > SMEM_OPTIN_ABOVE) {
-    cudaFuncSetAttribute(k_bcr_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    cudaFuncSetAttribute(k_bcr_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-  }
-  count_launch();
-  k_elem_fwd<T><<<ceil_div(P.N, SOLVE_WARPS), tpb, sme, st>>>(P, F, b);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  auto grid = [](bool wide, int items) { return wide ? items : ceil_div(items, SOLVE_G); };
+  auto run = [&](auto kern, int g, size_t sm, auto... args) -> cudaError_t {
+    opt_in_smem(kern, sm);
+    count_launch();
+    kern<<<g, FBS, sm, st>>>(args..., sm);
+    return cudaGetLastError();
+  };
+  auto elems = [&](int fwd) {
+    return run(ew ? k_elem_solve<T, SOLVE_G> : k_elem_solve<T, 1>, grid(ew, P.N), sme, P, F, S, b,
+               sol, fwd);
+  };
+  auto level = [&](int fwd, int s, int fin) {
+    const int g = grid(bw, fin ? 1 : bcr_level_blocks(P.N, s));
+    return run(bw ? k_bcr_solve<T, SOLVE_G> : k_bcr_solve<T, 1>, g, smb, P, F, S, sol, fwd, s, fin);
+  };
+  if ((e = elems(1)) != cudaSuccess) return e;
   std::vector<int> strides;
   for (int s = 1; s < P.N; s *= 2) strides.push_back(s);
-  for (int s : strides) {
-    int nblk = bcr_level_blocks(P.N, s);
-    count_launch();
-    k_bcr_fwd<T><<<ceil_div(nblk, SOLVE_WARPS), tpb, smb, st>>>(P, F, s, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  count_launch();
-  k_bcr_fwd<T><<<1, tpb, smb, st>>>(P, F, 1, 1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  size_t smt = sizeof(double) * (size_t)(P.p > 0 ? P.p : 1);
+  for (int s : strides)
+    if ((e = level(1, s, 0)) != cudaSuccess) return e;
+  if ((e = level(1, 1, 1)) != cudaSuccess) return e;
   if ((e = launch_chunk_sums(F.Rth, 2 * P.N, P.p, F.chunkR, st)) != cudaSuccess) return e;
-  count_launch();
-  k_theta_solve<<<1, SBS, smt, st>>>(P, F.chunkR, b, S, sol);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  count_launch();
-  k_bcr_bwd<T><<<1, tpb, smb, st>>>(P, F, S, sol, 1, 1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  for (int k = (int)strides.size() - 1; k >= 0; --k) {
-    int s = strides[k];
-    int nblk = bcr_level_blocks(P.N, s);
-    count_launch();
-    k_bcr_bwd<T><<<ceil_div(nblk, SOLVE_WARPS), tpb, smb, st>>>(P, F, S, sol, s, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  count_launch();
-  k_elem_bwd<T><<<ceil_div(P.N, SOLVE_WARPS), tpb, sme, st>>>(P, F, S, sol);
-  return cudaGetLastError();
+  if ((e = run(k_theta_solve, 1, smt, P, (const double*)F.chunkR, b, S, sol, &F.gbar->err)) !=
+      cudaSuccess)
+    return e;
+  if ((e = level(0, 1, 1)) != cudaSuccess) return e;
+  for (int k = (int)strides.size() - 1; k >= 0; --k)
+    if ((e = level(0, strides[k], 0)) != cudaSuccess) return e;
+  return elems(0);
 }
 
 // Batched launchers.  `grid_cap` limits the grid when some instance uses its
@@ -2493,18 +2569,19 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
 }
 
 template <typename T>
-cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
-                           const int* pre_lv, int maxL, int lsplit, const int* pre_cs, int ir,
-                           int per_warp,
-                           GridBar* gb, int max_p, int grid_want, cudaStream_t st, int reserve) {
+cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
+                           const int* const elem[2], const int* const lv[2], const int* pre_lv,
+                           int maxL, int lsplit, const int* pre_cs, int ir, int pn, bool many,
+                           int pw, GridBar* gb, int max_p, int grid_want, cudaStream_t st,
+                           int reserve) {
   if (A == 0) return cudaSuccess;
-  size_t smem = std::max(sizeof(T) * (size_t)per_warp * (FBS / 32),
-                         sizeof(double) * (size_t)std::max(max_p, 1));
+  size_t smem = solve_smem<T>(pn, many, pw, std::max(max_p, 1));
   opt_in_smem(k_solve_b<T>, smem);
   int grid = coop_grid(k_solve_b<T>, FBS, smem, grid_want, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
-  void* args[] = {(void*)&insts, (void*)&act, &A, (void*)&pre_elem, (void*)&pre_lv, &maxL,
-                  &lsplit, (void*)&pre_cs, &ir, &per_warp, &gb};
+  SolvePlan sp{{elem[0], elem[1]}, {lv[0], lv[1]}};
+  void* args[] = {(void*)&insts, (void*)&act, &A, &sp, (void*)&pre_lv, &maxL,
+                  &lsplit, (void*)&pre_cs, &ir, &pn, &pw, &max_p, &smem, &gb};
   count_launch();
   return cudaLaunchCooperativeKernel((void*)k_solve_b<T>, dim3(grid), dim3(FBS), args, smem, st);
 }
@@ -2528,12 +2605,13 @@ size_t bcr_rt_stage_bytes(const DevProb& P, bool f32) {
 int elem_rt_threads(const DevProb& P, bool f32) {
   return f32 ? rt_block_threads<float>(P.ext) : rt_block_threads<double>(P.ext);
 }
-template cudaError_t launch_solve_b<float>(const DevInst*, const int*, int, const int*, const int*,
-                                           int, int, const int*, int, int, GridBar*, int, int,
-                                           cudaStream_t, int);
-template cudaError_t launch_solve_b<double>(const DevInst*, const int*, int, const int*,
-                                            const int*, int, int, const int*, int, int, GridBar*,
-                                            int, int, cudaStream_t, int);
+bool solve_wide(const DevProb& P, bool elem) { return elem ? elem_solve_wide(P) : bcr_solve_wide(P); }
+template cudaError_t launch_solve_b<float>(const DevInst*, const int*, int, const int* const[2],
+                                           const int* const[2], const int*, int, int, const int*,
+                                           int, int, bool, int, GridBar*, int, int, cudaStream_t, int);
+template cudaError_t launch_solve_b<double>(const DevInst*, const int*, int, const int* const[2],
+                                            const int* const[2], const int*, int, int, const int*,
+                                            int, int, bool, int, GridBar*, int, int, cudaStream_t, int);
 template size_t elem_factor_smem<float>(const DevProb&, bool);
 template size_t elem_factor_smem<double>(const DevProb&, bool);
 template size_t bcr_factor_smem<float>(const DevProb&, bool);

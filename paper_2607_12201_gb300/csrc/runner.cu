@@ -44,11 +44,14 @@ struct Plan {
   cudaEvent_t ev_int = nullptr, ev_prm = nullptr;
   bool int_pending = false, prm_pending = false;
   size_t off_act = 0, off_elem = 0, off_lv = 0, off_cs_s = 0, off_cs_r = 0, off_f32 = 0,
-         off_f64 = 0;
+         off_f64 = 0, off_se[2] = {0, 0}, off_sl[2] = {0, 0};
   int sweep_threads = 0;
   size_t smem_eval = 0, smem_f[2] = {0, 0}, smem_sweep = 0;
   int cap_f[2] = {1 << 30, 1 << 30};
-  int per_warp[2] = {0, 0};
+  int solve_pw = 0;             // rows of the largest block a CUDA block solves
+  int solve_pn = 0;             // ... that one warp solves
+  bool solve_many = false;      // several of those for every warp the device holds
+  int solve_want = 0;           // CUDA blocks that hold every element at once
   int rt_threads[2] = {0, 0};   // block size of the register-tiled element kernel
   size_t rt_smem[2] = {0, 0};   // its dynamic shared memory
   int big_grid[2] = {0, 0};     // grid of the large-element kernel (0: no such element)
@@ -59,6 +62,8 @@ struct Plan {
   const int* act() const { return d_int + off_act; }
   const int* pre_elem() const { return d_int + off_elem; }
   const int* pre_lv() const { return d_int + off_lv; }
+  const int* solve_elem(int wide) const { return d_int + off_se[wide]; }
+  const int* solve_lv(int wide) const { return d_int + off_sl[wide]; }
   const int* pre_cs_s() const { return d_int + off_cs_s; }
   const int* pre_cs_r() const { return d_int + off_cs_r; }
   const int* flags(int prec) const { return d_int + (prec ? off_f32 : off_f64); }
@@ -210,7 +215,7 @@ struct Runner {
     pl.max_p = maxp;
     pl.max_n = 0;
     for (int s : slots) pl.max_n = std::max(pl.max_n, P(s).np * P(s).n);
-    const size_t n_int = (size_t)A + (A + 1) * (size_t)(4 + maxL + 1) + 2 * (size_t)A;
+    const size_t n_int = (size_t)A + (A + 1) * (size_t)(4 + maxL + 1 + 2 * (maxL + 2)) + 2 * (size_t)A;
     cudaError_t e = grow(&pl.d_int, &pl.h_int, &pl.cap_int, n_int);
     if (e == cudaSuccess) e = grow(&pl.d_ll, &pl.h_ll, &pl.cap_ll, (size_t)A + 1);
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return COLLO_ERR_OOM; }
@@ -225,8 +230,11 @@ struct Runner {
     for (int lv = maxL; lv >= 0; --lv) {
       int most = 0;
       for (int k = 0; k < A; ++k) {
+        // blocks a CUDA block would solve one after another, in rounds of as
+        // many as it solves at once
         const int N = P(slots[k]).N, st = 1 << lv;
-        most = std::max(most, (lv < maxL && N > st) ? (N - st + 2 * st - 1) / (2 * st) : 0);
+        const int nb = (lv < maxL && N > st) ? (N - st + 2 * st - 1) / (2 * st) : 0;
+        most = std::max(most, solve_wide(P(slots[k]), false) ? 8 * nb : nb);
       }
       if (most > schedule().solve_top) break;
       pl.lsplit = lv;
@@ -240,6 +248,36 @@ struct Runner {
       }
       o += A + 1;
     }
+    // the solve's lists: the same prefixes over the narrow / wide instances
+    pl.solve_pw = 0;
+    pl.solve_pn = 0;
+    pl.solve_want = A;
+    for (int k = 0; k < A; ++k) {
+      const DevProb& Q = P(slots[k]);
+      for (int elem = 0; elem < 2; ++elem)
+        (solve_wide(Q, elem != 0) ? pl.solve_pw : pl.solve_pn) =
+            std::max(solve_wide(Q, elem != 0) ? pl.solve_pw : pl.solve_pn, elem ? Q.ext : Q.bext);
+    }
+    int items[2] = {0, 0};
+    for (int wide = 0; wide < 2; ++wide) {
+      pl.off_se[wide] = o; h[o] = 0;
+      for (int k = 0; k < A; ++k)
+        h[o + k + 1] = h[o + k] + (solve_wide(P(slots[k]), true) == (wide != 0) ? P(slots[k]).N : 0);
+      items[wide] = h[o + A];
+      o += A + 1;
+      pl.off_sl[wide] = o;
+      for (int lv = 0; lv <= maxL; ++lv) {
+        const int* all = h + pl.off_lv + (size_t)lv * (A + 1);
+        h[o] = 0;
+        for (int k = 0; k < A; ++k)
+          h[o + k + 1] = h[o + k] + (solve_wide(P(slots[k]), false) == (wide != 0)
+                                         ? all[k + 1] - all[k] : 0);
+        o += A + 1;
+      }
+    }
+    const int per = std::max(1, schedule().solve_elems);
+    pl.solve_want = std::max(A, items[1] + (items[0] + per - 1) / per);
+    pl.solve_many = items[0] > 2 * probs[slots[0]]->n_slabs * 8;   // n_slabs: two per SM
     pl.off_cs_s = o; h[o] = 0;
     for (int k = 0; k < A; ++k) {
       const DevProb& Q = P(slots[k]);
@@ -257,7 +295,7 @@ struct Runner {
       const bool f32 = prec == 1;
       const size_t off = o;
       size_t smem = 0;
-      int cap = 1 << 30, pw = 0, tpt = 0, btpt = 0, bfull = 0;
+      int cap = 1 << 30, tpt = 0, btpt = 0, bfull = 0;
       size_t rts = 0, bsm = 0;
       int bcap = 1 << 30, nbig = 0;
       for (int k = 0; k < A; ++k) {
@@ -287,19 +325,17 @@ struct Runner {
           need = std::max(need, vb);
           if (sb <= KSMEM_LIMIT) { fl |= 2; need = std::max(need, sb); }
         }
-        const size_t ss = sizeof(double) * ((size_t)Q.p * Q.p + Q.p);
+        const size_t ss = sizeof(double) * schur_doubles(Q.p);
         if (ss <= KSMEM_LIMIT) need = std::max(need, ss);
         // the cooperative kernel uses a global slab only for reduction blocks
         if (!(fl & 2)) cap = std::min(cap, probs[slots[k]]->n_slabs);
         smem = std::max(smem, need);
         h[off + k] = fl;
-        pw = std::max(pw, std::max(Q.ext, Q.bext));
       }
       o += A;
       if (f32) pl.off_f32 = off; else pl.off_f64 = off;
       pl.smem_f[prec] = smem;
       pl.cap_f[prec] = cap;
-      pl.per_warp[prec] = pw;
       pl.rt_threads[prec] = tpt;
       pl.rt_smem[prec] = rts;
       pl.big_grid[prec] = nbig > 0 ? std::min(bcap, pl.tot_elem) : 0;
@@ -432,16 +468,11 @@ struct Runner {
     Plan& pl = plans[which];
     err_fresh = false;
     cudaError_t e;
-    const int per = std::max(1, schedule().solve_elems);
-    const int want = std::max(pl.A, (pl.tot_elem + per - 1) / per);
-    if (prec == COLLO_PRECISION_MIXED)
-      e = launch_solve_b<float>(d_insts, pl.act(), pl.A, pl.pre_elem(), pl.pre_lv(), pl.maxL, pl.lsplit,
-                                pl.pre_cs_r(), ir, pl.per_warp[1], gbar, pl.max_p, want, stream,
-                                reserve_sms);
-    else
-      e = launch_solve_b<double>(d_insts, pl.act(), pl.A, pl.pre_elem(), pl.pre_lv(), pl.maxL, pl.lsplit,
-                                 pl.pre_cs_r(), ir, pl.per_warp[0], gbar, pl.max_p, want, stream,
-                                 reserve_sms);
+    const int* elem[2] = {pl.solve_elem(0), pl.solve_elem(1)};
+    const int* lv[2] = {pl.solve_lv(0), pl.solve_lv(1)};
+    auto launch = prec == COLLO_PRECISION_MIXED ? launch_solve_b<float> : launch_solve_b<double>;
+    e = launch(d_insts, pl.act(), pl.A, elem, lv, pl.pre_lv(), pl.maxL, pl.lsplit, pl.pre_cs_r(), ir,
+               pl.solve_pn, pl.solve_many, pl.solve_pw, gbar, pl.max_p, pl.solve_want, stream, reserve_sms);
     COLLO_CUDA(e);
     return COLLO_OK;
   }

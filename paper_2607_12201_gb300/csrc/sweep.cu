@@ -36,6 +36,7 @@
 #include <mutex>
 
 #include "problem.cuh"
+#include "subst.cuh"
 
 namespace collo {
 
@@ -221,28 +222,6 @@ __device__ bool sweep_invert_mem(float* m, int dim, const SweepMem& s) {
     sweep_bar<NW>();
   }
   return true;
-}
-
-// Sums over the warp of y[0 .. R-1] per lane, R = 8 or 16: halves are exchanged
-// instead of adding every value across all lanes (R - 1 + 5 - log2 R shuffles
-// instead of 5 R).  Lane l returns the sum of row l >> (5 - log2 R).
-template <int R>
-__device__ inline float warp_rows_sum(float (&y)[R]) {
-  const int lane = threadIdx.x & 31;
-  int o = 16;
-#pragma unroll
-  for (int h = R / 2; h > 0; h >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const float keep = up ? y[k + h] : y[k], give = up ? y[k] : y[k + h];
-      y[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-    }
-  }
-  float v = y[0];
-#pragma unroll
-  for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // CPL > 0: the inverse in registers (RPW x CPL per thread); CPL = 0: in memory
@@ -448,7 +427,7 @@ __device__ void sweep_one(const DevProb& P, double* __restrict__ x, int* __restr
 #pragma unroll
               for (int c = 0; c < CPL; ++c) y[k] = fmaf(m[k][c], bv[c], y[k]);
           }
-          const float mine = warp_rows_sum<R2>(y);
+          const float mine = warp_rows_sum<float, R2>(y);
           if (my_z >= 0) apply(my_z, mine);
         } else {
           for (int i2 = warp; i2 < dim; i2 += NW) {
