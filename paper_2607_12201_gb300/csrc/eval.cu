@@ -50,6 +50,23 @@ __global__ void k_obs_weights(DevProb P, int M, int N, double T, const double* _
   }
 }
 
+// Doubles of an element's states, multipliers and reaction terms in shared memory.
+__host__ __device__ inline int eval_base(const DevProb& P) {
+  return 2 * P.np * P.n + 3 * P.r + 4 * P.K * P.r;
+}
+// Doubles of the staging buffer of the derivative rows: all of an element's rows,
+// or as many as fit 40 KB (five blocks per SM at 30 species), at least one if
+// the shared memory has room.
+__host__ __device__ inline int eval_stage(const DevProb& P) {
+  const int width = 2 * (P.n + P.p), rows = P.K * P.n;
+  const int room = 224 * 1024 / 8 - eval_base(P);
+  int fit = 40 * 1024 / 8 / width;
+  if (fit < 1) fit = 1;
+  if (fit > rows) fit = rows;
+  if (fit * width > room) fit = room > 0 ? room / width : 0;
+  return width * fit;
+}
+
 // Rate constant of reaction j and its first and second theta derivatives.
 __device__ inline void rate_const(const DevProb& P, int j, const double* x, const double* dx,
                                   double alpha, double& k, double& dk, double& d2k) {
@@ -73,11 +90,15 @@ __device__ inline void rate_const(const DevProb& P, int j, const double* x, cons
 
 // One block per element i.  Evaluates at x + alpha dx (dx may be null).
 // DERIV = false: residuals, objective and norms only (line-search trials).
+// sm: eval_smem_bytes, of them the last `stage` doubles for the derivative rows.
+// Bound: the derivative blocks' stores (HBM).  30 species, 60 parameters, 2000
+// elements: 259 us with rows written entry by entry from their threads, XXX us
+// through shared memory.
 template <bool DERIV>
 __device__ void eval_elem(const DevProb& P, const double* __restrict__ x,
                           const double* __restrict__ dx, double alpha,
                           const double* __restrict__ lam, double obj_factor, const DevEval& E,
-                          int i, double* sm, double* red) {
+                          int i, double* sm, int stage, double* red) {
   const int n = P.n, r = P.r, p = P.p, K = P.K, np = P.np;
   const int tid = threadIdx.x;
   double* ze = sm;              // [K+1][n]
@@ -216,12 +237,12 @@ __device__ void eval_elem(const DevProb& P, const double* __restrict__ x,
   // (into column pidx[r]).  Row t of Wzz / Wzt at node k accumulates, over the
   // reactions consuming t, -h om_r k_r d2mon_r/dz_t dz_u and
   // -h om_r dk_r dmon_r/dz_t.  Each row is owned by one thread (fixed order).
-  for (int idx = tid; idx < K * n; idx += EVAL_BS) {
+  // Rows are mostly zeros: as many as fit the staging buffer are accumulated in
+  // shared memory and leave in coalesced stores (an element's rows are
+  // contiguous in each array).
+  const int rows = K * n, width = 2 * (n + p);
+  auto jac_row = [&](double* jz, double* jt, int idx) {
     const int k = idx / n + 1, s = idx - (k - 1) * n;
-    double* jz = E.JZ + (((size_t)i * K + (k - 1)) * n + s) * n;
-    double* jt = E.JT + (((size_t)i * K + (k - 1)) * n + s) * p;
-    for (int t = 0; t < n; ++t) jz[t] = 0.0;
-    for (int q = 0; q < p; ++q) jt[q] = 0.0;
     for (int e = P.nu_ptr[s]; e < P.nu_ptr[s + 1]; ++e) {
       const int rr = P.nu_r[e];
       const int a = P.react[2 * rr], b = P.react[2 * rr + 1];
@@ -232,29 +253,59 @@ __device__ void eval_elem(const DevProb& P, const double* __restrict__ x,
       const int q = P.pidx[rr];
       if (q >= 0) jt[q] += c * dkr[rr] * mon[mi];
     }
-  }
-  for (int idx = tid; idx < K * n; idx += EVAL_BS) {
-    const int k = idx / n + 1, t = idx - (k - 1) * n;
-    double* wz = E.Wzz + (((size_t)i * K + (k - 1)) * n + t) * n;
-    double* wt = E.Wzt + (((size_t)i * K + (k - 1)) * n + t) * p;
-    for (int u = 0; u < n; ++u) wz[u] = 0.0;
-    for (int q = 0; q < p; ++q) wt[q] = 0.0;
-    for (int e = P.rs_ptr[t]; e < P.rs_ptr[t + 1]; ++e) {
+  };
+  auto hess_row = [&](double* wz, double* wt, int idx) {
+    const int k = idx / n + 1, s = idx - (k - 1) * n;
+    for (int e = P.rs_ptr[s]; e < P.rs_ptr[s + 1]; ++e) {
       const int rr = P.rs_r[e];
       const int a = P.react[2 * rr], b = P.react[2 * rr + 1];
       const int mi = (k - 1) * r + rr;
       const double c = mh * om[mi];
       if (b >= 0) {
-        if (a == b) wz[t] += c * kr[rr] * 2.0;
-        else wz[a == t ? b : a] += c * kr[rr];
+        if (a == b) wz[s] += c * kr[rr] * 2.0;
+        else wz[a == s ? b : a] += c * kr[rr];
       }
       const int q = P.pidx[rr];
       if (q >= 0) {
         double dm = 0.0;
-        if (a == t) dm += da[mi];
-        if (b == t) dm += db[mi];
+        if (a == s) dm += da[mi];
+        if (b == s) dm += db[mi];
         wt[q] += c * dkr[rr] * dm;
       }
+    }
+  };
+  const size_t oz = (size_t)i * rows * n, ot = (size_t)i * rows * p;
+  if (stage < width) {   // no room beside a very large network: in place
+    for (int t = tid; t < rows * n; t += EVAL_BS) E.JZ[oz + t] = E.Wzz[oz + t] = 0.0;
+    for (int t = tid; t < rows * p; t += EVAL_BS) E.JT[ot + t] = E.Wzt[ot + t] = 0.0;
+    __syncthreads();
+    for (int t = tid; t < 2 * rows; t += EVAL_BS) {
+      const int idx = t < rows ? t : t - rows;
+      const size_t z = oz + (size_t)idx * n, q = ot + (size_t)idx * p;
+      if (t < rows) jac_row(E.JZ + z, E.JT + q, idx);
+      else hess_row(E.Wzz + z, E.Wzt + q, idx);
+    }
+  } else {
+    double* st = om + K * r;
+    const int RB = min(rows, stage / width);
+    for (int r0 = 0; r0 < rows; r0 += RB) {
+      const int nr = min(RB, rows - r0);
+      double* sjz = st;                 // [nr][n]
+      double* sjt = sjz + nr * n;       // [nr][p]
+      double* swz = sjt + nr * p;       // [nr][n]
+      double* swt = swz + nr * n;       // [nr][p]
+      for (int t = tid; t < nr * width; t += EVAL_BS) st[t] = 0.0;
+      __syncthreads();
+      for (int t = tid; t < 2 * nr; t += EVAL_BS) {
+        const int row = t < nr ? t : t - nr;
+        if (t < nr) jac_row(sjz + row * n, sjt + row * p, r0 + row);
+        else hess_row(swz + row * n, swt + row * p, r0 + row);
+      }
+      __syncthreads();
+      const size_t z = oz + (size_t)r0 * n, q = ot + (size_t)r0 * p;
+      for (int t = tid; t < nr * n; t += EVAL_BS) { E.JZ[z + t] = sjz[t]; E.Wzz[z + t] = swz[t]; }
+      for (int t = tid; t < nr * p; t += EVAL_BS) { E.JT[q + t] = sjt[t]; E.Wzt[q + t] = swt[t]; }
+      __syncthreads();
     }
   }
   // theta-theta diagonal partial sums of this element
@@ -276,7 +327,7 @@ k_eval(DevProb P, const double* __restrict__ x, const double* __restrict__ dx, d
        const double* __restrict__ lam, double obj_factor, DevEval E) {
   extern __shared__ double sm[];
   __shared__ double red[EVAL_BS];
-  eval_elem<DERIV>(P, x, dx, alpha, lam, obj_factor, E, blockIdx.x, sm, red);
+  eval_elem<DERIV>(P, x, dx, alpha, lam, obj_factor, E, blockIdx.x, sm, eval_stage(P), red);
 }
 
 // Vector selectors of the batched kernels (which per-instance array to use).
@@ -306,65 +357,67 @@ k_eval_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
   const int k = find_item(pre, A, t);
   const DevInst& I = insts[act[k]];
   eval_elem<DERIV>(I.P, pick_vec(I, xsel), pick_vec(I, dxsel), prm[k].alpha, pick_vec(I, lsel),
-                   prm[k].obj_factor, I.E, t - pre[k], sm, red);
+                   prm[k].obj_factor, I.E, t - pre[k], sm, eval_stage(I.P), red);
 }
 
-// Sum the per-element partials in a fixed order: phi, |c|_1, |c|_inf, W_thth.
-__device__ void eval_reduce_one(const DevProb& P, const DevEval& E, int deriv, double* out,
+// Sum the per-element partials in a fixed order: block 0 of the instance's
+// theta_blocks phi, |c|_1, |c|_inf (its first RED_BS threads: strided partial sums
+// and a fixed tree), the others 32 columns of W_thth each.  TH_BS threads.
+__device__ void eval_reduce_one(const DevProb& P, const DevEval& E, double* out, int block,
                                 double* sh) {
   const int tid = threadIdx.x;
-  double a = 0.0, b = 0.0, c = 0.0;
-  for (int i = tid; i < P.N; i += RED_BS) {
-    a += E.part[i * 4 + 0];
-    b += E.part[i * 4 + 1];
-    c = fmax(c, E.part[i * 4 + 2]);
+  if (block > 0) {
+    const int q0 = 32 * (block - 1);
+    const double v = column_sums(E.wtt_part, P.N, P.p, q0, sh);
+    if (tid < 32 && q0 + tid < P.p) E.wtt[q0 + tid] = v;
+    return;
   }
-  a = block_sum<RED_BS>(a, sh);
-  b = block_sum<RED_BS>(b, sh);
-  c = block_max<RED_BS>(c, sh);
+  double a = 0.0, b = 0.0, c = 0.0;
+  if (tid < RED_BS)
+    for (int i = tid; i < P.N; i += RED_BS) {
+      a += E.part[i * 4 + 0];
+      b += E.part[i * 4 + 1];
+      c = fmax(c, E.part[i * 4 + 2]);
+    }
+  a = first_sum<RED_BS>(a, sh);
+  b = first_sum<RED_BS>(b, sh);
+  c = first_max<RED_BS>(c, sh);
   if (tid == 0) {
     E.red[0] = a; E.red[1] = b; E.red[2] = c;
     if (out) { out[O_PHI] = a; out[O_C1] = b; out[O_CINF] = c; }
   }
-  if (!deriv) return;
-  // W_thth: warp w sums column q over elements lane, lane + 32, ... then a
-  // fixed shuffle tree
-  const int lane = tid & 31, warp = tid >> 5;
-  for (int q = warp; q < P.p; q += RED_BS / 32) {
-    double v = 0.0;
-    for (int i = lane; i < P.N; i += 32) v += E.wtt_part[(size_t)i * P.p + q];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) E.wtt[q] = v;
-  }
 }
 
-__global__ void __launch_bounds__(RED_BS) k_eval_reduce(DevProb P, DevEval E, int deriv) {
-  __shared__ double sh[RED_BS];
-  eval_reduce_one(P, E, deriv, nullptr, sh);
+__global__ void __launch_bounds__(TH_BS) k_eval_reduce(DevProb P, DevEval E) {
+  __shared__ double sh[32 * 33];
+  eval_reduce_one(P, E, nullptr, blockIdx.x, sh);
 }
 
 // Reduction of collo_eval_noalloc: the partials in the fixed scratch, Phi
 // into the caller's output (out[0] = Phi).
-__global__ void __launch_bounds__(RED_BS) k_eval_reduce_noalloc(DevProb P, DevEval E, double* phi) {
-  __shared__ double sh[RED_BS];
-  eval_reduce_one(P, E, 1, nullptr, sh);
-  if (threadIdx.x == 0) *phi = E.red[0];
+__global__ void __launch_bounds__(TH_BS) k_eval_reduce_noalloc(DevProb P, DevEval E, double* phi) {
+  __shared__ double sh[32 * 33];
+  eval_reduce_one(P, E, nullptr, blockIdx.x, sh);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *phi = E.red[0];
 }
 
-__global__ void __launch_bounds__(RED_BS)
-k_eval_reduce_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int deriv) {
-  __shared__ double sh[RED_BS];
+__global__ void __launch_bounds__(TH_BS)
+k_eval_reduce_b(const DevInst* __restrict__ insts, const int* __restrict__ act) {
+  __shared__ double sh[32 * 33];
   const DevInst& I = insts[act[blockIdx.x]];
-  eval_reduce_one(I.P, I.E, deriv, I.out, sh);
+  if ((int)blockIdx.y >= theta_blocks(I.P.p)) return;
+  eval_reduce_one(I.P, I.E, I.out, blockIdx.y, sh);
 }
 
 __global__ void __launch_bounds__(EVAL_BS)
 k_kkt_resid(DevProb P, DevEval E, const double* __restrict__ sigma, double dw, double dc,
             const double* __restrict__ vx, const double* __restrict__ vl,
             const double* __restrict__ bx, double bxs, const double* __restrict__ bc, double bcs,
-            double* __restrict__ rout, double* __restrict__ thpart, double* __restrict__ npart) {
-  __shared__ double red[EVAL_BS];
-  resid_elem(P, E, sigma, dw, dc, vx, vl, bx, bxs, bc, bcs, rout, thpart, npart, blockIdx.x, red);
+            double* __restrict__ rout, double* __restrict__ thpart, double* __restrict__ npart,
+            double* __restrict__ out) {
+  __shared__ unsigned long long red[3 * EVAL_BS / 32];
+  resid_elem(P, E, sigma, dw, dc, vx, vl, bx, bxs, bc, bcs, rout, thpart, npart, blockIdx.x, red,
+             out);
 }
 
 // BS: 64 when every instance of the batch has at most 64 state rows per
@@ -373,39 +426,41 @@ template <int BS>
 __global__ void __launch_bounds__(BS)
 k_kkt_resid_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
               const int* __restrict__ pre, const InstParams* __restrict__ prm, int mode) {
-  __shared__ double red[BS];
+  __shared__ unsigned long long red[3 * BS / 32];
   const int t = blockIdx.x;
   const int k = find_item(pre, A, t);
   const DevInst& I = insts[act[k]];
   const ResidArgs a = resid_args(I, prm[k], mode);
   resid_elem<BS>(I.P, I.E, a.sigma, a.dw, a.dc, a.vx, a.vl, a.bx, a.bxs, a.bc, a.bcs, a.rout,
-                 I.thpart, I.npart, t - pre[k], red);
+                 I.thpart, I.npart, t - pre[k], red, I.out + O_RX);
 }
 
-__global__ void __launch_bounds__(RED_BS)
+__global__ void __launch_bounds__(TH_BS)
 k_kkt_resid_theta(DevProb P, DevEval E, const double* __restrict__ sigma, double dw,
                   const double* __restrict__ vx, const double* __restrict__ bx, double bxs,
                   const double* __restrict__ bc, double* __restrict__ rout,
                   const double* __restrict__ thpart, const double* __restrict__ npart,
                   const double* __restrict__ th_extra, double* __restrict__ out) {
-  __shared__ double sh[RED_BS];
-  resid_theta_one(P, E, sigma, dw, vx, bx, bxs, bc, rout, thpart, npart, th_extra, out, sh);
+  __shared__ double sh[32 * 33];
+  resid_theta_one(P, E, sigma, dw, vx, bx, bxs, bc, rout, thpart, npart, th_extra, out,
+                  blockIdx.y, sh);
 }
 
-__global__ void __launch_bounds__(RED_BS)
+__global__ void __launch_bounds__(TH_BS)
 k_kkt_resid_theta_b(const DevInst* __restrict__ insts, const int* __restrict__ act,
                     const InstParams* __restrict__ prm, int mode) {
-  __shared__ double sh[RED_BS];
+  __shared__ double sh[32 * 33];
   const int k = blockIdx.x;
   const DevInst& I = insts[act[k]];
+  if ((int)blockIdx.y >= theta_blocks(I.P.p)) return;
   const ResidArgs a = resid_args(I, prm[k], mode);
   resid_theta_one(I.P, I.E, a.sigma, a.dw, a.vx, a.bx, a.bxs, a.bc, a.rout, I.thpart, I.npart,
-                  a.th_extra, I.out + O_RX, sh);
+                  a.th_extra, I.out + O_RX, blockIdx.y, sh);
 }
 
 // ---- host launchers -------------------------------------------------------------
-size_t eval_smem_bytes(const DevProb& P) {
-  return sizeof(double) * (size_t)(2 * P.np * P.n + 3 * P.r + 4 * P.K * P.r);
+size_t eval_smem_bytes(const DevProb& P, bool deriv) {
+  return sizeof(double) * ((size_t)eval_base(P) + (deriv ? eval_stage(P) : 0));
 }
 
 cudaError_t launch_obs_weights(const DevProb& P, int M, int N, double T, const double* t,
@@ -419,7 +474,7 @@ cudaError_t launch_obs_weights(const DevProb& P, int M, int N, double T, const d
 cudaError_t launch_eval(const DevProb& P, const DevEval& E, const double* x, const double* dx,
                         double alpha, const double* lam, double obj_factor, bool deriv,
                         cudaStream_t st) {
-  size_t sm = eval_smem_bytes(P);
+  size_t sm = eval_smem_bytes(P, deriv);
   if (deriv) {
     if (sm > SMEM_OPTIN_ABOVE)
       cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -434,7 +489,7 @@ cudaError_t launch_eval(const DevProb& P, const DevEval& E, const double* x, con
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   count_launch();
-  k_eval_reduce<<<1, RED_BS, 0, st>>>(P, E, deriv ? 1 : 0);
+  k_eval_reduce<<<deriv ? theta_blocks(P.p) : 1, TH_BS, 0, st>>>(P, E);
   return cudaGetLastError();
 }
 
@@ -448,11 +503,11 @@ cudaError_t launch_kkt_resid(const DevProb& P, const DevEval& E, const double* s
                              cudaStream_t st) {
   count_launch();
   k_kkt_resid<<<P.N, EVAL_BS, 0, st>>>(P, E, sigma, dw, dc, vx, vl, bx, bxs, bc, bcs, rout,
-                                       thpart, npart);
+                                       thpart, npart, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   count_launch();
-  k_kkt_resid_theta<<<1, RED_BS, 0, st>>>(P, E, sigma, dw, vx, bx, bxs, bc, rout, thpart, npart,
+  k_kkt_resid_theta<<<dim3(1, theta_blocks(P.p)), TH_BS, 0, st>>>(P, E, sigma, dw, vx, bx, bxs, bc, rout, thpart, npart,
                                           th_extra, out);
   return cudaGetLastError();
 }
@@ -493,7 +548,7 @@ static cudaError_t noalloc_scratch(int dev, double** out) {
 // ---- batched launchers (plan arrays in device memory) --------------------------
 cudaError_t launch_eval_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
                           int total_elems, const InstParams* prm, int xsel, int dxsel, int lsel,
-                          bool deriv, size_t smem, cudaStream_t st) {
+                          bool deriv, size_t smem, int max_p, cudaStream_t st) {
   if (A == 0) return cudaSuccess;
   if (deriv) {
     if (smem > SMEM_OPTIN_ABOVE)
@@ -509,12 +564,12 @@ cudaError_t launch_eval_b(const DevInst* insts, const int* act, int A, const int
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   count_launch();
-  k_eval_reduce_b<<<A, RED_BS, 0, st>>>(insts, act, deriv ? 1 : 0);
+  k_eval_reduce_b<<<dim3(A, deriv ? theta_blocks(max_p) : 1), TH_BS, 0, st>>>(insts, act);
   return cudaGetLastError();
 }
 
 cudaError_t launch_resid_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
-                           int total_elems, int max_n, const InstParams* prm, int mode,
+                           int total_elems, int max_n, int max_p, const InstParams* prm, int mode,
                            cudaStream_t st) {
   if (A == 0) return cudaSuccess;
   count_launch();
@@ -525,7 +580,7 @@ cudaError_t launch_resid_b(const DevInst* insts, const int* act, int A, const in
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   count_launch();
-  k_kkt_resid_theta_b<<<A, RED_BS, 0, st>>>(insts, act, prm, mode);
+  k_kkt_resid_theta_b<<<dim3(A, theta_blocks(max_p)), TH_BS, 0, st>>>(insts, act, prm, mode);
   return cudaGetLastError();
 }
 
@@ -605,14 +660,14 @@ extern "C" collo_status collo_eval_noalloc(collo_problem* prob, const double* x,
   E.wtt_part = scratch + (size_t)P.N * 4;             // [N][p]
   E.red = scratch + (size_t)P.N * (4 + (size_t)P.p);  // [8]
   cudaStream_t st = stream ? (cudaStream_t)stream : prob->stream;
-  const size_t sm = eval_smem_bytes(P);
+  const size_t sm = eval_smem_bytes(P, true);
   if (sm > SMEM_OPTIN_ABOVE)
     COLLO_CUDA(cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   count_launch();
   k_eval<true><<<P.N, EVAL_BS, sm, st>>>(P, x, nullptr, 0.0, lambda, obj_factor, E);
   COLLO_CUDA(cudaGetLastError());
   count_launch();
-  k_eval_reduce_noalloc<<<1, RED_BS, 0, st>>>(P, E, out->phi);
+  k_eval_reduce_noalloc<<<theta_blocks(P.p), TH_BS, 0, st>>>(P, E, out->phi);
   COLLO_CUDA(cudaGetLastError());
   return COLLO_OK;
 }

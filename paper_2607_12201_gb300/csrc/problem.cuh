@@ -11,7 +11,7 @@ struct collo_problem;
 namespace collo {
 
 // launchers (eval.cu)
-size_t eval_smem_bytes(const DevProb& P);
+size_t eval_smem_bytes(const DevProb& P, bool deriv);
 cudaError_t launch_obs_weights(const DevProb& P, int M, int N, double T, const double* t,
                                int* elem, double* w, cudaStream_t st);
 cudaError_t launch_eval(const DevProb& P, const DevEval& E, const double* x, const double* dx,
@@ -63,9 +63,9 @@ size_t sweep_work_floats(const DevProb& P);
 // grids leave to kernels of another stream
 cudaError_t launch_eval_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
                           int total_elems, const InstParams* prm, int xsel, int dxsel, int lsel,
-                          bool deriv, size_t smem, cudaStream_t st);
+                          bool deriv, size_t smem, int max_p, cudaStream_t st);
 cudaError_t launch_resid_b(const DevInst* insts, const int* act, int A, const int* pre_elem,
-                           int total_elems, int max_n, const InstParams* prm, int mode,
+                           int total_elems, int max_n, int max_p, const InstParams* prm, int mode,
                            cudaStream_t st);
 template <typename T>
 cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const int* pre_elem,

@@ -9,6 +9,72 @@ namespace collo {
 
 constexpr int EVAL_BS = 128;
 constexpr int RED_BS = 256;
+constexpr int TH_BS = 1024;   // threads of the per-instance reductions over elements
+
+// |v| as bits that order like the values, a value that is not a number as zero
+// (fmax passes over one).  Comparing them costs integer instructions; an FP64
+// one holds its pipe for 64 cycles per warp.
+__device__ inline unsigned long long abs_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return b > 0x7ff0000000000000ull ? 0ull : b;
+}
+__device__ inline unsigned long long max_bits(unsigned long long a, unsigned long long b) {
+  return a > b ? a : b;
+}
+// Block-wide maxima of three such values, valid on warp 0; sh: 3 (BS / 32)
+// words.  The values are maxima: their order does not matter.
+template <int BS>
+__device__ inline void block_max3(unsigned long long& a, unsigned long long& b,
+                                  unsigned long long& c, unsigned long long* sh) {
+  constexpr int NW = BS / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto shuffle = [&](unsigned long long& v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_bits(v, __shfl_xor_sync(0xffffffffu, v, o));
+  };
+  shuffle(a); shuffle(b); shuffle(c);
+  if (lane == 0) { sh[warp] = a; sh[NW + warp] = b; sh[2 * NW + warp] = c; }
+  __syncthreads();
+  if (warp == 0) {
+    a = lane < NW ? sh[lane] : 0ull;
+    b = lane < NW ? sh[NW + lane] : 0ull;
+    c = lane < NW ? sh[2 * NW + lane] : 0ull;
+    shuffle(a); shuffle(b); shuffle(c);
+  }
+}
+// Column sums of v[N][L] for the 32 columns from q0 on, by TH_BS threads: per
+// column 32 partial sums over i = l, l + 32, ... in that order, then a fixed tree;
+// the sum of column q0 + tid is valid on threads tid < 32.  A warp reads 32
+// neighbouring columns of a row, so the loads are whole lines (one warp per column
+// read a sector per lane: 50 species, 2000 elements 225 us for all columns on one
+// SM, now a few us on p / 32 of them).  sh: 32 x 33 doubles.
+__device__ inline double column_sums(const double* __restrict__ v, int N, int L, int q0,
+                                     double* sh) {
+  const int ql = threadIdx.x & 31, l = threadIdx.x >> 5, q = q0 + ql;
+  double y = 0.0;
+  if (q < L)
+    for (int i0 = l; i0 < N; i0 += 256) {
+      double t[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) t[j] = i0 + 32 * j < N ? v[(size_t)(i0 + 32 * j) * L + q] : 0.0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (i0 + 32 * j < N) y += t[j];
+    }
+  sh[l * 33 + ql] = y;
+  __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (l < o) {
+      y += sh[(l + o) * 33 + ql];
+      sh[l * 33 + ql] = y;
+    }
+    __syncthreads();
+  }
+  return y;
+}
+// Blocks of an instance's reductions: the scalars, and 32 columns each.
+__host__ __device__ inline int theta_blocks(int p) { return 1 + (p + 31) / 32; }
 
 // Deterministic block reductions (fixed tree over a fixed thread order).
 template <int BS>
@@ -41,6 +107,36 @@ __device__ inline double block_max(double v, double* sh) {
   return r;
 }
 
+// The same over the first BS threads of a larger block (all its threads call).
+template <int BS>
+__device__ inline double first_sum(double v, double* sh) {
+  const int t = threadIdx.x;
+  if (t < BS) sh[t] = v;
+  __syncthreads();
+#pragma unroll
+  for (int s = BS / 2; s > 0; s >>= 1) {
+    if (t < s) sh[t] += sh[t + s];
+    __syncthreads();
+  }
+  double r = sh[0];
+  __syncthreads();
+  return r;
+}
+template <int BS>
+__device__ inline double first_max(double v, double* sh) {
+  const int t = threadIdx.x;
+  if (t < BS) sh[t] = v;
+  __syncthreads();
+#pragma unroll
+  for (int s = BS / 2; s > 0; s >>= 1) {
+    if (t < s) sh[t] = fmax(sh[t], sh[t + s]);
+    __syncthreads();
+  }
+  double r = sh[0];
+  __syncthreads();
+  return r;
+}
+
 // Structured FP64 product y = K v of the regularised KKT matrix
 //   [ W + diag(sigma) + dw I   J^T  ] [vx]
 //   [ J                       -dc I ] [vl]
@@ -50,14 +146,15 @@ __device__ inline double block_max(double v, double* sh) {
 // zeros).  One block per element computes the
 // element's 2 (K + 1) n rows and its contribution to the p parameter rows; norms per
 // element go to npart[i][0..2] (max |r_x|, max |r_c|, max |b| over the
-// element's rows).
+// element's rows).  The first element clears norms[0..2] for resid_theta_one.
 template <int BS = EVAL_BS>
 __device__ inline void resid_elem(const DevProb& P, const DevEval& E, const double* __restrict__ sigma,
                            double dw, double dc, const double* __restrict__ vx,
                            const double* __restrict__ vl, const double* __restrict__ bx,
                            double bxs, const double* __restrict__ bc, double bcs,
                            double* __restrict__ rout, double* __restrict__ thpart,
-                           double* __restrict__ npart, int i, double* red) {
+                           double* __restrict__ npart, int i, unsigned long long* red,
+                           double* __restrict__ norms) {
   const int n = P.n, p = P.p, N = P.N, K = P.K, np = P.np;
   const int tid = threadIdx.x;
   const size_t nz = (size_t)N * np * n, nx = nz + p;
@@ -71,7 +168,8 @@ __device__ inline void resid_elem(const DevProb& P, const DevEval& E, const doub
   const double* Wzt = E.Wzt + (size_t)i * K * np_;
   const double* Wob = E.Wobj + (size_t)i * n * np * np;
   const bool next = chain_next(P, i);
-  double mx = 0.0, mc = 0.0, mb = 0.0;
+  if (i == 0 && tid < 3) norms[tid] = 0.0;
+  unsigned long long mx = 0, mc = 0, mb = 0;
   for (int idx = tid; idx < np * n; idx += BS) {
     const int j = idx / n, s = idx - j * n;
     // primal row z[i][j][s]
@@ -109,11 +207,11 @@ __device__ inline void resid_elem(const DevProb& P, const DevEval& E, const doub
         else y -= vl[zoff + np * n + s];
       }
     }
-    if (bx) mb = fmax(mb, fabs(bx[zoff + idx]));
-    if (bc) mb = fmax(mb, fabs(bc[zoff + idx]));
+    if (bx) mb = max_bits(mb, abs_bits(bx[zoff + idx]));
+    if (bc) mb = max_bits(mb, abs_bits(bc[zoff + idx]));
     double rr = (bx ? bxs * bx[zoff + idx] : 0.0) - y;
     if (rout) rout[zoff + idx] = rr;
-    mx = fmax(mx, fabs(rr));
+    mx = max_bits(mx, abs_bits(rr));
     // dual row c[i][j][s]
     double yc = 0.0;
     if (vz) {
@@ -145,7 +243,7 @@ __device__ inline void resid_elem(const DevProb& P, const DevEval& E, const doub
     if (vl) yc -= dc * vl[zoff + idx];
     double rc = (bc ? bcs * bc[zoff + idx] : 0.0) - yc;
     if (rout) rout[nx + zoff + idx] = rc;
-    mc = fmax(mc, fabs(rc));
+    mc = max_bits(mc, abs_bits(rc));
   }
   // this element's part of the parameter rows
   for (int q = tid; q < p; q += BS) {
@@ -158,10 +256,12 @@ __device__ inline void resid_elem(const DevProb& P, const DevEval& E, const doub
       }
     thpart[(size_t)i * p + q] = y;
   }
-  mx = block_max<BS>(mx, red);
-  mc = block_max<BS>(mc, red);
-  mb = block_max<BS>(mb, red);
-  if (tid == 0) { npart[i * 3 + 0] = mx; npart[i * 3 + 1] = mc; npart[i * 3 + 2] = mb; }
+  block_max3<BS>(mx, mc, mb, red);
+  if (tid == 0) {
+    npart[i * 3 + 0] = __longlong_as_double((long long)mx);
+    npart[i * 3 + 1] = __longlong_as_double((long long)mc);
+    npart[i * 3 + 2] = __longlong_as_double((long long)mb);
+  }
 }
 
 // Residual modes of the batched product (which vectors of the instance):
@@ -192,9 +292,9 @@ __device__ inline ResidArgs resid_args(const DevInst& I, const InstParams& pr, i
 
 // Parameter rows of r = b - K v, and the global norms:
 // out[0] = max|r_x|, out[1] = max|r_c|, out[2] = max|b| (b may be null).
-// The element contributions thpart[N][p] are summed by warp w for the
-// columns q = w, w + 8, ...: lane-strided partial sums, then a fixed
-// shuffle tree.
+// Block 0 of the instance's theta_blocks takes the norms of the elements, block b
+// the parameters from 32 (b - 1) on (column_sums of thpart[N][p]); all raise
+// out[0..2] (cleared by resid_elem) to their maxima.  TH_BS threads.
 __device__ inline void resid_theta_one(const DevProb& P, const DevEval& E,
                                 const double* __restrict__ sigma, double dw,
                                 const double* __restrict__ vx, const double* __restrict__ bx,
@@ -202,34 +302,36 @@ __device__ inline void resid_theta_one(const DevProb& P, const DevEval& E,
                                 double* __restrict__ rout, const double* __restrict__ thpart,
                                 const double* __restrict__ npart,
                                 const double* __restrict__ th_extra, double* __restrict__ out,
-                                double* sh) {
+                                int block, double* sh) {
   const int tid = threadIdx.x, p = P.p, N = P.N;
-  const int lane = tid & 31, warp = tid >> 5;
   const size_t nz = (size_t)N * P.np * P.n;
-  double mx = 0.0, mc = 0.0, mb = 0.0;
-  for (int q = warp; q < p; q += RED_BS / 32) {
-    double y = 0.0;
-    for (int i = lane; i < N; i += 32) y += thpart[(size_t)i * p + q];
-    for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-    if (lane == 0) {
+  unsigned long long mx = 0, mc = 0, mb = 0;
+  if (block == 0) {
+    for (int i = tid; i < N; i += TH_BS) {
+      mx = max_bits(mx, abs_bits(npart[i * 3 + 0]));
+      mc = max_bits(mc, abs_bits(npart[i * 3 + 1]));
+      mb = max_bits(mb, abs_bits(npart[i * 3 + 2]));
+    }
+    if (bx)
+      for (int q = tid; q < p; q += TH_BS) mb = max_bits(mb, abs_bits(bx[nz + q]));
+  } else {
+    const int q0 = 32 * (block - 1), q = q0 + tid;
+    double y = column_sums(thpart, N, p, q0, sh);
+    if (tid < 32 && q < p) {
       if (vx) y += (E.wtt[q] + (sigma ? sigma[nz + q] : 0.0) + dw) * vx[nz + q];
       if (th_extra) y -= th_extra[q];
       const double rr = (bx ? bxs * bx[nz + q] : 0.0) - y;
       if (rout) rout[nz + q] = rr;
-      mx = fmax(mx, fabs(rr));
+      mx = abs_bits(rr);
     }
   }
-  for (int i = tid; i < N; i += RED_BS) {
-    mx = fmax(mx, npart[i * 3 + 0]);
-    mc = fmax(mc, npart[i * 3 + 1]);
-    mb = fmax(mb, npart[i * 3 + 2]);
+  block_max3<TH_BS>(mx, mc, mb, reinterpret_cast<unsigned long long*>(sh));
+  if (tid == 0) {
+    unsigned long long* o = reinterpret_cast<unsigned long long*>(out);
+    atomicMax(o, mx);
+    atomicMax(o + 1, mc);
+    atomicMax(o + 2, mb);
   }
-  if (bx)
-    for (int q = tid; q < p; q += RED_BS) mb = fmax(mb, fabs(bx[nz + q]));
-  mx = block_max<RED_BS>(mx, sh);
-  mc = block_max<RED_BS>(mc, sh);
-  mb = block_max<RED_BS>(mb, sh);
-  if (tid == 0) { out[0] = mx; out[1] = mc; out[2] = mb; }
 }
 
 }  // namespace collo

@@ -46,7 +46,8 @@ struct Plan {
   size_t off_act = 0, off_elem = 0, off_lv = 0, off_cs_s = 0, off_cs_r = 0, off_f32 = 0,
          off_f64 = 0, off_se[2] = {0, 0}, off_sl[2] = {0, 0};
   int sweep_threads = 0;
-  size_t smem_eval = 0, smem_f[2] = {0, 0}, smem_sweep = 0;
+  size_t smem_eval[2] = {0, 0};   // without / with derivatives
+  size_t smem_f[2] = {0, 0}, smem_sweep = 0;
   int cap_f[2] = {1 << 30, 1 << 30};
   int solve_pw = 0;             // rows of the largest block a CUDA block solves
   int solve_pn = 0;             // ... that one warp solves
@@ -350,8 +351,11 @@ struct Runner {
       pl.sweep_threads = std::max(pl.sweep_threads, sweep_block_threads(P(slots[k])));
       pl.smem_sweep = std::max(pl.smem_sweep, sweep_smem_bytes(P(slots[k])));
     }
-    pl.smem_eval = 0;
-    for (int k = 0; k < A; ++k) pl.smem_eval = std::max(pl.smem_eval, eval_smem_bytes(P(slots[k])));
+    for (int d = 0; d < 2; ++d) {
+      pl.smem_eval[d] = 0;
+      for (int k = 0; k < A; ++k)
+        pl.smem_eval[d] = std::max(pl.smem_eval[d], eval_smem_bytes(P(slots[k]), d != 0));
+    }
     pl.h_ll[0] = 0;
     for (int k = 0; k < A; ++k)
       pl.h_ll[k + 1] = pl.h_ll[k] + h_insts[slots[k]].n_x + h_insts[slots[k]].n_c;
@@ -417,13 +421,13 @@ struct Runner {
   collo_status eval(int which, int xsel, int dxsel, int lsel, bool deriv) {
     Plan& pl = plans[which];
     COLLO_CUDA(launch_eval_b(d_insts, pl.act(), pl.A, pl.pre_elem(), pl.tot_elem, pl.d_prm, xsel,
-                             dxsel, lsel, deriv, pl.smem_eval, stream));
+                             dxsel, lsel, deriv, pl.smem_eval[deriv ? 1 : 0], pl.max_p, stream));
     return COLLO_OK;
   }
   collo_status resid(int which, int mode) {
     Plan& pl = plans[which];
     COLLO_CUDA(launch_resid_b(d_insts, pl.act(), pl.A, pl.pre_elem(), pl.tot_elem, pl.max_n,
-                              pl.d_prm, mode, stream));
+                              pl.max_p, pl.d_prm, mode, stream));
     return COLLO_OK;
   }
   // parts: 1 register-tiled element condensation, 4 large-element condensation,
