@@ -92,7 +92,7 @@ __device__ inline void rate_const(const DevProb& P, int j, const double* x, cons
 // DERIV = false: residuals, objective and norms only (line-search trials).
 // sm: eval_smem_bytes, of them the last `stage` doubles for the derivative rows.
 // Bound: the derivative blocks' stores (HBM).  30 species, 60 parameters, 2000
-// elements: 259 us with rows written entry by entry from their threads, XXX us
+// elements: 259 us with rows written entry by entry from their threads, 240 us
 // through shared memory.
 template <bool DERIV>
 __device__ void eval_elem(const DevProb& P, const double* __restrict__ x,
