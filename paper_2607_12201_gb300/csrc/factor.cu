@@ -49,6 +49,33 @@ __device__ inline void pivot_inertia(double a, double b, double d, int& pos, int
 // Packed lower triangle: entry (r, c), c <= r, at r (r + 1) / 2 + c.
 __host__ __device__ inline int tri_at(int r, int c) { return r * (r + 1) / 2 + c; }
 
+// Layouts of a block's lower triangle.  PackedTri (shared memory, where every
+// byte counts): rows one after the other.  RowBlockTri (global slab): blocks
+// of 32 rows, each row-major with its leading dimension cut to the block's last
+// column, so that 32 x 32 tiles start on 128-byte lines (16 entries per row are
+// above the diagonal on average and never used).
+struct PackedTri {
+  static __host__ __device__ int at(int r, int c) { return tri_at(r, c); }
+  static __host__ __device__ size_t elems(int msz) {
+    return ((size_t)msz * (msz + 1) / 2 + 3) & ~size_t(3);   // a multiple of 16 bytes
+  }
+};
+struct RowBlockTri {
+  static __host__ __device__ int at(int r, int c) {
+    const int b = r >> 5;
+    return 32 * (b + 1) * (16 * b + (r & 31)) + c;
+  }
+  static __host__ __device__ size_t elems(int msz) {
+    const size_t b = (msz + 31) >> 5;
+    return 512 * b * (b + 1);
+  }
+};
+// The symmetric entry (a, b) of a triangle A.
+template <class Lay, typename T>
+__device__ inline T sym_at(const T* A, int a, int b) {
+  return A[a >= b ? Lay::at(a, b) : Lay::at(b, a)];
+}
+
 // Tile t of a lower triangle of tiles, numbered row by row: (ti, tj), tj <= ti.
 __device__ inline void tri_tile(int t, int& ti, int& tj) {
   int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
@@ -73,7 +100,7 @@ __host__ __device__ inline int panel_ld(int msz) { return (((msz + 92) >> 3) << 
 // sum in ascending k, subtracted once (the same arithmetic per entry as
 // trailing_update, so the result does not depend on which of the two a
 // launch uses).
-template <typename T>
+template <typename T, class Lay>
 __device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* __restrict__ Lp,
                                        const T* __restrict__ W, int ldw) {
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -93,7 +120,7 @@ __device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* 
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
           const int r = r0 + u, c = cb + v;
-          cur[u][v] = (r < msz && c <= r) ? A[tri_at(r, c)] : T(0);
+          cur[u][v] = (r < msz && c <= r) ? A[Lay::at(r, c)] : T(0);
         }
       T acc[4][4];
 #pragma unroll
@@ -119,7 +146,7 @@ __device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* 
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
           const int c = cb + v;
-          if (c <= r) A[tri_at(r, c)] = cur[u][v] - acc[u][v];
+          if (c <= r) A[Lay::at(r, c)] = cur[u][v] - acc[u][v];
         }
       }
     }
@@ -170,6 +197,26 @@ struct TileAcc {
 #pragma unroll
       for (int v = 0; v < TC; ++v) a[u][v] = fma(lr[u], uc[v], a[u][v]);
   }
+  // the same with w in runs of two columns, the runs 16 apart
+  __device__ void add_runs(const T* __restrict__ l, const T* __restrict__ w) {
+    T lr[TR], uc[TC];
+#pragma unroll
+    for (int u = 0; u < TR; u += 2) {
+      const double2 q = *reinterpret_cast<const double2*>(l + u);
+      lr[u] = q.x;
+      lr[u + 1] = q.y;
+    }
+#pragma unroll
+    for (int v = 0; v < TC; v += 2) {
+      const double2 q = *reinterpret_cast<const double2*>(w + 8 * v);
+      uc[v] = q.x;
+      uc[v + 1] = q.y;
+    }
+#pragma unroll
+    for (int u = 0; u < TR; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) a[u][v] = fma(lr[u], uc[v], a[u][v]);
+  }
   __device__ T get(int u, int v) const { return a[u][v]; }
 };
 template <int TR, int TC>
@@ -188,6 +235,28 @@ struct TileAcc<float, TR, TC> {
     for (int u = 0; u < TR / 4; ++u) lr[u] = reinterpret_cast<const ulonglong2*>(l)[u];
 #pragma unroll
     for (int v = 0; v < TC; ++v) uc[v] = pack2(w[8 * v], w[8 * v]);
+#pragma unroll
+    for (int u = 0; u < TR / 4; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) {
+        a[2 * u][v] = fma2(lr[u].x, uc[v], a[2 * u][v]);
+        a[2 * u + 1][v] = fma2(lr[u].y, uc[v], a[2 * u + 1][v]);
+      }
+  }
+  // the same with w in runs of four columns, the runs 32 apart
+  __device__ void add_runs(const float* __restrict__ l, const float* __restrict__ w) {
+    ulonglong2 lr[TR / 4];
+    unsigned long long uc[TC];
+#pragma unroll
+    for (int u = 0; u < TR / 4; ++u) lr[u] = reinterpret_cast<const ulonglong2*>(l)[u];
+#pragma unroll
+    for (int v = 0; v < TC; v += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(w + 8 * v);
+      uc[v] = pack2(q.x, q.x);
+      uc[v + 1] = pack2(q.y, q.y);
+      uc[v + 2] = pack2(q.z, q.z);
+      uc[v + 3] = pack2(q.w, q.w);
+    }
 #pragma unroll
     for (int u = 0; u < TR / 4; ++u)
 #pragma unroll
@@ -271,6 +340,60 @@ template <typename T>
 struct alignas(16) Quad {
   T v[16 / sizeof(T)];
 };
+
+// The same update of a triangle in the slab (RowBlockTri), in tiles on its
+// 128-byte lines: a warp owns a block's 32 rows x 8 TC columns, lane (ty, tx) the
+// rows 8 ty .. 8 ty + 7 and TC columns in 16-byte runs, 8 lanes side by side.
+// Every access is 16 bytes per lane over whole lines and none is predicated:
+// entries above the diagonal, past msz or before cend (in the tiles that
+// straddle it) take part too and are never read again.
+// Bound: the shared-memory loads of the products (12 wavefronts per 32
+// multiply-adds of a lane) and, at the start of a tile, L2.  50 species, 2000
+// elements, cycles per element in all trailing updates (condensation and
+// reduction): 756 000 with the packed triangle in the slab, whose rows start
+// anywhere (4 to 8 lines per access, each predicated), 498 000 so.
+template <typename T, int TC>
+__device__ __noinline__ void trailing_update_slab(T* A, int msz, int cend, int K,
+                                                  const T* __restrict__ Lp,
+                                                  const T* __restrict__ W, int ldw) {
+  constexpr int TR = 8, Q = 16 / sizeof(T), WC = 8 * TC;
+  static_assert(WC <= 32 && 32 + WC <= PANEL_PAD, "tiles inside the row blocks and panel buffers");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int ty = lane >> 3, tx = lane & 7;
+  if (msz <= cend) return;
+  const int nb = (msz + 31) >> 5, cb = cend & ~(WC - 1);
+  int blk = warp;
+  for (int b = cend >> 5; b < nb; ++b) {
+    const int ld = 32 * (b + 1), nbc = (ld - cb) / WC;
+    for (; blk < nbc; blk += nw) {
+      const int c0 = cb + blk * WC + Q * tx;
+      T* a = A + 512 * b * (b + 1) + TR * ty * ld + c0;
+      const T* lb = Lp + 32 * b + TR * ty;
+      const T* wb = W + c0;
+      // the tile's entries are loaded first, so that their latency overlaps the
+      // products
+      Quad<T> cur[TR][TC / Q];
+#pragma unroll
+      for (int u = 0; u < TR; ++u)
+#pragma unroll
+        for (int g = 0; g < TC / Q; ++g)
+          cur[u][g] = *reinterpret_cast<const Quad<T>*>(a + u * ld + 8 * Q * g);
+      TileAcc<T, TR, TC> acc;
+      acc.clear();
+#pragma unroll 2
+      for (int k = 0; k < K; ++k) acc.add_runs(lb + k * ldw, wb + k * ldw);
+#pragma unroll
+      for (int u = 0; u < TR; ++u)
+#pragma unroll
+        for (int g = 0; g < TC / Q; ++g) {
+#pragma unroll
+          for (int i = 0; i < Q; ++i) cur[u][g].v[i] -= acc.get(u, Q * g + i);
+          *reinterpret_cast<Quad<T>*>(a + u * ld + 8 * Q * g) = cur[u][g];
+        }
+    }
+    blk -= nbc;
+  }
+}
 
 // One pair's update of a row's remaining panel columns: x[j] -= l0 U0[j] +
 // l1 U1[j] for j = kk + 2 .. 2 PB - 1, each by two multiply-adds.  U0, U1: the
@@ -398,7 +521,7 @@ __device__ __noinline__ void panel_rows(T* W, T* Lp, int ldw, int msz, int cp, i
 // PB is 8 for blocks held in shared memory and 16 for blocks in the global
 // slab (half the trailing passes over global memory, twice the arithmetic per
 // entry read and written).
-template <typename T, int PB, int TR, int TC>
+template <typename T, class Lay, int PB, int TR, int TC>
 __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__ Lout, int lds,
                                       T* __restrict__ Dout, T* Lp, T* W,
                                       int* __restrict__ inert) {
@@ -420,7 +543,7 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
 #pragma unroll
         for (int i = 0; i < B; ++i) {
           const int ri = r + i * step * RW;
-          v[i] = (j < K && ri < hi && cp + j <= ri) ? A[tri_at(ri, cp + j)] : T(0);
+          v[i] = (j < K && ri < hi && cp + j <= ri) ? A[Lay::at(ri, cp + j)] : T(0);
         }
 #pragma unroll
         for (int i = 0; i < B; ++i) {
@@ -451,7 +574,9 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
     __syncthreads();
     // trailing rank-K update of rows / columns >= cend (lower part)
     if constexpr (TR == 0)
-      trailing_update_tiles4<T>(A, msz, cend, K, Lp, W, ldw);
+      trailing_update_tiles4<T, Lay>(A, msz, cend, K, Lp, W, ldw);
+    else if constexpr (std::is_same<Lay, RowBlockTri>::value)
+      trailing_update_slab<T, 16 / sizeof(T)>(A, msz, cend, K, Lp, W, ldw);
     else
       trailing_update<T, TR, TC>(A, msz, cend, K, Lp, W, ldw);
     __syncthreads();
@@ -470,28 +595,25 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
 // factorization limit; otherwise (PB = 16) the triangle in a per-CUDA-block
 // global slab (L2-resident) and the panel buffers in shared memory, or, when
 // even they do not fit, in the slab behind the triangle.
-__host__ __device__ inline size_t big_tri_elems(int msz) {
-  return ((size_t)msz * (msz + 1) / 2 + 3) & ~size_t(3);   // a multiple of 16 bytes
-}
 template <typename T>
 __host__ __device__ inline int big_pb(int msz) {
-  const size_t full8 = sizeof(T) * (2 * (size_t)16 * panel_ld(msz) + big_tri_elems(msz));
+  const size_t full8 = sizeof(T) * (2 * (size_t)16 * panel_ld(msz) + PackedTri::elems(msz));
   return full8 <= FACTOR_SMEM_LIMIT ? 8 : 16;
 }
 template <typename T>
 __host__ __device__ inline size_t big_panel_elems(int msz) {
   return 2 * (size_t)(2 * big_pb<T>(msz)) * panel_ld(msz);
 }
-// pair_eliminate_packed with PB = pb (8, or 16 for a block in the global slab,
-// whose panel buffers are sized for 16)
-template <typename T, int TR, int TC>
+// pair_eliminate_packed with PB = 8 (triangle in shared memory) or pb (8 or 16,
+// triangle in the global slab, whose panel buffers are sized for 16)
+template <typename T, class Lay, int TR, int TC>
 __device__ inline void pair_eliminate_big(T* A, int msz, int npairs, T* __restrict__ Lout,
                                           int lds, T* __restrict__ Dout, T* Lp, T* W,
                                           int* __restrict__ inert, int pb) {
-  if (pb == 16)
-    pair_eliminate_packed<T, 16, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
+  if (std::is_same<Lay, RowBlockTri>::value && pb == 16)
+    pair_eliminate_packed<T, Lay, 16, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
   else
-    pair_eliminate_packed<T, 8, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
+    pair_eliminate_packed<T, Lay, 8, TR, TC>(A, msz, npairs, Lout, lds, Dout, Lp, W, inert);
 }
 template <typename T>
 __host__ __device__ inline bool panel_in_global(int msz) {
@@ -499,7 +621,7 @@ __host__ __device__ inline bool panel_in_global(int msz) {
 }
 template <typename T>
 __host__ __device__ inline size_t slab_elems(int msz) {
-  return big_tri_elems(msz) + (panel_in_global<T>(msz) ? big_panel_elems<T>(msz) : 0);
+  return RowBlockTri::elems(msz) + (panel_in_global<T>(msz) ? big_panel_elems<T>(msz) : 0);
 }
 template <typename T>
 struct BigPlace {
@@ -513,9 +635,26 @@ __device__ inline BigPlace<T> big_place(unsigned char* smraw, T* work, int msz, 
   const size_t pn = big_panel_elems<T>(msz) / 2;
   T* slab = work + (size_t)blockIdx.x * slab_elems<T>(msz);
   const bool pg = !full && panel_in_global<T>(msz);
-  T* Lp = pg ? slab + big_tri_elems(msz) : reinterpret_cast<T*>(smraw);
+  T* Lp = pg ? slab + RowBlockTri::elems(msz) : reinterpret_cast<T*>(smraw);
   T* A = full ? Lp + 2 * pn : slab;
   return {A, Lp, Lp + pn};
+}
+
+// use(load(i)) for i = 0 .. cnt - 1 over the threads of the block, B independent
+// loads of a thread in flight before the first use (stores in use() would
+// otherwise keep the compiler from moving the next load up).
+template <int B, class Load, class Use>
+__device__ inline void for_loaded(int cnt, Load load, Use use) {
+  const int nt = blockDim.x;
+  for (int i = threadIdx.x; i < cnt; i += B * nt) {
+    decltype(load(0)) v[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (i + b * nt < cnt) v[b] = load(i + b * nt);
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (i + b * nt < cnt) use(i + b * nt, v[b]);
+  }
 }
 
 // Scatter assembly of element e's KKT block (packed lower triangle blk, zeroed)
@@ -526,7 +665,7 @@ __device__ inline BigPlace<T> big_place(unsigned char* smraw, T* work, int msz, 
 // threads of the block: disjoint entries (point Hessian blocks, the identity
 // parts of the collocation rows D[k][j], continuity / initial rows, -delta_c,
 // border), sums onto those (objective blocks, -h df/dz), then the diagonal.
-template <typename T>
+template <typename T, class Lay>
 __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double* Wzz,
                                           const double* JZ, const double* Wzt, const double* JT,
                                           const double* Wobj, const double* sig, double dw,
@@ -542,7 +681,7 @@ __device__ __noinline__ void gauss_chain_out(const DevProb& P, const DevFactor<T
 // -I; Gauss: gauss_chain_out).  For blocks above the register-tile limit
 // (elem_factor_rt below).  TR x TC: the trailing update's register tile
 // (trailing_update), set by the calling kernel's register budget.
-template <typename T, int TR, int TC>
+template <typename T, class Lay, int TR, int TC>
 __device__ void elem_factor_big(const DevProb& P, const DevEval& E,
                                 const double* __restrict__ sigma, double dw, double dc,
                                 const DevFactor<T>& F, int e, const BigPlace<T>& pl, int pb) {
@@ -552,39 +691,39 @@ __device__ void elem_factor_big(const DevProb& P, const DevEval& E,
   const int i0 = 2 * nint;         // first chain row (2Kn)
   const size_t nn = (size_t)n * n, np = (size_t)n * p;
   T* A = pl.A;
-  const int ntri = ext * (ext + 1) / 2;
-  for (int i = tid; i < ntri; i += nt) A[i] = T(0);
+  const int nq = (int)(Lay::elems(ext) * sizeof(T) / 16);
+  for (int i = tid; i < nq; i += nt) reinterpret_cast<int4*>(A)[i] = make_int4(0, 0, 0, 0);
   __syncthreads();
-  elem_scatter<T>(P, e, E.Wzz + (size_t)e * K * nn, E.JZ + (size_t)e * K * nn,
+  elem_scatter<T, Lay>(P, e, E.Wzz + (size_t)e * K * nn, E.JZ + (size_t)e * K * nn,
                   E.Wzt + (size_t)e * K * np, E.JT + (size_t)e * K * np,
                   E.Wobj + (size_t)e * npt * npt * n,
                   sigma ? sigma + (size_t)e * npt * n : nullptr, dw, dc, A);
   const int ldl = factor_ld<T>(ext);
-  pair_eliminate_big<T, TR, TC>(A, ext, nint, F.Lel + (size_t)e * (2 * nint) * ldl, ldl,
+  pair_eliminate_big<T, Lay, TR, TC>(A, ext, nint, F.Lel + (size_t)e * (2 * nint) * ldl, ldl,
                                 F.Del + (size_t)e * nint * 3, pl.Lp, pl.W,
                                 F.inert + (size_t)e * 3, pb);
   const int n2 = 2 * n;
-  auto tr = [&](int a, int b) { return a >= b ? A[tri_at(a, b)] : A[tri_at(b, a)]; };
+  auto tr = [&](int a, int b) { return sym_at<Lay>(A, a, b); };
   double* Sc = F.Scon + (size_t)e * p * p;
-  for (int idx = tid; idx < p * p; idx += nt) {
+  for_loaded<4>(p * p, [&](int idx) {
     const int q = idx / p, q2 = idx - q * p;
-    Sc[idx] = (double)tr(m + q, m + q2);
-  }
+    return tr(m + q, m + q2);
+  }, [&](int idx, T v) { Sc[idx] = (double)v; });
   if (P.gauss) {
     gauss_chain_out<T>(P, F, e, i0, dc, tr);
     __syncthreads();
     return;
   }
   T* Aif = F.Aif + (size_t)e * n2 * n2;
-  for (int idx = tid; idx < n2 * n2; idx += nt) {
+  for_loaded<4>(n2 * n2, [&](int idx) {
     const int u = idx / n2, v = idx - u * n2;
-    Aif[idx] = tr(i0 + u, i0 + v);
-  }
+    return tr(i0 + u, i0 + v);
+  }, [&](int idx, T v) { Aif[idx] = v; });
   T* Bif = F.Bif + (size_t)e * n2 * p;
-  for (int idx = tid; idx < n2 * p; idx += nt) {
+  for_loaded<4>(n2 * p, [&](int idx) {
     const int u = idx / p, q = idx - u * p;
-    Bif[idx] = A[tri_at(m + q, i0 + u)];
-  }
+    return A[Lay::at(m + q, i0 + u)];
+  }, [&](int idx, T v) { Bif[idx] = v; });
   T* C = F.Cpl + (size_t)e * n * n;
   for (int idx = tid; idx < n * n; idx += nt) {
     const int s2 = idx / n, t = idx - s2 * n;
@@ -599,9 +738,10 @@ k_elem_factor(DevProb P, DevEval E, const double* __restrict__ sigma, double dw,
               DevFactor<T> F, int use_smem, int slab_pb) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const BigPlace<T> pl = big_place<T>(smraw, F.work, P.ext, use_smem != 0);
+  constexpr int TC = sizeof(T) == 4 ? 8 : 4;
   for (int e = blockIdx.x; e < P.N; e += gridDim.x)
-    elem_factor_big<T, 8, sizeof(T) == 4 ? 8 : 4>(P, E, sigma, dw, dc, F, e, pl,
-                                                  use_smem ? 8 : slab_pb);
+    if (use_smem) elem_factor_big<T, PackedTri, 8, TC>(P, E, sigma, dw, dc, F, e, pl, 8);
+    else elem_factor_big<T, RowBlockTri, 8, TC>(P, E, sigma, dw, dc, F, e, pl, slab_pb);
 }
 
 // ---- 1'. pair elimination with the block held in registers -------------------------
@@ -948,10 +1088,10 @@ __device__ __noinline__ void elem_assemble_rt(const DevProb& P, const DevEval& E
   for (int i = tid; i < ntri; i += nt) blk[i] = T(0);
   cp_async_wait_all();
   __syncthreads();
-  elem_scatter<T>(P, e, Wzz, JZ, Wzt, JT, Wobj, sig, dw, dc, blk);
+  elem_scatter<T, PackedTri>(P, e, Wzz, JZ, Wzt, JT, Wobj, sig, dw, dc, blk);
 }
 
-template <typename T>
+template <typename T, class Lay>
 __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double* Wzz,
                                           const double* JZ, const double* Wzt, const double* JT,
                                           const double* Wobj, const double* sig, double dw,
@@ -959,17 +1099,27 @@ __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double*
   const int n = P.n, p = P.p, m = P.m, K = P.K, np = P.np;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nn = n * n, np_ = n * p;
-  auto put = [&](int a, int b, T v) { blk[a >= b ? tri_at(a, b) : tri_at(b, a)] = v; };
-  auto add = [&](int a, int b, T v) { blk[a >= b ? tri_at(a, b) : tri_at(b, a)] += v; };
+  auto put = [&](int a, int b, T v) { blk[a >= b ? Lay::at(a, b) : Lay::at(b, a)] = v; };
+  // an entry and what is added to it
+  struct Sum {
+    T* at;
+    T old;
+    double v;
+  };
+  auto sum = [&](int a, int b, double v) {
+    T* t = blk + (a >= b ? Lay::at(a, b) : Lay::at(b, a));
+    return Sum{t, *t, v};
+  };
+  auto store = [&](int, const Sum& q) { *q.at = q.old + (T)q.v; };
   // 1. disjoint entries: point Hessian blocks, the identity parts of the
   //    collocation rows (D[k][j]), continuity / initial rows, -delta_c, border
   const float inv_n = 1.f / (float)n, inv_p = p > 0 ? 1.f / (float)p : 0.f;
   const float inv_np = 1.f / (float)np;
-  for (int i = tid; i < K * nn; i += nt) {
+  for_loaded<4>(K * nn, [&](int i) { return Wzz[i]; }, [&](int i, double v) {
     const int rs = quot(i, n, inv_n), sb = i - rs * n;   // rs = k n + sa
     const int k = quot(rs, n, inv_n), sa = rs - k * n;
-    if (sa >= sb) put(loc_state(P, k + 1, sa), loc_state(P, k + 1, sb), (T)Wzz[i]);
-  }
+    if (sa >= sb) put(loc_state(P, k + 1, sa), loc_state(P, k + 1, sb), (T)v);
+  });
   for (int i = tid; i < K * np * n; i += nt) {
     const int kj = quot(i, n, inv_n), s2 = i - kj * n;
     const int k1 = quot(kj, np, inv_np), j = kj - k1 * np;
@@ -990,34 +1140,35 @@ __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double*
     const int a = loc_dual(P, k, s2);
     put(a, a, (T)(-dc));
   }
-  for (int i = tid; i < K * np_; i += nt) {
+  for_loaded<4>(K * np_, [&](int i) { return make_double2(Wzt[i], JT[i]); },
+                [&](int i, double2 v) {
     const int ks = quot(i, p, inv_p), q = i - ks * p;     // ks = k n + s
     const int k = quot(ks, n, inv_n), s2 = ks - k * n;
-    put(m + q, loc_state(P, k + 1, s2), (T)Wzt[i]);
-    put(m + q, loc_dual(P, k + 1, s2), (T)JT[i]);
-  }
+    put(m + q, loc_state(P, k + 1, s2), (T)v.x);
+    put(m + q, loc_dual(P, k + 1, s2), (T)v.y);
+  });
   __syncthreads();
   // 2. sums onto those: objective blocks (same species across points) and the
   //    -h df/dz part of the collocation rows
   const int np2 = np * np;
   const float inv_np2 = 1.f / (float)np2;
-  for (int i = tid; i < np2 * n; i += nt) {
+  for_loaded<4>(np2 * n, [&](int i) {
     const int s2 = quot(i, np2, inv_np2), jj = i - s2 * np2;
     const int ja = quot(jj, np, inv_np), jb = jj - ja * np;
     const int a = loc_state(P, ja, s2), b = loc_state(P, jb, s2);
-    if (a >= b) add(a, b, (T)Wobj[i]);
-  }
-  for (int i = tid; i < K * nn; i += nt) {
+    return a >= b ? sum(a, b, Wobj[i]) : Sum{nullptr, T(0), 0.0};
+  }, [&](int i, const Sum& q) { if (q.at) store(i, q); });
+  for_loaded<4>(K * nn, [&](int i) {
     const int rs = quot(i, n, inv_n), sp = i - rs * n;   // rs = k n + sd
     const int k = quot(rs, n, inv_n), sd = rs - k * n;
-    add(loc_dual(P, k + 1, sd), loc_state(P, k + 1, sp), (T)JZ[i]);
-  }
+    return sum(loc_dual(P, k + 1, sd), loc_state(P, k + 1, sp), JZ[i]);
+  }, store);
   __syncthreads();
   // 3. barrier diagonal and delta_w on the states
   for (int i = tid; i < np * n; i += nt) {
     const int j = quot(i, n, inv_n), s2 = i - j * n;
     const int a = loc_state(P, j, s2);
-    add(a, a, (T)((sig ? sig[i] : 0.0) + dw));
+    store(i, sum(a, a, (sig ? sig[i] : 0.0) + dw));
   }
   __syncthreads();
 }
@@ -1162,7 +1313,7 @@ k_elem_factor_rt(DevProb P, DevEval E, const double* __restrict__ sigma, double 
 // Kept out of line: inside the cooperative kernel (80 registers per thread for
 // the latency-bound register-tiled reduction blocks) its register demand would
 // otherwise shape the whole kernel.
-template <typename T, int TR, int TC>
+template <typename T, class Lay, int TR, int TC>
 __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>& F, int stride,
                                             int final_level, int bi, const BigPlace<T> pl,
                                             int pb) {
@@ -1176,29 +1327,39 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
   const T* CR = R >= 0 ? F.Cpl + (size_t)R * n * n : nullptr;
   const T* Bi = F.Bif + (size_t)i * n2 * p;
   T* A = pl.A;
-  for (int a = tid >> 5; a < bext; a += nt >> 5)
-    for (int b = tid & 31; b <= a; b += 32) {
-      T v = T(0);
-      if (a < n2) {
-        v = Ai[a * n2 + b];
-      } else if (b < n2) {
-        if (a < 3 * n) {                       // z3 of left neighbour, t = a - 2n
-          if (L >= 0 && (b & 1)) v = Ci[(b >> 1) * n + (a - n2)];
-        } else if (a < 4 * n) {                // c0 of right neighbour, s = a - 3n
-          if (R >= 0 && !(b & 1)) v = CR[(a - 3 * n) * n + (b >> 1)];
-        } else {                               // theta row q = a - 4n
-          v = Bi[b * p + (a - 4 * n)];
-        }
+  auto entry = [&](int a, int b) {
+    T v = T(0);
+    if (a < n2) {
+      v = Ai[a * n2 + b];
+    } else if (b < n2) {
+      if (a < 3 * n) {                       // z3 of left neighbour, t = a - 2n
+        if (L >= 0 && (b & 1)) v = Ci[(b >> 1) * n + (a - n2)];
+      } else if (a < 4 * n) {                // c0 of right neighbour, s = a - 3n
+        if (R >= 0 && !(b & 1)) v = CR[(a - 3 * n) * n + (b >> 1)];
+      } else {                               // theta row q = a - 4n
+        v = Bi[b * p + (a - 4 * n)];
       }
-      A[tri_at(a, b)] = v;
+    }
+    return v;
+  };
+  // a warp per row, four columns of a lane in flight
+  for (int a = tid >> 5; a < bext; a += nt >> 5)
+    for (int b0 = tid & 31; b0 <= a; b0 += 128) {
+      T v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (b0 + 32 * i <= a) v[i] = entry(a, b0 + 32 * i);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (b0 + 32 * i <= a) A[Lay::at(a, b0 + 32 * i)] = v[i];
     }
   __syncthreads();
   const int ldl = factor_ld<T>(bext);
-  pair_eliminate_big<T, TR, TC>(A, bext, n, F.Lb + (size_t)i * n2 * ldl, ldl,
+  pair_eliminate_big<T, Lay, TR, TC>(A, bext, n, F.Lb + (size_t)i * n2 * ldl, ldl,
                                 F.Db + (size_t)i * n * 3, pl.Lp, pl.W,
                                 F.inert + (size_t)(N + i) * 3, pb);
   // scatter the trailing (Schur) block into the neighbours
-  auto tr = [&](int a, int b) { return a >= b ? A[tri_at(a, b)] : A[tri_at(b, a)]; };
+  auto tr = [&](int a, int b) { return sym_at<Lay>(A, a, b); };
   if (L >= 0) {
     T* AL = F.Aif + (size_t)L * n2 * n2;
     for (int idx = tid; idx < n * n; idx += nt) {
@@ -1208,7 +1369,7 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
     T* BL = F.Bif + (size_t)L * n2 * p;
     for (int idx = tid; idx < n * p; idx += nt) {
       const int t = idx / p, q = idx - t * p;
-      BL[(2 * t) * p + q] += A[tri_at(4 * n + q, n2 + t)];
+      BL[(2 * t) * p + q] += A[Lay::at(4 * n + q, n2 + t)];
     }
   }
   if (R >= 0) {
@@ -1217,19 +1378,19 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
     for (int idx = tid; idx < n * n; idx += nt) {
       const int s2 = idx / n, s3 = idx - s2 * n;
       AR[(2 * s2 + 1) * n2 + 2 * s3 + 1] += tr(3 * n + s2, 3 * n + s3);
-      CRw[idx] = (L >= 0) ? A[tri_at(3 * n + s2, n2 + s3)] : T(0);
+      CRw[idx] = (L >= 0) ? A[Lay::at(3 * n + s2, n2 + s3)] : T(0);
     }
     T* BR = F.Bif + (size_t)R * n2 * p;
     for (int idx = tid; idx < n * p; idx += nt) {
       const int s2 = idx / p, q = idx - s2 * p;
-      BR[(2 * s2 + 1) * p + q] += A[tri_at(4 * n + q, 3 * n + s2)];
+      BR[(2 * s2 + 1) * p + q] += A[Lay::at(4 * n + q, 3 * n + s2)];
     }
   }
   double* Sc = F.Scon + (size_t)(N + i) * p * p;
-  for (int idx = tid; idx < p * p; idx += nt) {
+  for_loaded<4>(p * p, [&](int idx) {
     const int q = idx / p, q2 = idx - q * p;
-    Sc[idx] = (double)tr(4 * n + q, 4 * n + q2);
-  }
+    return tr(4 * n + q, 4 * n + q2);
+  }, [&](int idx, T v) { Sc[idx] = (double)v; });
   __syncthreads();
 }
 
@@ -1388,9 +1549,12 @@ k_bcr_factor(DevProb P, DevFactor<T> F, int stride, int final_level, int use_sme
                            ub[half].v, stage, pivs[half], cnt[half]);
   } else {
     const BigPlace<T> pl = big_place<T>(smraw, F.work, P.bext, use_smem != 0);
+    constexpr int TC = sizeof(T) == 4 ? 8 : 4;
     for (int bi = blockIdx.x; bi < nblk; bi += gridDim.x)
-      bcr_factor_big<T, 8, sizeof(T) == 4 ? 8 : 4>(P, F, stride, final_level, bi, pl,
-                                                    use_smem ? 8 : slab_pb);
+      if (use_smem)
+        bcr_factor_big<T, PackedTri, 8, TC>(P, F, stride, final_level, bi, pl, 8);
+      else
+        bcr_factor_big<T, RowBlockTri, 8, TC>(P, F, stride, final_level, bi, pl, slab_pb);
   }
 }
 
@@ -2048,8 +2212,10 @@ k_elem_factor_big_b(const DevInst* __restrict__ insts, const int* __restrict__ a
     const BigPlace<T> pl = big_place<T>(smraw, F.work, I.P.ext, full);
     // trailing tiles: 8 x 4 (FP32) or 8 x 2 (FP64) within 128 registers per thread
     constexpr int TC = sizeof(T) == 4 ? 4 : 2;
-    elem_factor_big<T, 8, TC>(I.P, I.E, I.sigma, prm[k].dw, prm[k].dc, F, t - pre_elem[k], pl,
-                              full ? 8 : slab_pb);
+    const int e = t - pre_elem[k];
+    const double dw = prm[k].dw, dc = prm[k].dc;
+    if (full) elem_factor_big<T, PackedTri, 8, TC>(I.P, I.E, I.sigma, dw, dc, F, e, pl, 8);
+    else elem_factor_big<T, RowBlockTri, 8, TC>(I.P, I.E, I.sigma, dw, dc, F, e, pl, slab_pb);
   }
 }
 
@@ -2125,12 +2291,12 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
       const DevFactor<T>& F = inst_factor<T>(I);
       const bool full = (flags[k] & 2) != 0;
       const BigPlace<T> pl = big_place<T>(smraw, F.work, I.P.bext, full);
-      const int pb = full ? 8 : slab_pb;
       // trailing tiles: warp-blocked 8 x 4 when the kernel runs one block per
       // SM (WIDE), else the 4 x 4 tiles that fit 80 registers per thread
       constexpr int TR = WIDE ? 8 : 0, TC = WIDE ? 4 : 0;
-      if (fin) bcr_factor_big<T, TR, TC>(I.P, F, 1, 1, 0, pl, pb);
-      else bcr_factor_big<T, TR, TC>(I.P, F, 1 << lv, 0, t - pre[k], pl, pb);
+      const int stride = fin ? 1 : 1 << lv, bi = fin ? 0 : t - pre[k];
+      if (full) bcr_factor_big<T, PackedTri, TR, TC>(I.P, F, stride, fin, bi, pl, 8);
+      else bcr_factor_big<T, RowBlockTri, TR, TC>(I.P, F, stride, fin, bi, pl, slab_pb);
     }
     grid_barrier(gb, ep);
   }
@@ -2313,7 +2479,7 @@ int bcr_levels(int N) {
 template <typename T>
 static size_t panel_smem(int msz, bool full) {
   const size_t panel = sizeof(T) * big_panel_elems<T>(msz);
-  if (full) return panel + sizeof(T) * big_tri_elems(msz);
+  if (full) return panel + sizeof(T) * PackedTri::elems(msz);
   return panel_in_global<T>(msz) ? 0 : panel;
 }
 template <typename T>
@@ -2554,10 +2720,12 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   const bool wide = sizeof(T) == 4 && bcr_full && 3 * (smem + 1024) > (size_t)smem_sm;
-  auto kern = wide ? (bcr_tpt == 1 ? k_factor_b<T, 1, 1>
-                      : bcr_tpt == 2 ? k_factor_b<T, 2, 1> : k_factor_b<T, 0, 1>)
-                   : (bcr_tpt == 1 ? k_factor_b<T, 1, 0>
-                      : bcr_tpt == 2 ? k_factor_b<T, 2, 0> : k_factor_b<T, 0, 0>);
+  auto kern = bcr_tpt == 1 ? k_factor_b<T, 1, 0>
+              : bcr_tpt == 2 ? k_factor_b<T, 2, 0> : k_factor_b<T, 0, 0>;
+  if constexpr (sizeof(T) == 4)
+    if (wide)
+      kern = bcr_tpt == 1 ? k_factor_b<T, 1, 1>
+             : bcr_tpt == 2 ? k_factor_b<T, 2, 1> : k_factor_b<T, 0, 1>;
   opt_in_smem(kern, smem);
   int grid = coop_grid(kern, FBS, smem, grid_cap, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
