@@ -26,6 +26,7 @@
 // T = double (plain path) or float (mixed path; residuals and refinement
 // are FP64 elsewhere).
 #include <algorithm>
+#include <climits>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -37,7 +38,6 @@
 namespace collo {
 
 constexpr int FBS = 256;   // threads per factor block
-constexpr int FTY = FBS / 32;
 
 __device__ inline void pivot_inertia(double a, double b, double d, int& pos, int& neg, int& zero) {
   const double det = fma(a, d, -(b * b));
@@ -93,6 +93,25 @@ __device__ inline void tri_tile(int t, int& ti, int& tj) {
 constexpr int PANEL_PAD = 89;
 __host__ __device__ inline int panel_ld(int msz) { return (((msz + 92) >> 3) << 3) + 4; }
 
+// The tiles of a trailing update that a warp takes: lo .. hi - 1 in turn, or, with
+// a counter in shared memory, lo and on, one after the other among the block's
+// warps (its next one is asked for before a tile is computed).
+struct TileTurns {
+  int lo, hi;
+  int* count;
+  int t, next;
+  __device__ int take() const {
+    int v = 0;
+    if ((threadIdx.x & 31) == 0) v = atomicAdd(count, 1);
+    return lo + __shfl_sync(0xffffffffu, v, 0);
+  }
+  __device__ int first() { return t = count ? take() : lo < hi ? lo : INT_MAX; }
+  __device__ void ahead() { next = count ? take() : t + 1 < hi ? t + 1 : INT_MAX; }
+  __device__ int step() { return t = next; }
+};
+__device__ inline TileTurns tiles_in_turn(int lo, int hi) { return {lo, hi, nullptr, 0, 0}; }
+__device__ inline TileTurns tiles_shared(int lo, int* count) { return {lo, 0, count, 0, 0}; }
+
 // Trailing update of pair_eliminate_packed for kernels with a small register
 // budget (the cyclic-reduction blocks inside the cooperative factorization
 // kernel when it runs three blocks per SM): 4 x 4 tiles of the packed
@@ -100,15 +119,19 @@ __host__ __device__ inline int panel_ld(int msz) { return (((msz + 92) >> 3) << 
 // sum in ascending k, subtracted once (the same arithmetic per entry as
 // trailing_update, so the result does not depend on which of the two a
 // launch uses).
+// Tiles go to the warps in chunks of 32 (lane by lane), taken by TileTurns.
 template <typename T, class Lay>
-__device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* __restrict__ Lp,
-                                       const T* __restrict__ W, int ldw) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int Tn = msz - cend;
-  if (Tn > 0) {
-    const int ntr = (Tn + 3) >> 2;
-    const int ntiles = ntr * (ntr + 1) / 2;
-    for (int t = tid; t < ntiles; t += nt) {
+__device__ __noinline__ void trailing_update_tiles4(T* A, int msz, int cend, int K,
+                                                    const T* __restrict__ Lp,
+                                                    const T* __restrict__ W, int ldw,
+                                                    TileTurns turns) {
+  const int lane = threadIdx.x & 31;
+  const int ntr = (msz - cend + 3) >> 2;
+  const int ntiles = ntr * (ntr + 1) / 2, nch = (ntiles + 31) >> 5;
+  for (int ch = turns.first(); ch < nch; ch = turns.step()) {
+    turns.ahead();
+    const int t = 32 * ch + lane;
+    if (t < ntiles) {
       int ti, tj;
       tri_tile(t, ti, tj);
       const int r0 = cend + 4 * ti, cb = cend + 4 * tj;
@@ -151,6 +174,10 @@ __device__ void trailing_update_tiles4(T* A, int msz, int cend, int K, const T* 
       }
     }
   }
+}
+// Chunks that hold the tiles of the next 2 PB rows and columns.
+__device__ inline int tiles4_head(int PB) {
+  return (PB / 2 * (PB / 2 + 1) / 2 + 31) >> 5;
 }
 
 // Two FP32 values in one 64-bit register, and the packed multiply-add on them
@@ -290,20 +317,20 @@ struct TileAcc<float, TR, TC> {
 template <typename T, int TR, int TC>
 __device__ __noinline__ void trailing_update(T* A, int msz, int cend, int K,
                                              const T* __restrict__ Lp, const T* __restrict__ W,
-                                             int ldw) {
+                                             int ldw, TileTurns turns) {
   constexpr int WR = 4 * TR, WC = 8 * TC;
   static_assert(WR <= PANEL_PAD && WC <= PANEL_PAD, "panel buffers padded for the warp tile");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int ty = lane >> 3, tx = lane & 7;
-  if (msz <= cend) return;
   const int rbase = cend & ~3;
   const int nbr = (msz - rbase + WR - 1) / WR;
-  int blk = 0;
+  int t = turns.first(), t0 = 0;
   for (int bi = 0; bi < nbr; ++bi) {
-    // blocks meeting the lower triangle
+    // tiles t0 .. t0 + nbc - 1: those of tile row bi that meet the lower triangle
     const int nbc = (min(msz, rbase + (bi + 1) * WR) - cend + WC - 1) / WC;
-    for (int bj = 0; bj < nbc; ++bj, ++blk) {
-      if (blk % nw != warp) continue;
+    for (; t - t0 < nbc; t = turns.step()) {
+      turns.ahead();
+      const int bj = t - t0;
       const int r0 = rbase + bi * WR + TR * ty, c0 = cend + bj * WC + tx;
       const T* lb = Lp + r0;
       const T* wb = W + c0;
@@ -332,7 +359,13 @@ __device__ __noinline__ void trailing_update(T* A, int msz, int cend, int K,
         }
       }
     }
+    t0 += nbc;
   }
+}
+// Tiles that hold the next 2 PB <= 4 TR rows and columns: the first tile row's.
+template <int TR, int TC>
+__device__ inline int packed_head(int msz, int cend) {
+  return (min(msz, (cend & ~3) + 4 * TR) - cend + 8 * TC - 1) / (8 * TC);
 }
 
 // Four (FP32) or two (FP64) consecutive entries at a 16-byte boundary.
@@ -342,57 +375,87 @@ struct alignas(16) Quad {
 };
 
 // The same update of a triangle in the slab (RowBlockTri), in tiles on its
-// 128-byte lines: a warp owns a block's 32 rows x 8 TC columns, lane (ty, tx) the
-// rows 8 ty .. 8 ty + 7 and TC columns in 16-byte runs, 8 lanes side by side.
+// 128-byte lines: a warp owns a block's 32 rows x 8 TC columns (FP32: 64, or 32 at
+// the end of a row block), lane (ty, tx) the rows 8 ty .. 8 ty + 7 and TC columns
+// in 16-byte runs, 8 lanes side by side.
 // Every access is 16 bytes per lane over whole lines and none is predicated:
 // entries above the diagonal, past msz or before cend (in the tiles that
 // straddle it) take part too and are never read again.
-// Bound: the shared-memory loads of the products (12 wavefronts per 32
-// multiply-adds of a lane) and, at the start of a tile, L2.  50 species, 2000
-// elements, cycles per element in all trailing updates (condensation and
-// reduction): 756 000 with the packed triangle in the slab, whose rows start
-// anywhere (4 to 8 lines per access, each predicated), 498 000 so.
+// Bound: the shared-memory loads of the products, which fill a warp's registers
+// at 128 bytes per cycle whether lanes share an address or not: 12 wavefronts
+// per 32 multiply-adds of a lane in an 8 x 4 tile, 8 in an 8 x 8 one; then L2 for
+// the tile itself.  50 species, 2000 elements, cycles per element in all trailing
+// updates (condensation and reduction): 756 000 with the packed triangle in the
+// slab, whose rows start anywhere (4 to 8 lines per access, each predicated),
+// 583 000 in 8 x 4 tiles on whole lines, 440 000 in 8 x 8 ones (both beside the
+// next diagonal block, below).  FP64 keeps 8 x 2 tiles: its pipe is the bound.
+template <typename T, int TC>
+__device__ inline void slab_tile(T* a, int ld, const T* lb, const T* wb, int K, int ldw) {
+  constexpr int TR = 8, Q = 16 / sizeof(T), NQ = TC / Q;
+  // rows whose entries are loaded before the products (the rest after them, in
+  // the registers of the operands): what the kernels' 128 registers hold
+  constexpr int AHEAD = NQ == 1 ? TR : 0, PART = NQ == 1 ? TR : TR / 2;
+  Quad<T> cur[PART][NQ];
+  auto load = [&](int u0) {
+#pragma unroll
+    for (int u = 0; u < PART; ++u)
+#pragma unroll
+      for (int g = 0; g < NQ; ++g)
+        cur[u][g] = *reinterpret_cast<const Quad<T>*>(a + (u0 + u) * ld + 8 * Q * g);
+  };
+  if (AHEAD) load(0);
+  TileAcc<T, TR, TC> acc;
+  acc.clear();
+#pragma unroll 2
+  for (int k = 0; k < K; ++k) acc.add_runs(lb + k * ldw, wb + k * ldw);
+#pragma unroll
+  for (int u0 = 0; u0 < TR; u0 += PART) {
+    if (!AHEAD) load(u0);
+#pragma unroll
+    for (int u = 0; u < PART; ++u)
+#pragma unroll
+      for (int g = 0; g < NQ; ++g) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) cur[u][g].v[i] -= acc.get(u0 + u, Q * g + i);
+        *reinterpret_cast<Quad<T>*>(a + (u0 + u) * ld + 8 * Q * g) = cur[u][g];
+      }
+  }
+}
 template <typename T, int TC>
 __device__ __noinline__ void trailing_update_slab(T* A, int msz, int cend, int K,
                                                   const T* __restrict__ Lp,
-                                                  const T* __restrict__ W, int ldw) {
-  constexpr int TR = 8, Q = 16 / sizeof(T), WC = 8 * TC;
-  static_assert(WC <= 32 && 32 + WC <= PANEL_PAD, "tiles inside the row blocks and panel buffers");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+                                                  const T* __restrict__ W, int ldw,
+                                                  TileTurns turns) {
+  constexpr int Q = 16 / sizeof(T), WC = 8 * TC, HC = 8 * Q;   // HC: columns of a narrow tile
+  static_assert(32 <= PANEL_PAD, "tiles inside the panel buffers");
+  const int lane = threadIdx.x & 31;
   const int ty = lane >> 3, tx = lane & 7;
   if (msz <= cend) return;
-  const int nb = (msz + 31) >> 5, cb = cend & ~(WC - 1);
-  int blk = warp;
+  const int nb = (msz + 31) >> 5, cb = cend & ~(HC - 1);
+  int t = turns.first(), t0 = 0;
   for (int b = cend >> 5; b < nb; ++b) {
-    const int ld = 32 * (b + 1), nbc = (ld - cb) / WC;
-    for (; blk < nbc; blk += nw) {
-      const int c0 = cb + blk * WC + Q * tx;
-      T* a = A + 512 * b * (b + 1) + TR * ty * ld + c0;
-      const T* lb = Lp + 32 * b + TR * ty;
-      const T* wb = W + c0;
-      // the tile's entries are loaded first, so that their latency overlaps the
-      // products
-      Quad<T> cur[TR][TC / Q];
-#pragma unroll
-      for (int u = 0; u < TR; ++u)
-#pragma unroll
-        for (int g = 0; g < TC / Q; ++g)
-          cur[u][g] = *reinterpret_cast<const Quad<T>*>(a + u * ld + 8 * Q * g);
-      TileAcc<T, TR, TC> acc;
-      acc.clear();
-#pragma unroll 2
-      for (int k = 0; k < K; ++k) acc.add_runs(lb + k * ldw, wb + k * ldw);
-#pragma unroll
-      for (int u = 0; u < TR; ++u)
-#pragma unroll
-        for (int g = 0; g < TC / Q; ++g) {
-#pragma unroll
-          for (int i = 0; i < Q; ++i) cur[u][g].v[i] -= acc.get(u, Q * g + i);
-          *reinterpret_cast<Quad<T>*>(a + u * ld + 8 * Q * g) = cur[u][g];
-        }
+    // tiles t0 .. t0 + nbc - 1: those of row block b
+    const int ld = 32 * (b + 1), nbc = (ld - cb + WC - 1) / WC;
+    for (; t - t0 < nbc; t = turns.step()) {
+      turns.ahead();
+      const int c0 = cb + (t - t0) * WC;
+      T* a = A + 512 * b * (b + 1) + 8 * ty * ld + c0 + Q * tx;
+      const T* lb = Lp + 32 * b + 8 * ty;
+      const T* wb = W + c0 + Q * tx;
+      if (TC > Q && c0 + HC < ld) slab_tile<T, TC>(a, ld, lb, wb, K, ldw);
+      else slab_tile<T, Q>(a, ld, lb, wb, K, ldw);
     }
-    blk -= nbc;
+    t0 += nbc;
   }
+}
+// columns per lane
+template <typename T>
+constexpr int SLAB_TC = sizeof(T) == 4 ? 8 : 2;
+// Tiles that hold the next panel's diagonal block: those of the first row block
+// (panels start at a multiple of 2 PB, so the block lies in it).
+template <typename T, int TC>
+__device__ inline int slab_head(int cend) {
+  return (32 * ((cend >> 5) + 1) - (cend & ~(8 * 16 / (int)sizeof(T) - 1)) + 8 * TC - 1) / (8 * TC);
 }
 
 // One pair's update of a row's remaining panel columns: x[j] -= l0 U0[j] +
@@ -428,92 +491,244 @@ __device__ inline void pivot_inverse(T a, T b, T d, T& ia, T& ib, T& id) {
   }
 }
 
-// The panel's diagonal block (rows and columns cp .. cp + K - 1, in W) by one
-// warp: lane r holds row cp + r in registers; a pair's two columns, final once
-// the earlier pairs are applied, go back to W, from where every lane reads them
-// and the pivot.  L columns of these rows to Lout, pivots to piv (shared).
-// Bound: the chain of pivots (a shared-memory round trip and a reciprocal per
-// pair).
-template <typename T, int PB>
-__device__ __noinline__ void panel_diag(T* W, int ldw, int cp, int K, T* __restrict__ Lout,
-                                        int lds, T (*piv)[3]) {
-  const int lane = threadIdx.x & 31;
-  T* Wr = W + cp + lane;
-  T x[2 * PB];
+// Entries cp .. cp + K - 1 of row r of the triangle (K even, the rest zero or
+// unused).
+template <class Lay, int N, typename T>
+__device__ inline void load_row(const T* A, int r, int cp, int K, T (&x)[N]) {
+  const T* row = A + Lay::at(r, cp);
+  if constexpr (std::is_same<Lay, RowBlockTri>::value) {
+    constexpr int Q = 16 / sizeof(T);
 #pragma unroll
-  for (int j = 0; j < 2 * PB; ++j) x[j] = (j <= lane && lane < K) ? Wr[j * ldw] : T(0);
+    for (int g = 0; g < N / Q; ++g) {
+      Quad<T> q{};
+      if (Q * g < K) q = reinterpret_cast<const Quad<T>*>(row)[g];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) x[Q * g + i] = q.v[i];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; ++j) x[j] = j < K ? row[j] : T(0);
+  }
+}
+
+// Two passes eliminate a panel's pairs.  panel_diag: the panel's own rows (rows
+// and columns cp .. cp + K - 1) by one warp, lane r holding row cp + r in
+// registers; a pair's two columns, final once the earlier pairs are applied, go
+// to ud (entry (r, c) at ud[c LU + r]), from where every lane reads them; L
+// columns of these rows to Lout, pivots to piv.  panel_rows: the rows below
+// (cp + K .. msz - 1), one thread per row, the row's panel entries in registers:
+// final unscaled entries to W, multipliers to Lp and Lout.  pinv: the pairs'
+// pivot inverses.
+// Bound: panel_diag the chain of pivots (a shuffle and a reciprocal per pair;
+// FP64: the FP64 pipe), panel_rows shared-memory loads and stores.
+template <int PB>
+constexpr int UD_LD = 2 * PB;
+// window_update reads up to PB entries past the last column
+template <int PB>
+constexpr int UD_ELEMS = 2 * PB * UD_LD<PB> + PB;
+
+template <class Lay, int PB>
+__device__ __noinline__ void panel_diag(const double* A, int cp, int K, double* ud,
+                                        double* __restrict__ Lout, int lds, double (*piv)[3]) {
+  constexpr int LU = UD_LD<PB>;
+  const int lane = threadIdx.x & 31;
+  double x[2 * PB];
+  load_row<Lay>(A, cp + (lane < K ? lane : 0), cp, K, x);
 #pragma unroll
   for (int kk = 0; kk < 2 * PB; kk += 2) {
     if (kk >= K) break;
+    double* U0 = ud + kk * LU;
+    double* U1 = U0 + LU;
     if (lane >= kk && lane < K) {
-      Wr[kk * ldw] = x[kk];
-      Wr[(kk + 1) * ldw] = x[kk + 1];
+      U0[lane] = x[kk];
+      U1[lane] = x[kk + 1];
     }
     __syncwarp();
-    const T* U0 = W + kk * ldw + cp;
-    const T* U1 = U0 + ldw;
-    const T a = U0[kk], b = U0[kk + 1], d = U1[kk + 1];
-    T ia, ib, id;
+    const double a = U0[kk], b = U0[kk + 1], d = U1[kk + 1];
+    double ia, ib, id;
     pivot_inverse(a, b, d, ia, ib, id);
     if (lane == 0) {
       piv[kk >> 1][0] = a; piv[kk >> 1][1] = b; piv[kk >> 1][2] = d;
     }
-    const T l0 = fma(x[kk], ia, x[kk + 1] * ib);
-    const T l1 = fma(x[kk], ib, x[kk + 1] * id);
+    const double l0 = fma(x[kk], ia, x[kk + 1] * ib);
+    const double l1 = fma(x[kk], ib, x[kk + 1] * id);
     if (lane > kk + 1 && lane < K) {
       Lout[(size_t)(cp + kk) * lds + cp + lane] = l0;
       Lout[(size_t)(cp + kk + 1) * lds + cp + lane] = l1;
     }
-    pair_row_update<T, PB>(x, kk, U0, U1, l0, l1);
+    pair_row_update<double, PB>(x, kk, U0, U1, l0, l1);
   }
 }
 
-// The panel's eliminations on the rows below it (cp + K .. msz - 1), one thread
-// per row, the row's panel entries in registers: final unscaled entries back to
-// W, multipliers to Lp and Lout.  pinv: the pairs' pivot inverses.
-template <typename T, int PB>
-__device__ __noinline__ void panel_rows(T* W, T* Lp, int ldw, int msz, int cp, int K,
-                                        T* __restrict__ Lout, int lds, const T (*pinv)[3]) {
+template <class Lay, int PB>
+__device__ __noinline__ void panel_rows(const double* A, double* W, double* Lp, int ldw, int msz,
+                                        int cp, int K, const double* ud,
+                                        double* __restrict__ Lout, int lds,
+                                        const double (*pinv)[3]) {
+  constexpr int LU = UD_LD<PB>;
   for (int r = cp + K + threadIdx.x; r < msz; r += blockDim.x) {
-    T x[2 * PB];
-#pragma unroll
-    for (int j = 0; j < 2 * PB; ++j) x[j] = j < K ? W[j * ldw + r] : T(0);
-    T* lo = Lout + (size_t)cp * lds + r;
+    double x[2 * PB];
+    load_row<Lay>(A, r, cp, K, x);
+    double* lo = Lout + (size_t)cp * lds + r;
 #pragma unroll
     for (int kk = 0; kk < 2 * PB; kk += 2) {
       if (kk >= K) break;
-      const T ia = pinv[kk >> 1][0], ib = pinv[kk >> 1][1], id = pinv[kk >> 1][2];
-      const T l0 = fma(x[kk], ia, x[kk + 1] * ib);
-      const T l1 = fma(x[kk], ib, x[kk + 1] * id);
-      if (kk > 0) {
-        W[kk * ldw + r] = x[kk];
-        W[(kk + 1) * ldw + r] = x[kk + 1];
-      }
+      const double ia = pinv[kk >> 1][0], ib = pinv[kk >> 1][1], id = pinv[kk >> 1][2];
+      const double l0 = fma(x[kk], ia, x[kk + 1] * ib);
+      const double l1 = fma(x[kk], ib, x[kk + 1] * id);
+      W[kk * ldw + r] = x[kk];
+      W[(kk + 1) * ldw + r] = x[kk + 1];
       Lp[kk * ldw + r] = l0;
       Lp[(kk + 1) * ldw + r] = l1;
       lo[(size_t)kk * lds] = l0;
       lo[(size_t)(kk + 1) * lds] = l1;
-      pair_row_update<T, PB>(x, kk, W + kk * ldw + cp, W + (kk + 1) * ldw + cp, l0, l1);
+      pair_row_update<double, PB>(x, kk, ud + kk * LU, ud + (kk + 1) * LU, l0, l1);
     }
   }
 }
 
+// FP32: a window of the row moves along it, x[i] holding the row's entries of
+// columns kk + 2i and kk + 2i + 1 (kk: the current pair's first column), so that
+// the multiply-adds go in packed pairs and one loop body serves two pairs:
+// panels of 16 pairs run a window of 16 over the first half and one of 8 over the
+// rest; panels of 8 are unrolled (the loop's idle entries cost more than its
+// shorter code gains).  Entries past the panel are computed from whatever lies
+// there and not used.
+
+// The pairs from column k0 on, at most PB / 2 of them and none from k1 on:
+// publish(kk, x0, x1) the pair's columns of this row, multipliers(kk, x0, x1,
+// l0, l1), then the update of the window's later entries from the pair's columns
+// at the panel's own rows (in ud; loaded between the two, so that the loads
+// overlap the multipliers' chain).
+template <int PB, int NW, class Publish, class Multipliers>
+__device__ inline void window_pairs(unsigned long long (&w)[NW], int k0, int k1, int K,
+                                    const float* ud, Publish publish, Multipliers multipliers) {
+  constexpr int LU = UD_LD<PB>;
+  // G: the window's packed entries that are done
+  auto one = [&](int kk, const float* U0, auto G) {
+    constexpr int g0 = decltype(G)::value;
+    float x0, x1, l0, l1;
+    unpack2(w[g0 - 1], x0, x1);
+    publish(kk, x0, x1);
+    ulonglong2 u0[NW / 2], u1[NW / 2];
+#pragma unroll
+    for (int g = g0 / 2; g < NW / 2; ++g) {
+      u0[g] = reinterpret_cast<const ulonglong2*>(U0)[g];
+      u1[g] = reinterpret_cast<const ulonglong2*>(U0 + LU)[g];
+    }
+    multipliers(kk, x0, x1, l0, l1);
+    const unsigned long long m0 = pack2(-l0, -l0), m1 = pack2(-l1, -l1);
+#pragma unroll
+    for (int g = g0 / 2; g < NW / 2; ++g) {
+      if (2 * g >= g0) w[2 * g] = fma2(m1, u1[g].x, fma2(m0, u0[g].x, w[2 * g]));
+      w[2 * g + 1] = fma2(m1, u1[g].y, fma2(m0, u0[g].y, w[2 * g + 1]));
+    }
+  };
+#pragma unroll(PB == 8 ? PB / 4 : 1)
+  for (int i = 0; i < PB / 4; ++i) {
+    const int kk = k0 + 4 * i;
+    if (kk >= k1) break;
+    const float* U = ud + kk * LU + kk;   // 16-byte aligned
+    one(kk, U, std::integral_constant<int, 1>());
+    if (kk + 2 < K) one(kk + 2, U + 2 * LU, std::integral_constant<int, 2>());
+#pragma unroll
+    for (int j = 0; j < NW; ++j) w[j] = j + 2 < NW ? w[j + 2] : 0ull;   // two pairs on
+  }
+}
+// All pairs of a panel on the row x.
+template <int PB, class Publish, class Multipliers>
+__device__ inline void panel_window(const float (&x)[2 * PB], int K, const float* ud,
+                                    Publish publish, Multipliers multipliers) {
+  unsigned long long w[PB], y[PB / 2];
+#pragma unroll
+  for (int i = 0; i < PB; ++i) w[i] = pack2(x[2 * i], x[2 * i + 1]);
+  window_pairs<PB>(w, 0, min(K, PB), K, ud, publish, multipliers);
+#pragma unroll
+  for (int i = 0; i < PB / 2; ++i) y[i] = w[i];
+  window_pairs<PB>(y, PB, K, K, ud, publish, multipliers);
+}
+
+template <class Lay, int PB>
+__device__ __noinline__ void panel_diag(const float* A, int cp, int K, float* ud,
+                                        float* __restrict__ Lout, int lds, float (*piv)[3]) {
+  constexpr int LU = UD_LD<PB>;
+  const int lane = threadIdx.x & 31;
+  float x[2 * PB];
+  load_row<Lay>(A, cp + (lane < K ? lane : 0), cp, K, x);
+  auto publish = [&](int kk, float x0, float x1) {
+    if (lane >= kk && lane < K) {
+      ud[kk * LU + lane] = x0;
+      ud[(kk + 1) * LU + lane] = x1;
+    }
+    __syncwarp();
+  };
+  panel_window<PB>(x, K, ud, publish, [&](int kk, float x0, float x1, float& l0, float& l1) {
+    const float a = __shfl_sync(0xffffffffu, x0, kk);
+    const float b = __shfl_sync(0xffffffffu, x0, kk + 1);
+    const float d = __shfl_sync(0xffffffffu, x1, kk + 1);
+    float ia, ib, id;
+    pivot_inverse(a, b, d, ia, ib, id);
+    if (lane == 0) {
+      piv[kk >> 1][0] = a; piv[kk >> 1][1] = b; piv[kk >> 1][2] = d;
+    }
+    l0 = fma(x0, ia, x1 * ib);
+    l1 = fma(x0, ib, x1 * id);
+    if (lane > kk + 1 && lane < K) {
+      Lout[(size_t)(cp + kk) * lds + cp + lane] = l0;
+      Lout[(size_t)(cp + kk + 1) * lds + cp + lane] = l1;
+    }
+  });
+}
+
+template <class Lay, int PB>
+__device__ __noinline__ void panel_rows(const float* A, float* W, float* Lp, int ldw, int msz,
+                                        int cp, int K, const float* ud,
+                                        float* __restrict__ Lout, int lds,
+                                        const float (*pinv)[3]) {
+  for (int r = cp + K + threadIdx.x; r < msz; r += blockDim.x) {
+    float x[2 * PB];
+    load_row<Lay>(A, r, cp, K, x);
+    float* lo = Lout + (size_t)cp * lds + r;
+    auto publish = [&](int kk, float x0, float x1) {
+      W[kk * ldw + r] = x0;
+      W[(kk + 1) * ldw + r] = x1;
+    };
+    panel_window<PB>(x, K, ud, publish, [&](int kk, float x0, float x1, float& l0, float& l1) {
+      const float ia = pinv[kk >> 1][0], ib = pinv[kk >> 1][1], id = pinv[kk >> 1][2];
+      l0 = fma(x0, ia, x1 * ib);
+      l1 = fma(x0, ib, x1 * id);
+      Lp[kk * ldw + r] = l0;
+      Lp[(kk + 1) * ldw + r] = l1;
+      lo[(size_t)kk * lds] = l0;
+      lo[(size_t)(kk + 1) * lds] = l1;
+    });
+  }
+}
+
+// The panel's own columns between the two passes, one buffer per CUDA block.
+template <typename T>
+__device__ inline T* ud_buffer() {
+  __shared__ __align__(16) T ud[UD_ELEMS<16>];
+  return ud;
+}
+
 // Eliminate the first npairs (state, multiplier) pairs of the symmetric msz x
-// msz matrix A, stored as a packed lower triangle (shared or global memory),
-// blocked right-looking: pairs are taken in panels of PB.  A panel's 2 PB
-// columns (rows >= the panel) are copied into W[j][r] (leading dimension
-// ldw = panel_ld(msz)), those of the panel's own rows by warp 0, which
-// eliminates the panel's pairs on them (panel_diag) while the other warps copy
-// the rows below; then every thread replays the same eliminations on its rows
+// msz matrix A, stored as a lower triangle (layout Lay), blocked right-looking:
+// pairs are taken in panels of PB.  Warp 0 eliminates the pairs on the panel's
+// own rows (panel_diag); every thread replays the same eliminations on its rows
 // below (panel_rows; a row's multipliers depend only on the diagonal block);
-// then the trailing matrix receives one rank-2PB update, in register tiles of
-// TR x TC (4 x 4 per thread at a time for TR = 0),
-// from the multipliers Lp[j][r] and the unscaled columns W.  Every entry sees the arithmetic, in the order, of the
-// pair-by-pair elimination: the pivot inverse ia = d / det, ib = -b / det,
-// id = a / det; multipliers l0 = x0 ia + x1 ib, l1 = x0 ib + x1 id; the
-// panel's remaining columns updated pair by pair; trailing entries by the sum
-// over the panel's 2 PB columns in ascending order, subtracted once
-// (trailing_update for TR x TC > 0, trailing_update_tiles4 for TR = 0).
+// then the trailing matrix receives one rank-2PB update from the multipliers
+// Lp[j][r] and the unscaled columns W[j][r] (leading dimension ldw =
+// panel_ld(msz)), in register tiles of TR x TC (4 x 4 per thread at a time for
+// TR = 0).  The next panel's diagonal block only needs the trailing tiles it
+// lies in: warp 0 takes those first and runs panel_diag for it while the other
+// warps go on with the rest (in sequence, this phase was 170 000 of the 1.05
+// million cycles of an element at 50 species, 81 000 of 402 000 at 27).
+// Every entry sees the arithmetic, in the order, of the pair-by-pair
+// elimination: the pivot inverse ia = d / det, ib = -b / det, id = a / det;
+// multipliers l0 = x0 ia + x1 ib, l1 = x0 ib + x1 id; the panel's remaining
+// columns updated pair by pair; trailing entries by the sum over the panel's
+// 2 PB columns in ascending order, subtracted once.
 // L columns go to Lout[c * lds + r] (rows r > pair), pivots (a, b, d) to
 // Dout[3 q]; inert[0..2] receives the pivots' inertia (counted off the
 // elimination's path, by the last warp: its FP64 sign tests are slow).  The
@@ -528,57 +743,53 @@ __device__ void pair_eliminate_packed(T* A, int msz, int npairs, T* __restrict__
   const int tid = threadIdx.x, nt = blockDim.x, ldw = panel_ld(msz);
   const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   __shared__ T piv[PB][3], pinv[PB][3];   // pivots and their inverses of the panel's pairs
+  __shared__ int turn;                    // trailing tiles taken so far
+  T* ud = ud_buffer<T>();
   int pos = 0, neg = 0, zero = 0;
+  auto diag = [&](int q0) {
+    const int K = 2 * (min(q0 + PB, npairs) - q0);
+    panel_diag<Lay, PB>(A, 2 * q0, K, ud, Lout, lds, piv);
+    __syncwarp();
+    if (lane < K / 2) {
+      pivot_inverse(piv[lane][0], piv[lane][1], piv[lane][2], pinv[lane][0], pinv[lane][1],
+                    pinv[lane][2]);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Dout[3 * (q0 + lane) + i] = piv[lane][i];
+    }
+  };
+  if (warp == 0) diag(0);
+  __syncthreads();
   for (int q0 = 0; q0 < npairs; q0 += PB) {
     const int pe = min(q0 + PB, npairs);
     const int cp = 2 * q0, cend = 2 * pe, K = cend - cp;
-    // panel columns cp .. cend-1 (the lower triangle; the entries above the
-    // diagonal are never used), 32 / (2 PB) rows per warp at a time
-    constexpr int RW = 32 / (2 * PB);
-    const int j = lane % (2 * PB), sub = lane / (2 * PB);
-    auto copy_rows = [&](int lo, int hi, int first, int step) {
-      constexpr int B = 8;   // loads in flight per lane
-      for (int r = lo + first * RW + sub; r < hi; r += B * step * RW) {
-        T v[B];
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-          const int ri = r + i * step * RW;
-          v[i] = (j < K && ri < hi && cp + j <= ri) ? A[Lay::at(ri, cp + j)] : T(0);
-        }
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-          const int ri = r + i * step * RW;
-          if (j < K && ri < hi && cp + j <= ri) W[j * ldw + ri] = v[i];
-        }
-      }
-    };
-    if (warp == 0) {
-      copy_rows(cp, cend, 0, 1);
-      __syncwarp();
-      panel_diag<T, PB>(W, ldw, cp, K, Lout, lds, piv);
-      __syncwarp();
-      if (lane < K / 2) {
-        pivot_inverse(piv[lane][0], piv[lane][1], piv[lane][2], pinv[lane][0], pinv[lane][1],
-                      pinv[lane][2]);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) Dout[3 * (q0 + lane) + i] = piv[lane][i];
-      }
-    } else {
-      copy_rows(cend, msz, warp - 1, nw - 1);
-    }
-    __syncthreads();
-    panel_rows<T, PB>(W, Lp, ldw, msz, cp, K, Lout, lds, pinv);
+    panel_rows<Lay, PB>(A, W, Lp, ldw, msz, cp, K, ud, Lout, lds, pinv);
+    if (tid == 0) turn = 0;
     if (warp == nw - 1 && lane < K / 2)
       pivot_inertia((double)piv[lane][0], (double)piv[lane][1], (double)piv[lane][2], pos, neg,
                     zero);
     __syncthreads();
     // trailing rank-K update of rows / columns >= cend (lower part)
-    if constexpr (TR == 0)
-      trailing_update_tiles4<T, Lay>(A, msz, cend, K, Lp, W, ldw);
-    else if constexpr (std::is_same<Lay, RowBlockTri>::value)
-      trailing_update_slab<T, 16 / sizeof(T)>(A, msz, cend, K, Lp, W, ldw);
-    else
-      trailing_update<T, TR, TC>(A, msz, cend, K, Lp, W, ldw);
+    auto trailing = [&](TileTurns turns) {
+      if constexpr (TR == 0)
+        trailing_update_tiles4<T, Lay>(A, msz, cend, K, Lp, W, ldw, turns);
+      else if constexpr (std::is_same<Lay, RowBlockTri>::value)
+        trailing_update_slab<T, SLAB_TC<T>>(A, msz, cend, K, Lp, W, ldw, turns);
+      else
+        trailing_update<T, TR, TC>(A, msz, cend, K, Lp, W, ldw, turns);
+    };
+    int head = 0;
+    if (pe < npairs) {
+      if constexpr (TR == 0) head = tiles4_head(PB);
+      else if constexpr (std::is_same<Lay, RowBlockTri>::value)
+        head = slab_head<T, SLAB_TC<T>>(cend);
+      else head = packed_head<TR, TC>(msz, cend);
+      if (warp == 0) {
+        trailing(tiles_in_turn(0, head));
+        __syncwarp();
+        diag(pe);
+      }
+    }
+    trailing(tiles_shared(head, &turn));
     __syncthreads();
   }
   if (warp == nw - 1) {
@@ -705,25 +916,40 @@ __device__ void elem_factor_big(const DevProb& P, const DevEval& E,
   const int n2 = 2 * n;
   auto tr = [&](int a, int b) { return sym_at<Lay>(A, a, b); };
   double* Sc = F.Scon + (size_t)e * p * p;
-  for_loaded<4>(p * p, [&](int idx) {
+  for (int idx = tid; idx < p * p; idx += nt) {
     const int q = idx / p, q2 = idx - q * p;
-    return tr(m + q, m + q2);
-  }, [&](int idx, T v) { Sc[idx] = (double)v; });
+    Sc[idx] = (double)tr(m + q, m + q2);
+  }
   if (P.gauss) {
     gauss_chain_out<T>(P, F, e, i0, dc, tr);
     __syncthreads();
     return;
   }
   T* Aif = F.Aif + (size_t)e * n2 * n2;
-  for_loaded<4>(n2 * n2, [&](int idx) {
+  for (int idx = tid; idx < n2 * n2; idx += nt) {
     const int u = idx / n2, v = idx - u * n2;
-    return tr(i0 + u, i0 + v);
-  }, [&](int idx, T v) { Aif[idx] = v; });
+    Aif[idx] = tr(i0 + u, i0 + v);
+  }
   T* Bif = F.Bif + (size_t)e * n2 * p;
-  for_loaded<4>(n2 * p, [&](int idx) {
-    const int u = idx / p, q = idx - u * p;
-    return A[Lay::at(m + q, i0 + u)];
-  }, [&](int idx, T v) { Bif[idx] = v; });
+  if constexpr (std::is_same<Lay, RowBlockTri>::value) {
+    // four rows q of a column per thread, so that the slab's rows are read along
+    // their lines
+    for (int idx = tid; idx < n2 * ((p + 3) >> 2); idx += nt) {
+      const int q4 = idx / n2, u = idx - q4 * n2;
+      T v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (4 * q4 + i < p) v[i] = A[Lay::at(m + 4 * q4 + i, i0 + u)];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (4 * q4 + i < p) Bif[u * p + 4 * q4 + i] = v[i];
+    }
+  } else {
+    for (int idx = tid; idx < n2 * p; idx += nt) {
+      const int u = idx / p, q = idx - u * p;
+      Bif[idx] = A[Lay::at(m + q, i0 + u)];
+    }
+  }
   T* C = F.Cpl + (size_t)e * n * n;
   for (int idx = tid; idx < n * n; idx += nt) {
     const int s2 = idx / n, t = idx - s2 * n;
@@ -1039,14 +1265,15 @@ __device__ inline int quot(int i, int d, float inv) {
 // constraint k (groups of grp_point / grp_con): Radau (z1,c1), (z2,c2),
 // (z0,c3), (z3,c0); Gauss (z1,c1) .. (z4,c4), (z0, c0 of the next element),
 // whose multiplier is k = 0 here
-__device__ inline int loc_state(const DevProb& P, int j, int s) {
-  const int K = P.K;
-  const int g = j == 0 ? (P.gauss ? K : K - 1) : ((!P.gauss && j == K) ? K : j - 1);
-  return 2 * (g * P.n + s);
-}
-__device__ inline int loc_dual(const DevProb& P, int k, int s) {
-  return 2 * ((k == 0 ? P.K : k - 1) * P.n + s) + 1;
-}
+struct LocIndex {
+  int n, K;
+  bool gauss;
+  __device__ int state(int j, int s) const {
+    const int g = j == 0 ? (gauss ? K : K - 1) : ((!gauss && j == K) ? K : j - 1);
+    return 2 * (g * n + s);
+  }
+  __device__ int dual(int k, int s) const { return 2 * ((k == 0 ? K : k - 1) * n + s) + 1; }
+};
 
 // Element condensation (same elimination as elem_factor_big) with
 // pair_eliminate_rt over the nt threads of the block.
@@ -1099,6 +1326,9 @@ __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double*
   const int n = P.n, p = P.p, m = P.m, K = P.K, np = P.np;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nn = n * n, np_ = n * p;
+  // by value: P may be in global memory, where each store to the triangle would
+  // have its fields read again
+  const LocIndex ix{n, K, P.gauss != 0};
   auto put = [&](int a, int b, T v) { blk[a >= b ? Lay::at(a, b) : Lay::at(b, a)] = v; };
   // an entry and what is added to it
   struct Sum {
@@ -1118,35 +1348,63 @@ __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double*
   for_loaded<4>(K * nn, [&](int i) { return Wzz[i]; }, [&](int i, double v) {
     const int rs = quot(i, n, inv_n), sb = i - rs * n;   // rs = k n + sa
     const int k = quot(rs, n, inv_n), sa = rs - k * n;
-    if (sa >= sb) put(loc_state(P, k + 1, sa), loc_state(P, k + 1, sb), (T)v);
+    if (sa >= sb) put(ix.state(k + 1, sa), ix.state(k + 1, sb), (T)v);
   });
   for (int i = tid; i < K * np * n; i += nt) {
     const int kj = quot(i, n, inv_n), s2 = i - kj * n;
     const int k1 = quot(kj, np, inv_np), j = kj - k1 * np;
-    put(loc_dual(P, k1 + 1, s2), loc_state(P, j, s2), (T)P.D[k1 + 1][j]);
+    put(ix.dual(k1 + 1, s2), ix.state(j, s2), (T)P.D[k1 + 1][j]);
   }
   if (!P.gauss) {
     // the element's own continuity / initial row c0 on z0
-    for (int s2 = tid; s2 < n; s2 += nt) put(loc_dual(P, 0, s2), loc_state(P, 0, s2), T(1));
+    for (int s2 = tid; s2 < n; s2 += nt) put(ix.dual(0, s2), ix.state(0, s2), T(1));
   } else if (chain_next(P, e)) {
     // the next element's continuity row: -b_j on every point of this element
     for (int i = tid; i < np * n; i += nt) {
       const int j = quot(i, n, inv_n), s2 = i - j * n;
-      put(loc_dual(P, 0, s2), loc_state(P, j, s2), (T)(-P.bw[j]));
+      put(ix.dual(0, s2), ix.state(j, s2), (T)(-P.bw[j]));
     }
   }
   for (int i = tid; i < np * n; i += nt) {
     const int k = quot(i, n, inv_n), s2 = i - k * n;
-    const int a = loc_dual(P, k, s2);
+    const int a = ix.dual(k, s2);
     put(a, a, (T)(-dc));
   }
-  for_loaded<4>(K * np_, [&](int i) { return make_double2(Wzt[i], JT[i]); },
-                [&](int i, double2 v) {
-    const int ks = quot(i, p, inv_p), q = i - ks * p;     // ks = k n + s
-    const int k = quot(ks, n, inv_n), s2 = ks - k * n;
-    put(m + q, loc_state(P, k + 1, s2), (T)v.x);
-    put(m + q, loc_dual(P, k + 1, s2), (T)v.y);
-  });
+  if constexpr (std::is_same<Lay, RowBlockTri>::value) {
+    // a warp takes 8 (point, species) x 16 parameters, four of them per lane, so
+    // that it meets few lines both in the derivatives' rows and in the slab's
+    // (50 species, cycles per element: 100 000 with a warp's lanes along either
+    // one, which then meet 32 lines in the other, 58 000 so)
+    const int Kn = K * n, nks = (Kn + 7) >> 3, nq = (p + 15) >> 4, lane = tid & 31;
+    for (int i = tid >> 5; i < nks * nq; i += nt >> 5) {
+      const int q16 = i / nks, q4 = 4 * q16 + (lane & 3);
+      const int ks = 8 * (i - q16 * nks) + (lane >> 2);   // ks = k n + s
+      if (ks >= Kn) continue;
+      const int k = quot(ks, n, inv_n), s2 = ks - k * n;
+      const int cz = ix.state(k + 1, s2), cl = ix.dual(k + 1, s2);
+      double w[4], j[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (4 * q4 + u < p) {
+          w[u] = Wzt[ks * p + 4 * q4 + u];
+          j[u] = JT[ks * p + 4 * q4 + u];
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (4 * q4 + u < p) {
+          put(m + 4 * q4 + u, cz, (T)w[u]);
+          put(m + 4 * q4 + u, cl, (T)j[u]);
+        }
+    }
+  } else {
+    for_loaded<4>(K * np_, [&](int i) { return make_double2(Wzt[i], JT[i]); },
+                  [&](int i, double2 v) {
+      const int ks = quot(i, p, inv_p), q = i - ks * p;     // ks = k n + s
+      const int k = quot(ks, n, inv_n), s2 = ks - k * n;
+      put(m + q, ix.state(k + 1, s2), (T)v.x);
+      put(m + q, ix.dual(k + 1, s2), (T)v.y);
+    });
+  }
   __syncthreads();
   // 2. sums onto those: objective blocks (same species across points) and the
   //    -h df/dz part of the collocation rows
@@ -1155,19 +1413,19 @@ __device__ __noinline__ void elem_scatter(const DevProb& P, int e, const double*
   for_loaded<4>(np2 * n, [&](int i) {
     const int s2 = quot(i, np2, inv_np2), jj = i - s2 * np2;
     const int ja = quot(jj, np, inv_np), jb = jj - ja * np;
-    const int a = loc_state(P, ja, s2), b = loc_state(P, jb, s2);
+    const int a = ix.state(ja, s2), b = ix.state(jb, s2);
     return a >= b ? sum(a, b, Wobj[i]) : Sum{nullptr, T(0), 0.0};
   }, [&](int i, const Sum& q) { if (q.at) store(i, q); });
   for_loaded<4>(K * nn, [&](int i) {
     const int rs = quot(i, n, inv_n), sp = i - rs * n;   // rs = k n + sd
     const int k = quot(rs, n, inv_n), sd = rs - k * n;
-    return sum(loc_dual(P, k + 1, sd), loc_state(P, k + 1, sp), JZ[i]);
+    return sum(ix.dual(k + 1, sd), ix.state(k + 1, sp), JZ[i]);
   }, store);
   __syncthreads();
   // 3. barrier diagonal and delta_w on the states
   for (int i = tid; i < np * n; i += nt) {
     const int j = quot(i, n, inv_n), s2 = i - j * n;
-    const int a = loc_state(P, j, s2);
+    const int a = ix.state(j, s2);
     store(i, sum(a, a, (sig ? sig[i] : 0.0) + dw));
   }
   __syncthreads();
@@ -1387,10 +1645,10 @@ __device__ __noinline__ void bcr_factor_big(const DevProb& P, const DevFactor<T>
     }
   }
   double* Sc = F.Scon + (size_t)(N + i) * p * p;
-  for_loaded<4>(p * p, [&](int idx) {
+  for (int idx = tid; idx < p * p; idx += nt) {
     const int q = idx / p, q2 = idx - q * p;
-    return tr(4 * n + q, 4 * n + q2);
-  }, [&](int idx, T v) { Sc[idx] = (double)v; });
+    Sc[idx] = (double)tr(4 * n + q, 4 * n + q2);
+  }
   __syncthreads();
 }
 
