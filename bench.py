@@ -71,9 +71,7 @@ TOL = 1e-8
 # kernel over the first 64 instances of the batch at their initial points,
 # from one ncu capture of that launch (--only-phase); None until captured or
 # once the kernel changes.
-TRAFFIC_C4_64 = {"elem_big": 6077422592 + 15532304896,
-                 "reduction_schur": 5363395072 + 4618892288,
-                 "solve": 18268539648 + 184806400}
+TRAFFIC_C4_64 = {}
 
 
 def parse_args():

@@ -591,11 +591,13 @@ typedef struct collo_schedule {
                                  blocks above 124 rows: 512 (one block per SM, the
                                  default) or 256 (two blocks per SM where their
                                  shared memory fits) */
-  int slab_pairs;             /* pairs per panel of blocks whose packed triangle is
-                                 held in the global slab: 8 or 16 (default 16) */
+  int slab_pairs;             /* pairs per panel of blocks whose triangle is held
+                                 in the global slab: 8 or 16 (default 16) */
   int solve_top_blocks;       /* the batched solve runs the reduction levels with
                                  at most this many blocks per instance in one CUDA
-                                 block per instance (default 8) */
+                                 block per instance (default 8; a block above 128
+                                 rows, which takes all eight warps, counts as
+                                 eight) */
   int solve_elems_per_block;  /* elements per 8-warp block of the solve's grid
                                  (default 8) */
   int reserved[4];
