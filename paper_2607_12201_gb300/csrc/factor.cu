@@ -2017,11 +2017,20 @@ static size_t group_smem(int msz, int groups, int most = SUB_STAGES) {
       if (bytes(st) <= cap * 1024) return bytes(st);
   return bytes(1);
 }
+// many[1]: the same for wide blocks (more than the device holds CUDA blocks, two
+// per SM), whose largest would leave an SM one CUDA block: two with one panel of
+// it each, and more panels of smaller blocks (64 problems of 5 to 50 species: 9.35
+// against 6.33 ms a solve; 50 species alone, 2000 elements: equal).
+constexpr size_t SOLVE_HALF_SM = 110 * 1024;
 template <typename T>
-size_t solve_smem(int pn, bool many, int pw, int max_p) {
+size_t solve_smem(int pn, int pw, int max_p, const bool (&many)[2]) {
   size_t b = max_p > 0 ? group_smem<double, SOLVE_G>(max_p, 1) : 0;
-  if (pn > 0) b = std::max(b, group_smem<T, 1>(pn, SOLVE_G, many ? 1 : SUB_STAGES));
-  if (pw > 0) b = std::max(b, group_smem<T, SOLVE_G>(pw, 1));
+  if (pn > 0) b = std::max(b, group_smem<T, 1>(pn, SOLVE_G, many[0] ? 1 : SUB_STAGES));
+  if (pw > 0) {
+    const size_t w = group_smem<T, SOLVE_G>(pw, 1);
+    const bool half = many[1] && group_smem<T, SOLVE_G>(pw, 1, 1) <= SOLVE_HALF_SM;
+    b = std::max(b, half ? std::min(w, SOLVE_HALF_SM) : w);
+  }
   return b;
 }
 // The part of the `bytes` of dynamic shared memory of this thread's group: all for
@@ -2900,9 +2909,10 @@ template <typename T>
 cudaError_t launch_solve(const DevProb& P, const DevFactor<T>& F, const DevSchur& S,
                          const double* b, double* sol, cudaStream_t st) {
   const bool ew = elem_solve_wide(P), bw = bcr_solve_wide(P);
-  const size_t sme = solve_smem<T>(ew ? 0 : P.ext, false, ew ? P.ext : 0, 0);
-  const size_t smb = solve_smem<T>(bw ? 0 : P.bext, false, bw ? P.bext : 0, 0);
-  const size_t smt = solve_smem<T>(0, false, 0, std::max(P.p, 1));
+  const bool few[2] = {false, false};
+  const size_t sme = solve_smem<T>(ew ? 0 : P.ext, ew ? P.ext : 0, 0, few);
+  const size_t smb = solve_smem<T>(bw ? 0 : P.bext, bw ? P.bext : 0, 0, few);
+  const size_t smt = solve_smem<T>(0, 0, std::max(P.p, 1), few);
   cudaError_t e;
   auto grid = [](bool wide, int items) { return wide ? items : ceil_div(items, SOLVE_G); };
   auto run = [&](auto kern, int g, size_t sm, auto... args) -> cudaError_t {
@@ -2997,11 +3007,11 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
 template <typename T>
 cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            const int* const elem[2], const int* const lv[2], const int* pre_lv,
-                           int maxL, int lsplit, const int* pre_cs, int ir, int pn, bool many,
-                           int pw, GridBar* gb, int max_p, int grid_want, cudaStream_t st,
+                           int maxL, int lsplit, const int* pre_cs, int ir, int pn, int pw,
+                           const bool (&many)[2], GridBar* gb, int max_p, int grid_want, cudaStream_t st,
                            int reserve) {
   if (A == 0) return cudaSuccess;
-  size_t smem = solve_smem<T>(pn, many, pw, std::max(max_p, 1));
+  size_t smem = solve_smem<T>(pn, pw, std::max(max_p, 1), many);
   opt_in_smem(k_solve_b<T>, smem);
   int grid = coop_grid(k_solve_b<T>, FBS, smem, grid_want, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
@@ -3034,10 +3044,12 @@ int elem_rt_threads(const DevProb& P, bool f32) {
 bool solve_wide(const DevProb& P, bool elem) { return elem ? elem_solve_wide(P) : bcr_solve_wide(P); }
 template cudaError_t launch_solve_b<float>(const DevInst*, const int*, int, const int* const[2],
                                            const int* const[2], const int*, int, int, const int*,
-                                           int, int, bool, int, GridBar*, int, int, cudaStream_t, int);
+                                           int, int, int, const bool (&)[2], GridBar*, int, int,
+                                           cudaStream_t, int);
 template cudaError_t launch_solve_b<double>(const DevInst*, const int*, int, const int* const[2],
                                             const int* const[2], const int*, int, int, const int*,
-                                            int, int, bool, int, GridBar*, int, int, cudaStream_t, int);
+                                            int, int, int, const bool (&)[2], GridBar*, int, int,
+                                           cudaStream_t, int);
 template size_t elem_factor_smem<float>(const DevProb&, bool);
 template size_t elem_factor_smem<double>(const DevProb&, bool);
 template size_t bcr_factor_smem<float>(const DevProb&, bool);

@@ -90,8 +90,8 @@ size_t bcr_rt_stage_bytes(const DevProb& P, bool f32);
 template <typename T>
 cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            const int* const elem[2], const int* const lv[2], const int* pre_lv,
-                           int maxL, int lsplit, const int* pre_cs, int ir, int pn, bool many,
-                           int pw, GridBar* gb, int max_p, int grid_want, cudaStream_t st,
+                           int maxL, int lsplit, const int* pre_cs, int ir, int pn, int pw,
+                           const bool (&many)[2], GridBar* gb, int max_p, int grid_want, cudaStream_t st,
                            int reserve = 0);
 // Whether P's element / reduction blocks are solved by a whole CUDA block each.
 bool solve_wide(const DevProb& P, bool elem);

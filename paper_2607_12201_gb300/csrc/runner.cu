@@ -51,7 +51,8 @@ struct Plan {
   int cap_f[2] = {1 << 30, 1 << 30};
   int solve_pw = 0;             // rows of the largest block a CUDA block solves
   int solve_pn = 0;             // ... that one warp solves
-  bool solve_many = false;      // several of those for every warp the device holds
+  bool solve_many[2] = {false, false};   // several one-warp / CUDA-block elements for each
+                                         // warp / CUDA block the device holds
   int solve_want = 0;           // CUDA blocks that hold every element at once
   int rt_threads[2] = {0, 0};   // block size of the register-tiled element kernel
   size_t rt_smem[2] = {0, 0};   // its dynamic shared memory
@@ -278,7 +279,9 @@ struct Runner {
     }
     const int per = std::max(1, schedule().solve_elems);
     pl.solve_want = std::max(A, items[1] + (items[0] + per - 1) / per);
-    pl.solve_many = items[0] > 2 * probs[slots[0]]->n_slabs * 8;   // n_slabs: two per SM
+    // n_slabs: two per SM
+    pl.solve_many[0] = items[0] > 2 * probs[slots[0]]->n_slabs * 8;
+    pl.solve_many[1] = items[1] > 2 * probs[slots[0]]->n_slabs;
     pl.off_cs_s = o; h[o] = 0;
     for (int k = 0; k < A; ++k) {
       const DevProb& Q = P(slots[k]);
@@ -476,7 +479,7 @@ struct Runner {
     const int* lv[2] = {pl.solve_lv(0), pl.solve_lv(1)};
     auto launch = prec == COLLO_PRECISION_MIXED ? launch_solve_b<float> : launch_solve_b<double>;
     e = launch(d_insts, pl.act(), pl.A, elem, lv, pl.pre_lv(), pl.maxL, pl.lsplit, pl.pre_cs_r(), ir,
-               pl.solve_pn, pl.solve_many, pl.solve_pw, gbar, pl.max_p, pl.solve_want, stream, reserve_sms);
+               pl.solve_pn, pl.solve_pw, pl.solve_many, gbar, pl.max_p, pl.solve_want, stream, reserve_sms);
     COLLO_CUDA(e);
     return COLLO_OK;
   }
