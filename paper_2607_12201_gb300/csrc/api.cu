@@ -4,6 +4,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <set>
 #include <type_traits>
 
@@ -18,6 +20,24 @@ void count_launch(int k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 Schedule& schedule() {
   static Schedule s;
   return s;
+}
+cudaError_t opt_in_smem(const void* kern, size_t bytes, bool max_carveout) {
+  if (bytes <= SMEM_OPTIN_ABOVE) return cudaSuccess;
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> done;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  size_t& cur = done[{dev, kern}];
+  if (bytes <= cur) return cudaSuccess;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && max_carveout)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) cur = bytes;
+  else cudaGetLastError();
+  return e;
 }
 
 // Collocation tables (Eq. 2b, 2c).  Points: Radau IIA for K = 3, the

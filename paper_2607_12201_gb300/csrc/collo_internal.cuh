@@ -243,6 +243,16 @@ __device__ inline int find_item(const int* __restrict__ pre, int A, int t) {
 // use 48 KB of static plus dynamic shared memory; the kernels here declare
 // at most 32 KB statically, so 16 KB of dynamic memory always fits.
 constexpr size_t SMEM_OPTIN_ABOVE = 16 * 1024;
+// That opt-in, for one device's kernel.  The limit belongs to the kernel, not to a
+// problem: problems of other sizes launch it from other threads, so it is only
+// ever raised, under a lock.  max_carveout: also ask for the largest
+// shared-memory carveout of the SM's L1 (by default the driver may pick a smaller
+// one that holds fewer of the kernel's blocks).
+cudaError_t opt_in_smem(const void* kern, size_t bytes, bool max_carveout = false);
+template <typename... Args>
+cudaError_t opt_in_smem(void (*kern)(Args...), size_t bytes, bool max_carveout = false) {
+  return opt_in_smem(reinterpret_cast<const void*>(kern), bytes, max_carveout);
+}
 // Dynamic shared memory of a factorization block above which its elimination
 // runs in a global slab instead (allocation and use both test against it).
 constexpr size_t FACTOR_SMEM_LIMIT = 200 * 1024;

@@ -475,19 +475,17 @@ cudaError_t launch_eval(const DevProb& P, const DevEval& E, const double* x, con
                         double alpha, const double* lam, double obj_factor, bool deriv,
                         cudaStream_t st) {
   size_t sm = eval_smem_bytes(P, deriv);
+  cudaError_t e;
   if (deriv) {
-    if (sm > SMEM_OPTIN_ABOVE)
-      cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if ((e = opt_in_smem(k_eval<true>, sm)) != cudaSuccess) return e;
     count_launch();
     k_eval<true><<<P.N, EVAL_BS, sm, st>>>(P, x, dx, alpha, lam, obj_factor, E);
   } else {
-    if (sm > SMEM_OPTIN_ABOVE)
-      cudaFuncSetAttribute(k_eval<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if ((e = opt_in_smem(k_eval<false>, sm)) != cudaSuccess) return e;
     count_launch();
     k_eval<false><<<P.N, EVAL_BS, sm, st>>>(P, x, dx, alpha, lam, obj_factor, E);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   count_launch();
   k_eval_reduce<<<deriv ? theta_blocks(P.p) : 1, TH_BS, 0, st>>>(P, E);
   return cudaGetLastError();
@@ -550,19 +548,17 @@ cudaError_t launch_eval_b(const DevInst* insts, const int* act, int A, const int
                           int total_elems, const InstParams* prm, int xsel, int dxsel, int lsel,
                           bool deriv, size_t smem, int max_p, cudaStream_t st) {
   if (A == 0) return cudaSuccess;
+  cudaError_t e;
   if (deriv) {
-    if (smem > SMEM_OPTIN_ABOVE)
-      cudaFuncSetAttribute(k_eval_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if ((e = opt_in_smem(k_eval_b<true>, smem)) != cudaSuccess) return e;
     count_launch();
     k_eval_b<true><<<total_elems, EVAL_BS, smem, st>>>(insts, act, A, pre_elem, prm, xsel, dxsel, lsel);
   } else {
-    if (smem > SMEM_OPTIN_ABOVE)
-      cudaFuncSetAttribute(k_eval_b<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if ((e = opt_in_smem(k_eval_b<false>, smem)) != cudaSuccess) return e;
     count_launch();
     k_eval_b<false><<<total_elems, EVAL_BS, smem, st>>>(insts, act, A, pre_elem, prm, xsel, dxsel, lsel);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   count_launch();
   k_eval_reduce_b<<<dim3(A, deriv ? theta_blocks(max_p) : 1), TH_BS, 0, st>>>(insts, act);
   return cudaGetLastError();
@@ -661,8 +657,7 @@ extern "C" collo_status collo_eval_noalloc(collo_problem* prob, const double* x,
   E.red = scratch + (size_t)P.N * (4 + (size_t)P.p);  // [8]
   cudaStream_t st = stream ? (cudaStream_t)stream : prob->stream;
   const size_t sm = eval_smem_bytes(P, true);
-  if (sm > SMEM_OPTIN_ABOVE)
-    COLLO_CUDA(cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  COLLO_CUDA(opt_in_smem(k_eval<true>, sm));
   count_launch();
   k_eval<true><<<P.N, EVAL_BS, sm, st>>>(P, x, nullptr, 0.0, lambda, obj_factor, E);
   COLLO_CUDA(cudaGetLastError());

@@ -2774,45 +2774,20 @@ size_t factor_work_elems(const DevProb& P, int n_slabs) {
   return w;
 }
 
-// cudaFuncAttributeMaxDynamicSharedMemorySize, set only when a launch needs
-// more than the kernel's setting so far (per device).
-template <typename KernelT>
-static void opt_in_smem(KernelT kern, size_t bytes) {
-  if (bytes <= SMEM_OPTIN_ABOVE) return;
-  static std::mutex mu;
-  static std::map<std::pair<int, const void*>, size_t> done;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(mu);
-  size_t& cur = done[{dev, (const void*)kern}];
-  if (bytes <= cur) return;
-  // a kernel that asks for this much shared memory also asks for the largest
-  // shared-memory carveout of the SM's L1: by default the driver may pick a
-  // smaller one that holds fewer of its blocks
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) ==
-          cudaSuccess &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared) == cudaSuccess)
-    cur = bytes;
-  else
-    cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t launch_elem_factor(const DevProb& P, const DevEval& E, const double* sigma, double dw,
                                double dc, const DevFactor<T>& F, cudaStream_t st) {
   const int rtn = rt_block_threads<T>(P.ext);
   if (rtn > 0) {
     const size_t sm = elem_stage_bytes<T>(P);
-    opt_in_smem(k_elem_factor_rt<T>, sm);
+    opt_in_smem(k_elem_factor_rt<T>, sm, true);
     count_launch();
     k_elem_factor_rt<T><<<P.N, rtn, sm, st>>>(P, E, sigma, dw, dc, F);
     return cudaGetLastError();
   }
   bool es = elem_uses_smem<T>(P);
   size_t sm = elem_factor_smem<T>(P, es);
-  if (sm > SMEM_OPTIN_ABOVE)
-    cudaFuncSetAttribute(k_elem_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  opt_in_smem(k_elem_factor<T>, sm);
   int grid = es ? P.N : std::min(P.N, F.n_slabs);
   count_launch();
   k_elem_factor<T><<<grid, FBS, sm, st>>>(P, E, sigma, dw, dc, F, es ? 1 : 0,
@@ -2874,13 +2849,10 @@ cudaError_t launch_factor(const DevProb& P, const DevEval& E, const double* sigm
     count_launch();
     if (bt == 1 || bt == 2) {
       auto kern = bt == 1 ? k_bcr_factor<T, 1> : k_bcr_factor<T, 2>;
-      if (smr > SMEM_OPTIN_ABOVE)
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
+      opt_in_smem(kern, smr);
       kern<<<(nblk + 1) / 2, FBS, smr, st>>>(P, F, s, fin, 1, schedule().slab_pairs);
     } else {
-      if (smb > SMEM_OPTIN_ABOVE)
-        cudaFuncSetAttribute(k_bcr_factor<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smb);
+      opt_in_smem(k_bcr_factor<T, 0>, smb);
       const int g = bs ? nblk : std::min(nblk, F.n_slabs);
       k_bcr_factor<T, 0><<<g, FBS, smb, st>>>(P, F, s, fin, bs ? 1 : 0, schedule().slab_pairs);
     }
@@ -2892,8 +2864,7 @@ cudaError_t launch_factor(const DevProb& P, const DevEval& E, const double* sigm
   // the Schur block works in shared memory up to the factorization limit,
   // otherwise in S.S itself
   const bool sg = sms > SMEM_LIMIT;
-  if (!sg && sms > SMEM_OPTIN_ABOVE)
-    cudaFuncSetAttribute(k_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms);
+  if (!sg) opt_in_smem(k_schur, sms);
   if ((e = launch_chunk_sums(F.Scon, 2 * P.N, P.p * P.p, F.chunkS, st)) != cudaSuccess) return e;
   if (P.p > 0) {
     count_launch();
@@ -2916,7 +2887,7 @@ cudaError_t launch_solve(const DevProb& P, const DevFactor<T>& F, const DevSchur
   cudaError_t e;
   auto grid = [](bool wide, int items) { return wide ? items : ceil_div(items, SOLVE_G); };
   auto run = [&](auto kern, int g, size_t sm, auto... args) -> cudaError_t {
-    opt_in_smem(kern, sm);
+    opt_in_smem(kern, sm, true);
     count_launch();
     kern<<<g, FBS, sm, st>>>(args..., sm);
     return cudaGetLastError();
@@ -2959,7 +2930,7 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
   if (A == 0) return cudaSuccess;
   if ((parts & 1) && rt_threads > 0 && tot_elem > 0) {
     if (rt_threads > RT_MAX_THREADS) return cudaErrorInvalidValue;
-    opt_in_smem(k_elem_factor_rt_b<T>, rt_smem);
+    opt_in_smem(k_elem_factor_rt_b<T>, rt_smem, true);
     count_launch();
     k_elem_factor_rt_b<T><<<tot_elem, rt_threads, rt_smem, st>>>(insts, act, A, pre_elem, prm,
                                                                  flags);
@@ -2970,11 +2941,11 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
   if ((parts & 4) && big_grid > 0) {
     count_launch();
     if (sch.big_threads == 256) {
-      opt_in_smem(k_elem_factor_big_b<T, 256>, big_smem);
+      opt_in_smem(k_elem_factor_big_b<T, 256>, big_smem, true);
       k_elem_factor_big_b<T, 256><<<big_grid, 256, big_smem, st>>>(insts, act, A, pre_elem, prm,
                                                                    flags, sch.slab_pairs);
     } else {
-      opt_in_smem(k_elem_factor_big_b<T, 512>, big_smem);
+      opt_in_smem(k_elem_factor_big_b<T, 512>, big_smem, true);
       k_elem_factor_big_b<T, 512><<<big_grid, 512, big_smem, st>>>(insts, act, A, pre_elem, prm,
                                                                    flags, sch.slab_pairs);
     }
@@ -2994,7 +2965,7 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
     if (wide)
       kern = bcr_tpt == 1 ? k_factor_b<T, 1, 1>
              : bcr_tpt == 2 ? k_factor_b<T, 2, 1> : k_factor_b<T, 0, 1>;
-  opt_in_smem(kern, smem);
+  opt_in_smem(kern, smem, true);
   int grid = coop_grid(kern, FBS, smem, grid_cap, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
   int slab_pb = sch.slab_pairs;
@@ -3012,7 +2983,7 @@ cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            int reserve) {
   if (A == 0) return cudaSuccess;
   size_t smem = solve_smem<T>(pn, pw, std::max(max_p, 1), many);
-  opt_in_smem(k_solve_b<T>, smem);
+  opt_in_smem(k_solve_b<T>, smem, true);
   int grid = coop_grid(k_solve_b<T>, FBS, smem, grid_want, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
   SolvePlan sp{{elem[0], elem[1]}, {lv[0], lv[1]}};

@@ -647,11 +647,6 @@ size_t elem_smem_bytes(int me) { return (tri(me) + me) * sizeof(double); }
 
 size_t bcr_smem_bytes(int n, int cw) { return ((size_t)n * n + (size_t)n * cw + n) * sizeof(double); }
 
-cudaError_t set_smem(const void* f, size_t bytes) {
-  if (bytes <= SMEM_OPTIN_ABOVE) return cudaSuccess;
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 // Storage of the lifted factorization (allocated on the first call).
@@ -779,17 +774,17 @@ cudaError_t lifted_factor_kernels(collo_problem* pr, bool elem_only) {
   const size_t sm_e = L.elem_smem ? elem_smem_bytes(L.me) : (size_t)L.me * sizeof(double);
   count_launch();
   if (L.me > 128) {
-    if ((e = set_smem((const void*)k_lifted_elem<512>, sm_e)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_lifted_elem<512>, sm_e)) != cudaSuccess) return e;
     k_lifted_elem<512><<<L.grid_e, 512, sm_e, st>>>(P, pr->E, L);
   } else {
-    if ((e = set_smem((const void*)k_lifted_elem<256>, sm_e)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_lifted_elem<256>, sm_e)) != cudaSuccess) return e;
     k_lifted_elem<256><<<L.grid_e, 256, sm_e, st>>>(P, pr->E, L);
   }
   if ((e = cudaGetLastError()) != cudaSuccess || elem_only) return e;
   count_launch();
   k_lifted_chain<<<N, LBS, 0, st>>>(P, L);
   const size_t sm_b = bcr_smem_bytes(n, L.cw);
-  if ((e = set_smem((const void*)k_lifted_bcr_elim, sm_b)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(k_lifted_bcr_elim, sm_b)) != cudaSuccess) return e;
   for (int lv = 0; (1 << lv) < N; ++lv) {
     const int h = 1 << lv, cnt = (N - h + 2 * h - 1) / (2 * h), surv = (N + 2 * h - 1) / (2 * h);
     count_launch(2);
@@ -806,7 +801,7 @@ cudaError_t lifted_factor_kernels(collo_problem* pr, bool elem_only) {
     k_lifted_theta_sum<<<tiles, LBS, 0, st>>>(P, pr->E, L);
     const size_t sm_t = ((size_t)p * p + p) * sizeof(double);
     const int in_smem = sm_t <= FACTOR_SMEM_LIMIT;
-    if ((e = set_smem((const void*)k_lifted_theta_chol, in_smem ? sm_t : 0)) != cudaSuccess)
+    if ((e = opt_in_smem(k_lifted_theta_chol, in_smem ? sm_t : 0)) != cudaSuccess)
       return e;
     count_launch();
     k_lifted_theta_chol<<<1, 1024, in_smem ? sm_t : 0, st>>>(P, L, in_smem);

@@ -156,8 +156,8 @@ static size_t defect_smem(const DevProb& P) {
 // (device); on the problem's stream.
 static cudaError_t launch_defect(collo_problem* pr, const double* x, double* def, double* mx) {
   const size_t sm = defect_smem(pr->P);
-  if (sm > SMEM_OPTIN_ABOVE)
-    cudaFuncSetAttribute(k_defect, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const cudaError_t e = opt_in_smem(k_defect, sm);
+  if (e != cudaSuccess) return e;
   count_launch(2);
   k_defect<<<pr->P.N, DEF_BS, sm, pr->stream>>>(pr->P, x, def);
   k_max<<<1, DEF_BS, 0, pr->stream>>>(def, pr->P.N, mx);

@@ -541,11 +541,8 @@ int sweep_block_threads(const DevProb& P) { return sweep_threads(P.K * P.n); }
 cudaError_t launch_sweep_b(const DevInst* insts, const int* act, int A, int threads, size_t smem,
                            cudaStream_t st) {
   if (A == 0) return cudaSuccess;
-  if (smem > SMEM_OPTIN_ABOVE) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_sweep_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = opt_in_smem(k_sweep_b, smem);
+  if (e != cudaSuccess) return e;
   count_launch();
   k_sweep_b<<<A, threads, smem, st>>>(insts, act);
   return cudaGetLastError();
