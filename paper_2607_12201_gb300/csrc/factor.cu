@@ -1878,9 +1878,10 @@ __global__ void __launch_bounds__(CS_BS) k_schur_total(double* chunkS, int N, in
   if (idx < p * p) schur_total(chunkS, N, p, idx);
 }
 
-// The same sum by four neighbouring lanes (part 0 .. 3 of a quad, the whole warp
-// calling): the four partial sums of sum_chunks, each with its loads in flight
-// at once, added in its order; every lane of the quad returns it.
+// The same sum by the four lanes of a quad (quarter 0 .. 3), which call together,
+// whatever the warp's other lanes do: the four partial sums of sum_chunks, each
+// with its loads in flight at once, added in its order; every lane of the quad
+// returns it.
 __device__ inline double sum_chunks4(const double* __restrict__ part, int G, int L, int l,
                                      int quarter) {
   const int G4 = G & ~3;
@@ -1895,9 +1896,9 @@ __device__ inline double sum_chunks4(const double* __restrict__ part, int G, int
   }
   if (quarter == 0)
     for (int g = G4; g < G; ++g) a += part[(size_t)g * L + l];
-  const unsigned m = __activemask();
-  a += __shfl_xor_sync(m, a, 1);
-  return a + __shfl_xor_sync(m, a, 2);
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  a += __shfl_xor_sync(quad, a, 1);
+  return a + __shfl_xor_sync(quad, a, 2);
 }
 
 constexpr int SBS = 256;
