@@ -1997,8 +1997,8 @@ k_schur(DevProb P, const int* __restrict__ inert, const double* __restrict__ chu
 // Blocks of at most SOLVE_NARROW rows are solved by one warp each, eight at a
 // time in a CUDA block; larger ones by the whole CUDA block (subst.cuh).  One
 // solve against one warp per block throughout, two columns loaded per step: 10
-// species, 400 elements 148 -> 128 us; 27 species, 415 elements 483 -> 206 us; 50
-// species, 2000 elements 1743 -> 969 us.
+// species, 400 elements 148 -> 133 us; 27 species, 415 elements 394 -> 166 us; 50
+// species, 2000 elements 1692 -> 671 us.
 constexpr int SOLVE_NARROW = 128;
 constexpr int SOLVE_G = FBS / 32;   // warps of a wide block's group
 __host__ __device__ inline bool elem_solve_wide(const DevProb& P) { return P.ext > SOLVE_NARROW; }
@@ -2006,33 +2006,35 @@ __host__ __device__ inline bool bcr_solve_wide(const DevProb& P) { return P.bext
 // Dynamic shared memory of a solve kernel: narrow blocks of at most pn rows, wide
 // ones of at most pw, a parameter block of max_p (each 0: none).  Three panels in
 // flight per group (two, one), if two CUDA blocks then still fit an SM; else as
-// many as one block has room for.  With many narrow blocks (several for each warp
-// the device holds) one panel: twice the warps hide the latency better than
-// the second panel does (32 problems of 10 species: 362 against 302 us a solve).
+// many as one block has room for.
+constexpr size_t SOLVE_HALF_SM = 110 * 1024;
 template <typename T, int G>
-static size_t group_smem(int msz, int groups, int most = SUB_STAGES) {
+static size_t group_smem(int msz, int groups, int most = SUB_STAGES, bool half = false) {
   const size_t v = sizeof(T) * sub_vec_elems(msz), pn = sub_slot_bytes<T, G>(msz);
   auto bytes = [&](int st) { return groups * ((v + st * pn + 15) & ~size_t(15)); };
-  for (size_t cap : {size_t(110), size_t(200)})
-    for (int st = most; st > 1; --st)
-      if (bytes(st) <= cap * 1024) return bytes(st);
+  for (size_t cap : {SOLVE_HALF_SM, size_t(200 * 1024)})
+    for (int st = most; st > 1 && !(half && cap > SOLVE_HALF_SM); --st)
+      if (bytes(st) <= cap) return bytes(st);
   return bytes(1);
 }
-// many[1]: the same for wide blocks (more than the device holds CUDA blocks, two
-// per SM), whose largest would leave an SM one CUDA block: two with one panel of
-// it each, and more panels of smaller blocks (64 problems of 5 to 50 species: 9.35
-// against 6.33 ms a solve; 50 species alone, 2000 elements: equal).
-constexpr size_t SOLVE_HALF_SM = 110 * 1024;
+// many[0], many[1]: many narrow / wide blocks (more than two for each warp / CUDA
+// block the device holds).  Then two CUDA blocks per SM hide the chains better than
+// more panels in flight, if one panel of each kind leaves room for them, and many
+// narrow blocks do with one panel each.  A solve of the first 64, 32 and 16 problems of 5
+// to 50 species (100 to 2000 elements): 7.2, 4.2 and 2.0 ms with one CUDA block per SM,
+// 4.6, 2.8 and 1.44 with two; one warp per block throughout 5.0, 3.3 and 2.1.  50
+// species alone, 2000 elements: 773 against 671 us.
 template <typename T>
 size_t solve_smem(int pn, int pw, int max_p, const bool (&many)[2]) {
-  size_t b = max_p > 0 ? group_smem<double, SOLVE_G>(max_p, 1) : 0;
-  if (pn > 0) b = std::max(b, group_smem<T, 1>(pn, SOLVE_G, many[0] ? 1 : SUB_STAGES));
-  if (pw > 0) {
-    const size_t w = group_smem<T, SOLVE_G>(pw, 1);
-    const bool half = many[1] && group_smem<T, SOLVE_G>(pw, 1, 1) <= SOLVE_HALF_SM;
-    b = std::max(b, half ? std::min(w, SOLVE_HALF_SM) : w);
-  }
-  return b;
+  auto need = [&](bool half) {
+    size_t b = max_p > 0 ? group_smem<double, SOLVE_G>(max_p, 1, SUB_STAGES, half) : 0;
+    if (pn > 0) b = std::max(b, group_smem<T, 1>(pn, SOLVE_G, many[0] ? 1 : SUB_STAGES, half));
+    if (pw > 0) b = std::max(b, group_smem<T, SOLVE_G>(pw, 1, SUB_STAGES, half));
+    return b;
+  };
+  const size_t b = many[0] || many[1] ? need(true) : 0;
+  if (b > 0 && b <= SOLVE_HALF_SM) return pw > 0 ? SOLVE_HALF_SM : b;
+  return need(false);
 }
 // The part of the `bytes` of dynamic shared memory of this thread's group: all for
 // G > 1 (blocks of up to msz rows), this warp's share for G = 1.
@@ -2159,7 +2161,7 @@ __device__ void elem_fwd_one(const DevProb& P, const DevFactor<T>& F, const doub
   const T* D = F.Del + (size_t)e * nint * 3;   // asked for before the substitution
   T d0 = T(0), d1 = T(0), d2 = T(0);
   if (tid < nint) { d0 = D[3 * tid]; d1 = D[3 * tid + 1]; d2 = D[3 * tid + 2]; }
-  sub_set(sm.ring, group_forward<G, true>(w, sm.ring, elem_cols(P, F, e)));
+  sm.ring.phases = group_forward<G, true>(w, sm.ring, elem_cols(P, F, e));
   next();
   T* V = F.Vint + (size_t)e * 2 * nint;
   for (int q = tid; q < nint; q += NT) {
@@ -2203,7 +2205,7 @@ __device__ void bcr_fwd_one(const DevProb& P, const DevFactor<T>& F, int stride,
     if (R >= 0) rr = RR[2 * tid + 1];
   }
   group_sync<G>();
-  sub_set(sm.ring, group_forward<G, true>(w, sm.ring, bcr_cols(P, F, i)));
+  sm.ring.phases = group_forward<G, true>(w, sm.ring, bcr_cols(P, F, i));
   next();
   T* V = F.Vb + (size_t)i * n2;
   for (int q = tid; q < n; q += NT) {
@@ -2238,14 +2240,14 @@ __device__ void theta_solve_block(const DevProb& P, const double* __restrict__ c
     if ((tid & 3) == 0) sv[q] = b[nz + q] + v;
   }
   __syncthreads();
-  sub_set(sm.ring, group_forward<SOLVE_G, false>(sv, sm.ring, L));
+  sm.ring.phases = group_forward<SOLVE_G, false>(sv, sm.ring, L);
   sub_start<SOLVE_G>(sm.ring, L, false);
   for (int k = tid; k < p; k += FBS) {
     const double d = S.Sd[k];
     sv[k] = (d != 0.0 && isfinite(d)) ? sv[k] / d : 0.0;
   }
   __syncthreads();
-  sub_set(sm.ring, group_backward<SOLVE_G, false>(sv, sm.sums, sm.ring, L));
+  sm.ring.phases = group_backward<SOLVE_G, false>(sv, sm.sums, sm.ring, L);
   for (int q = tid; q < p; q += FBS) { sol[nz + q] = sv[q]; S.xth[q] = sv[q]; }
   sub_release();
   __syncthreads();
@@ -2256,7 +2258,7 @@ k_theta_solve(DevProb P, const double* __restrict__ chunkR, const double* __rest
               DevSchur S, double* __restrict__ sol, int* err, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SUB_STAGES];
-  sub_init(bars, SUB_STAGES);
+  sub_init<SOLVE_G>(bars, 0, 1);
   SubMem<double, SOLVE_G> sm = sub_mem<double, SOLVE_G>(smraw, smem, P.p, bars, err);
   theta_solve_block(P, chunkR, b, S, sol, sm);
 }
@@ -2288,7 +2290,7 @@ __device__ void bcr_bwd_one(const DevProb& P, const DevFactor<T>& F, const DevSc
     x[a] = v;
   }
   group_sync<G>();
-  sub_set(sm.ring, group_backward<G, true>(x, sm.sums, sm.ring, bcr_cols(P, F, i)));
+  sm.ring.phases = group_backward<G, true>(x, sm.sums, sm.ring, bcr_cols(P, F, i));
   next();
   for (int s = tid; s < n; s += NT) {
     sol[((size_t)i * np + cpt) * n + s] = (double)x[2 * s];
@@ -2314,7 +2316,7 @@ __device__ void elem_bwd_one(const DevProb& P, const DevFactor<T>& F, const DevS
   }
   for (int a = m + tid; a < ext; a += NT) x[a] = (T)S.xth[a - m];
   group_sync<G>();
-  sub_set(sm.ring, group_backward<G, true>(x, sm.sums, sm.ring, elem_cols(P, F, e)));
+  sm.ring.phases = group_backward<G, true>(x, sm.sums, sm.ring, elem_cols(P, F, e));
   next();
   if (!P.gauss)
     for (int a = tid; a < 2 * nint; a += NT) sol[elem_global(P, e, a)] = (double)x[a];
@@ -2331,7 +2333,7 @@ k_elem_solve(DevProb P, DevFactor<T> F, DevSchur S, const double* __restrict__ b
              double* __restrict__ sol, int fwd, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SOLVE_BARS];
-  sub_init(bars, SOLVE_BARS);
+  sub_init<SOLVE_G>(bars, G > 1 ? 0 : SOLVE_G, G > 1 ? 1 : 0);
   SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.ext, bars, &F.gbar->err);
   const int e = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
   if (e >= P.N) return;
@@ -2346,7 +2348,7 @@ k_bcr_solve(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int
             int final_level, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SOLVE_BARS];
-  sub_init(bars, SOLVE_BARS);
+  sub_init<SOLVE_G>(bars, G > 1 ? 0 : SOLVE_G, G > 1 ? 1 : 0);
   SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.bext, bars, &F.gbar->err);
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
   const int bi = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
@@ -2625,7 +2627,7 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
   __shared__ unsigned long long bars[SOLVE_BARS + 2 * SUB_STAGES];
   __shared__ LoneInst lone;
   lone_load(lone, insts, act, A);
-  sub_init(bars, SOLVE_BARS + 2 * SUB_STAGES);
+  sub_init<SOLVE_G>(bars, SOLVE_G, 2);
   auto inst = [&](int k) -> const DevInst& {
     return A == 1 ? *reinterpret_cast<const DevInst*>(lone.b) : insts[act[k]];
   };

@@ -86,7 +86,8 @@ size_t elem_rt_stage_bytes(const DevProb& P, bool f32);
 size_t bcr_rt_stage_bytes(const DevProb& P, bool f32);
 // Solve work lists: elem, lv as SolvePlan (prefix arrays of the narrow [0] and
 // wide [1] instances), pre_lv all instances' blocks per level; pn, pw: rows of the
-// largest narrow / wide block (0: none); many: several narrow blocks per warp.
+// largest narrow / wide block (0: none); many: more than two narrow / wide elements
+// for each warp / CUDA block the device holds.
 template <typename T>
 cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            const int* const elem[2], const int* const lv[2], const int* pre_lv,

@@ -51,8 +51,8 @@ struct Plan {
   int cap_f[2] = {1 << 30, 1 << 30};
   int solve_pw = 0;             // rows of the largest block a CUDA block solves
   int solve_pn = 0;             // ... that one warp solves
-  bool solve_many[2] = {false, false};   // several one-warp / CUDA-block elements for each
-                                         // warp / CUDA block the device holds
+  bool solve_many[2] = {false, false};   // more than two one-warp / CUDA-block elements
+                                         // for each warp / CUDA block the device holds
   int solve_want = 0;           // CUDA blocks that hold every element at once
   int rt_threads[2] = {0, 0};   // block size of the register-tiled element kernel
   size_t rt_smem[2] = {0, 0};   // its dynamic shared memory

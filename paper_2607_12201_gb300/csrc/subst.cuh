@@ -7,6 +7,8 @@
 // to shared memory one or two panels ahead by bulk copies (one per column, a
 // transaction barrier per panel), the first panels of the group's next block
 // while the current one finishes, so the chain itself rarely waits for memory.
+// The group's shared memory is divided for the block at hand, so that a smaller
+// block than the launch's largest has more panels ahead.
 // Per panel, the group's first warp solves the diagonal
 // block, one right-hand-side entry per lane, passing each solved pair on by
 // shuffles; then every thread applies the panel to its rows below (forward), or
@@ -93,8 +95,8 @@ __host__ __device__ inline size_t sub_slot_bytes(int msz) {
 }
 
 // ---- transaction barriers and bulk copies ---------------------------------------------
-__device__ inline void mbar_init(unsigned bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+__device__ inline void mbar_init(unsigned bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ inline void mbar_expect(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
@@ -122,27 +124,20 @@ __device__ inline bool mbar_try(unsigned bar, unsigned parity) {
 // by the hardware) and records the error.
 constexpr int SUB_WAIT_TRIES = 1 << 22;
 
-// A group's ring of panels in shared memory: the slot and the barrier phase of
-// the next panel to wait for (the same on every thread of the group).  Kept in
-// registers and passed by value.
+constexpr int SUB_STAGES = 3;   // most panels in flight
+
+// A group's ring of panels in shared memory (the same on every thread of the
+// group): `bytes` of it, divided into slots by the block at hand (sub_start), as
+// many as it has room for; slot: the next panel's; phases: each barrier's
+// phase, a bit per slot.  Kept in registers and passed by value.
 struct SubRing {
   unsigned char* slots;     // [stages][slot_bytes]
-  unsigned bar;             // [stages] barriers, shared-space address
-  int slot_bytes, stages;
+  unsigned bar;             // [SUB_STAGES] barriers, shared-space address
+  int bytes, slot_bytes, stages;
   int slot;
-  unsigned phase;
+  unsigned phases;
   int* err;                 // GridBar::err
-  __device__ void advance() {
-    if (++slot == stages) { slot = 0; phase ^= 1u; }
-  }
 };
-// What a substitution changes of it.
-struct SubPos {
-  int slot;
-  unsigned phase;
-};
-
-constexpr int SUB_STAGES = 3;   // most panels in flight
 
 template <int G>
 __device__ inline void group_sync() {
@@ -172,17 +167,24 @@ __device__ inline SubMem<T, G> sub_carve(unsigned char* p, size_t bytes, int msz
   m.sums = m.w + (v - 32);
   m.ring.slots = reinterpret_cast<unsigned char*>(m.w + v);
   m.ring.bar = (unsigned)__cvta_generic_to_shared(bar);
-  m.ring.slot_bytes = (int)sub_slot_bytes<T, G>(msz);
-  m.ring.stages = (int)min((size_t)SUB_STAGES,
-                           (bytes - sizeof(T) * v) / (size_t)m.ring.slot_bytes);
-  m.ring.slot = 0;
-  m.ring.phase = 0;
+  m.ring.bytes = (int)(bytes - sizeof(T) * v);
+  m.ring.slot_bytes = m.ring.stages = m.ring.slot = 0;
+  m.ring.phases = 0;
   m.ring.err = err;
   return m;
 }
-// Initialises n barriers (the whole block calls).
-__device__ inline void sub_init(unsigned long long* bar, int n) {
-  if ((int)threadIdx.x < n) mbar_init((unsigned)__cvta_generic_to_shared(bar + threadIdx.x));
+// Warps of a group that ask for panels (a barrier's arrivals): all but the one that
+// carries the chain, where there are others.
+template <int G>
+constexpr int SUB_ASKING = G > 1 ? G - 1 : 1;
+// Initialises the barriers of n1 groups of one warp and, behind them, nG groups of G
+// (the whole block calls).
+template <int G>
+__device__ inline void sub_init(unsigned long long* bar, int n1, int nG) {
+  const int t = threadIdx.x;
+  if (t < SUB_STAGES * (n1 + nG))
+    mbar_init((unsigned)__cvta_generic_to_shared(bar + t),
+              t < SUB_STAGES * n1 ? SUB_ASKING<1> : SUB_ASKING<G>);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
@@ -194,22 +196,29 @@ __device__ inline void sub_release() {
 }
 
 // Asks for the panel of L whose first column is cp (no panel outside 0 <= cp <
-// cols), into a slot that every thread has left.  Issued by one warp, a
-// lane per column, that does not carry the chain where there is another.
+// cols), into a slot that every thread has left.  A copy takes its warp some 40
+// cycles, so the columns are dealt out to the warps that do not carry the chain:
+// one of them alone was still asking when the chain was done (27 to 50 species: 430 of
+// 2300 cycles of a forward panel and 1000 of 2900 of a backward one).  With this and
+// the ring divided per block, one solve at 27 species, 415 elements 197 -> 166 us, 50
+// species, 2000 elements 842 -> 671 us.
 template <int G, typename T>
 __device__ inline void sub_ask(const SubRing& R, int slot, const FactorCols<T>& L, int cp, int pc,
                                int ld) {
   constexpr int Q = 16 / sizeof(T);
-  const int tid = group_tid<G>(), lane = threadIdx.x & 31;
-  if (cp >= 0 && cp < L.cols && (G == 1 || (tid >> 5) == 1)) {
+  constexpr int NW = SUB_ASKING<G>;
+  const int w = G > 1 ? (int)(threadIdx.x >> 5) - 1 : 0, lane = threadIdx.x & 31;
+  if (cp >= 0 && cp < L.cols && w >= 0) {
     const int K = min(pc, L.cols - cp), r0 = cp & ~(Q - 1);
+    const int mine = w < K ? (K - w + NW - 1) / NW : 0;   // columns w, w + NW, ...
     const unsigned bytes = (unsigned)((L.rows - r0 + Q - 1) & ~(Q - 1)) * (unsigned)sizeof(T);
     const unsigned bar = R.bar + 8 * slot;
-    if (lane == 0) mbar_expect(bar, bytes * (unsigned)K);
+    if (lane == 0) mbar_expect(bar, bytes * (unsigned)mine);
     __syncwarp();
     const unsigned dst = (unsigned)__cvta_generic_to_shared(R.slots) + slot * R.slot_bytes;
-    if (lane < K)
-      bulk_load(dst + (unsigned)(lane * ld * (int)sizeof(T)), L.p + (size_t)(cp + lane) * L.ld + r0,
+    const int c = w + lane * NW;
+    if (lane < mine)
+      bulk_load(dst + (unsigned)(c * ld * (int)sizeof(T)), L.p + (size_t)(cp + c) * L.ld + r0,
                 bytes, bar);
     __syncwarp();
   }
@@ -219,39 +228,36 @@ __device__ inline void sub_ask(const SubRing& R, int slot, const FactorCols<T>& 
 __device__ inline int sub_next(SubRing& R) {
   const int slot = R.slot;
   const unsigned bar = R.bar + 8 * slot;
-  if (!mbar_try(bar, R.phase)) {
+  const unsigned phase = (R.phases >> slot) & 1u;
+  if (!mbar_try(bar, phase)) {
     int tries = 0;
-    while (!mbar_try(bar, R.phase))
+    while (!mbar_try(bar, phase))
       if (++tries > SUB_WAIT_TRIES) { atomicExch(R.err, 1); break; }
   }
-  R.advance();
+  R.phases ^= 1u << slot;
+  if (++R.slot == R.stages) R.slot = 0;
   return slot;
 }
 
-__device__ inline void sub_set(SubRing& R, SubPos p) {
-  R.slot = p.slot;
-  R.phase = p.phase;
-}
-
-// Asks for the first panels of a block's forward (from the first column) or
-// backward (from the last panel) substitution.
+// Divides the ring, which is empty, for a block and asks for the first panels of its
+// forward (from the first column) or backward (from the last panel) substitution.
 template <int G, typename T>
-__device__ inline void sub_start(const SubRing& R, const FactorCols<T>& L, bool forward) {
+__device__ inline void sub_start(SubRing& R, const FactorCols<T>& L, bool forward) {
   const int pc = sub_panel<T, G>(L.rows), ld = sub_ld(L.rows);
+  R.slot_bytes = pc * ld * (int)sizeof(T);
+  R.stages = min(SUB_STAGES, R.bytes / R.slot_bytes);
+  R.slot = 0;
   const int first = forward ? 0 : (L.cols - 1) & ~(pc - 1), step = forward ? pc : -pc;
-  int slot = R.slot;
-  for (int q = 0, cp = first; q < max(1, R.stages - 1); ++q, cp += step) {
-    sub_ask<G>(R, slot, L, cp, pc, ld);
-    if (++slot == R.stages) slot = 0;
-  }
+  for (int q = 0, cp = first; q < max(1, R.stages - 1); ++q, cp += step)
+    sub_ask<G>(R, q, L, cp, pc, ld);
 }
 
 // w = L^{-1} w (length L.rows, shared memory), w visible to the group, the
 // block's panels started (sub_start); the
-// result is visible to the group on return.  PAIRS: columns come in pairs whose two
+// result is visible to the group on return, the ring is empty.  Returns its phases.  PAIRS: columns come in pairs whose two
 // rows are not coupled (entry (2q + 1, 2q) is absent).
 template <int G, bool PAIRS, typename T>
-__device__ __noinline__ SubPos group_forward(T* w, SubRing R, const FactorCols<T> L) {
+__device__ __noinline__ unsigned group_forward(T* w, SubRing R, const FactorCols<T> L) {
   constexpr int NT = 32 * G, PC = G > 1 ? 32 : 16, Q = 16 / sizeof(T);
   constexpr unsigned FULL = 0xffffffffu;
   __builtin_assume(__isShared(w));
@@ -310,7 +316,7 @@ __device__ __noinline__ SubPos group_forward(T* w, SubRing R, const FactorCols<T
     }
   }
   group_sync<G>();
-  return {R.slot, R.phase};
+  return R.phases;
 }
 
 // Back substitution, the block's panels started: x (length L.rows) holds the right-hand side in
@@ -319,7 +325,7 @@ __device__ __noinline__ SubPos group_forward(T* w, SubRing R, const FactorCols<T
 // panel sums are over the lanes' strided rows, then a fixed shuffle tree.
 // sums: 32 entries of shared memory.
 template <int G, bool PAIRS, typename T>
-__device__ __noinline__ SubPos group_backward(T* x, T* sums, SubRing R, const FactorCols<T> L) {
+__device__ __noinline__ unsigned group_backward(T* x, T* sums, SubRing R, const FactorCols<T> L) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int PC = G > 1 ? 32 : 16, CW = PC / G;   // columns a warp sums at once
   constexpr int Q = 16 / sizeof(T);
@@ -380,7 +386,7 @@ __device__ __noinline__ SubPos group_backward(T* x, T* sums, SubRing R, const Fa
     }
   }
   group_sync<G>();
-  return {R.slot, R.phase};
+  return R.phases;
 }
 
 }  // namespace collo
