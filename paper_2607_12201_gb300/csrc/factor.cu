@@ -1993,14 +1993,18 @@ k_schur(DevProb P, const int* __restrict__ inert, const double* __restrict__ chu
   schur_block(P, inert, chunkS, wtt, sigma, dw, S, in_global ? S.S : sS);
 }
 
-// ---- solves: one warp or one CUDA block per block ------------------------------------
+// ---- solves: one warp or a group of them per block -----------------------------------
 // Blocks of at most SOLVE_NARROW rows are solved by one warp each, eight at a
-// time in a CUDA block; larger ones by the whole CUDA block (subst.cuh).  One
-// solve against one warp per block throughout, two columns loaded per step: 10
+// time in a CUDA block; larger ones by the whole CUDA block, or, many of them at
+// once, by groups of its warps (subst.cuh, launch_solve_b).  One solve against one warp per block throughout, two columns loaded per step: 10
 // species, 400 elements 148 -> 133 us; 27 species, 415 elements 394 -> 166 us; 50
 // species, 2000 elements 1692 -> 671 us.
 constexpr int SOLVE_NARROW = 128;
-constexpr int SOLVE_G = FBS / 32;   // warps of a wide block's group
+constexpr int SOLVE_G = SUB_WARPS;
+// Rows up to which groups of four warps beat one of eight when there are many wide
+// blocks (launch_solve_b).
+constexpr int SOLVE_G4_ROWS = 320;
+static_assert(SUB_WARPS == FBS / 32, "one block's warps");
 __host__ __device__ inline bool elem_solve_wide(const DevProb& P) { return P.ext > SOLVE_NARROW; }
 __host__ __device__ inline bool bcr_solve_wide(const DevProb& P) { return P.bext > SOLVE_NARROW; }
 // Dynamic shared memory of a solve kernel: narrow blocks of at most pn rows, wide
@@ -2036,18 +2040,14 @@ size_t solve_smem(int pn, int pw, int max_p, const bool (&many)[2]) {
   if (b > 0 && b <= SOLVE_HALF_SM) return pw > 0 ? SOLVE_HALF_SM : b;
   return need(false);
 }
-// The part of the `bytes` of dynamic shared memory of this thread's group: all for
-// G > 1 (blocks of up to msz rows), this warp's share for G = 1.
+// The part of the `bytes` of dynamic shared memory of this thread's group, for
+// blocks of up to msz rows.
 template <typename T, int G>
 __device__ inline SubMem<T, G> sub_mem(unsigned char* sm, size_t bytes, int msz,
                                        unsigned long long* bars, int* err) {
-  if constexpr (G > 1) {
-    return sub_carve<T, G>(sm, bytes, msz, bars, err);
-  } else {
-    const int warp = threadIdx.x >> 5;
-    const size_t share = (bytes / SOLVE_G) & ~size_t(15);
-    return sub_carve<T, 1>(sm + warp * share, share, msz, bars + warp * SUB_STAGES, err);
-  }
+  const int g = group_index<G>();
+  const size_t share = (bytes / (SOLVE_G / G)) & ~size_t(15);
+  return sub_carve<T, G>(sm + g * share, share, msz, bars + g * SUB_STAGES, err);
 }
 constexpr int SOLVE_BARS = SOLVE_G * SUB_STAGES;   // barriers of a kernel's narrow groups
 
@@ -2258,7 +2258,8 @@ k_theta_solve(DevProb P, const double* __restrict__ chunkR, const double* __rest
               DevSchur S, double* __restrict__ sol, int* err, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SUB_STAGES];
-  sub_init<SOLVE_G>(bars, 0, 1);
+  sub_init<SOLVE_G>(bars, 1);
+  sub_ready();
   SubMem<double, SOLVE_G> sm = sub_mem<double, SOLVE_G>(smraw, smem, P.p, bars, err);
   theta_solve_block(P, chunkR, b, S, sol, sm);
 }
@@ -2333,7 +2334,8 @@ k_elem_solve(DevProb P, DevFactor<T> F, DevSchur S, const double* __restrict__ b
              double* __restrict__ sol, int fwd, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SOLVE_BARS];
-  sub_init<SOLVE_G>(bars, G > 1 ? 0 : SOLVE_G, G > 1 ? 1 : 0);
+  sub_init<G>(bars, SOLVE_G / G);
+  sub_ready();
   SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.ext, bars, &F.gbar->err);
   const int e = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
   if (e >= P.N) return;
@@ -2348,7 +2350,8 @@ k_bcr_solve(DevProb P, DevFactor<T> F, DevSchur S, double* __restrict__ sol, int
             int final_level, size_t smem) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[SOLVE_BARS];
-  sub_init<SOLVE_G>(bars, G > 1 ? 0 : SOLVE_G, G > 1 ? 1 : 0);
+  sub_init<G>(bars, SOLVE_G / G);
+  sub_ready();
   SubMem<T, G> sm = sub_mem<T, G>(smraw, smem, P.bext, bars, &F.gbar->err);
   const int nblk = final_level ? 1 : bcr_level_blocks(P.N, stride);
   const int bi = G > 1 ? blockIdx.x : blockIdx.x * SOLVE_G + (threadIdx.x >> 5);
@@ -2617,34 +2620,40 @@ struct SolvePlan {
 // same block then solves the parameter system and substitutes back down to
 // level `lsplit`.  Every block solve is the same code as in the
 // single-instance launches, so the result does not depend on the split.
-template <typename T>
+template <typename T, int WG>
 __global__ void __launch_bounds__(FBS, sizeof(T) == 4 ? 2 : 1)
 k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A, SolvePlan sp,
           const int* __restrict__ pre_lv, int maxL, int lsplit,
           const int* __restrict__ pre_cs, int ir, int pn, int pw, int max_p, size_t smem,
           GridBar* gb) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ unsigned long long bars[SOLVE_BARS + 2 * SUB_STAGES];
+  constexpr int WIDE = SOLVE_G / WG;   // groups for wide blocks
+  __shared__ unsigned long long bars[SOLVE_BARS + (WIDE + 1) * SUB_STAGES];
   __shared__ LoneInst lone;
   lone_load(lone, insts, act, A);
-  sub_init<SOLVE_G>(bars, SOLVE_G, 2);
+  unsigned long long* wide_bars = bars + SOLVE_BARS;
+  unsigned long long* theta_bars = wide_bars + WIDE * SUB_STAGES;
+  sub_init<1>(bars, SOLVE_G);
+  sub_init<WG>(wide_bars, WIDE);
+  sub_init<SOLVE_G>(theta_bars, 1);
+  sub_ready();
   auto inst = [&](int k) -> const DevInst& {
     return A == 1 ? *reinterpret_cast<const DevInst*>(lone.b) : insts[act[k]];
   };
   unsigned int ep = 0;
   const int warp = threadIdx.x >> 5, wpb = FBS / 32;
   const int gw = blockIdx.x * wpb + warp, nw = gridDim.x * wpb;
+  const int wg = blockIdx.x * WIDE + group_index<WG>(), nwg = gridDim.x * WIDE;
   // the three groups use the same shared memory, one at a time
   SubMem<T, 1> narrow = sub_mem<T, 1>(smraw, smem, max(pn, 1), bars, &gb->err);
-  SubMem<T, SOLVE_G> wide =
-      sub_mem<T, SOLVE_G>(smraw, smem, max(pw, 1), bars + SOLVE_BARS, &gb->err);
+  SubMem<T, WG> wide = sub_mem<T, WG>(smraw, smem, max(pw, 1), wide_bars, &gb->err);
   SubMem<double, SOLVE_G> theta =
-      sub_mem<double, SOLVE_G>(smraw, smem, max(max_p, 1), bars + SOLVE_BARS + SUB_STAGES, &gb->err);
+      sub_mem<double, SOLVE_G>(smraw, smem, max(max_p, 1), theta_bars, &gb->err);
   auto phase_end = [&]() { sub_release(); grid_barrier(gb, ep); };
   // Items t0, t0 + step, ... of a list for one group: cols(I, i) are an item's L
   // columns, run(I, i, next) its substitution.
   auto list = [&](const int* pre, int t0, int step, auto& sm, bool fwd, auto&& cols, auto&& run) {
-    constexpr int G = std::is_same_v<std::decay_t<decltype(sm)>, SubMem<T, 1>> ? 1 : SOLVE_G;
+    constexpr int G = std::is_same_v<std::decay_t<decltype(sm)>, SubMem<T, 1>> ? 1 : WG;
     const int tot = pre[A];
     auto find = [&](int t) { return A == 1 ? 0 : find_item(pre, A, t); };
     int k = t0 < tot ? find(t0) : 0;
@@ -2664,7 +2673,7 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
         else elem_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, e, sm, next);
       };
     };
-    list(sp.elem[1], blockIdx.x, gridDim.x, wide, fwd, cols, one(wide));
+    list(sp.elem[1], wg, nwg, wide, fwd, cols, one(wide));
     sub_release();
     __syncthreads();
     list(sp.elem[0], gw, nw, narrow, fwd, cols, one(narrow));
@@ -2680,7 +2689,7 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
         else bcr_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, 1 << lv, 0, bi, sm, next);
       };
     };
-    list(sp.lv[1] + o, blockIdx.x, gridDim.x, wide, fwd, cols, one(wide));
+    list(sp.lv[1] + o, wg, nwg, wide, fwd, cols, one(wide));
     sub_release();
     __syncthreads();
     list(sp.lv[0] + o, gw, nw, narrow, fwd, cols, one(narrow));
@@ -2697,7 +2706,8 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
       else bcr_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, stride, fin, bi, sm, [] {});
     };
     if (bcr_solve_wide(I.P))
-      for (int bi = 0; bi < nb; ++bi) run(bi, wide, std::integral_constant<int, SOLVE_G>{});
+      for (int bi = group_index<WG>(); bi < nb; bi += WIDE)
+        run(bi, wide, std::integral_constant<int, WG>{});
     else
       for (int bi = warp; bi < nb; bi += wpb) run(bi, narrow, std::integral_constant<int, 1>{});
     sub_release();
@@ -2982,18 +2992,32 @@ template <typename T>
 cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            const int* const elem[2], const int* const lv[2], const int* pre_lv,
                            int maxL, int lsplit, const int* pre_cs, int ir, int pn, int pw,
-                           const bool (&many)[2], GridBar* gb, int max_p, int grid_want, cudaStream_t st,
-                           int reserve) {
+                           const bool (&many)[2], bool most, GridBar* gb, int max_p,
+                           int grid_want, cudaStream_t st, int reserve) {
   if (A == 0) return cudaSuccess;
   size_t smem = solve_smem<T>(pn, pw, std::max(max_p, 1), many);
-  opt_in_smem(k_solve_b<T>, smem, true);
-  int grid = coop_grid(k_solve_b<T>, FBS, smem, grid_want, reserve);
+  // Wide blocks: a group's chain costs the same whatever its size, and only the rows
+  // below it gain from more warps.  With several blocks for each CUDA block the device
+  // holds, more and smaller groups cover one another's chains: two warps each
+  // as long as four such groups have a panel each in the memory (about 200 rows in
+  // FP32), four warps from twice as many blocks on up to SOLVE_G4_ROWS.  One solve of A problems of
+  // 400 elements by groups of 8 / 4 / 2 warps, us: 16 species, A = 2 182 / 177 / 172, A = 32
+  // 754 / 560 / 518; 20 species, A = 32 978 / 773 / 736; 27 species (one panel of 35 KB), A =
+  // 2 233 / 245, A = 4 312 / 302, A = 32 1395 / 1189; 33 species, A = 4 372 / 371; 36, A = 8
+  // 590 / 615.
+  auto kern = k_solve_b<T, SOLVE_G>;
+  if (many[1] && SOLVE_G / 2 * group_smem<T, 2>(pw, 1, 1) <= smem)
+    kern = k_solve_b<T, 2>;
+  else if (most && pw <= SOLVE_G4_ROWS && SOLVE_G / 4 * group_smem<T, 4>(pw, 1, 1) <= smem)
+    kern = k_solve_b<T, 4>;
+  opt_in_smem(kern, smem, true);
+  int grid = coop_grid(kern, FBS, smem, grid_want, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
   SolvePlan sp{{elem[0], elem[1]}, {lv[0], lv[1]}};
   void* args[] = {(void*)&insts, (void*)&act, &A, &sp, (void*)&pre_lv, &maxL,
                   &lsplit, (void*)&pre_cs, &ir, &pn, &pw, &max_p, &smem, &gb};
   count_launch();
-  return cudaLaunchCooperativeKernel((void*)k_solve_b<T>, dim3(grid), dim3(FBS), args, smem, st);
+  return cudaLaunchCooperativeKernel((void*)kern, dim3(grid), dim3(FBS), args, smem, st);
 }
 
 template cudaError_t launch_factor_b<float>(const DevInst*, const int*, int, const int*,
@@ -3018,11 +3042,11 @@ int elem_rt_threads(const DevProb& P, bool f32) {
 bool solve_wide(const DevProb& P, bool elem) { return elem ? elem_solve_wide(P) : bcr_solve_wide(P); }
 template cudaError_t launch_solve_b<float>(const DevInst*, const int*, int, const int* const[2],
                                            const int* const[2], const int*, int, int, const int*,
-                                           int, int, int, const bool (&)[2], GridBar*, int, int,
+                                           int, int, int, const bool (&)[2], bool, GridBar*, int, int,
                                            cudaStream_t, int);
 template cudaError_t launch_solve_b<double>(const DevInst*, const int*, int, const int* const[2],
                                             const int* const[2], const int*, int, int, const int*,
-                                            int, int, int, const bool (&)[2], GridBar*, int, int,
+                                            int, int, int, const bool (&)[2], bool, GridBar*, int, int,
                                            cudaStream_t, int);
 template size_t elem_factor_smem<float>(const DevProb&, bool);
 template size_t elem_factor_smem<double>(const DevProb&, bool);

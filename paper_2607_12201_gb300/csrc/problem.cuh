@@ -87,14 +87,14 @@ size_t bcr_rt_stage_bytes(const DevProb& P, bool f32);
 // Solve work lists: elem, lv as SolvePlan (prefix arrays of the narrow [0] and
 // wide [1] instances), pre_lv all instances' blocks per level; pn, pw: rows of the
 // largest narrow / wide block (0: none); many: more than two narrow / wide elements
-// for each warp / CUDA block the device holds.
+// for each warp / CUDA block the device holds; most: four wide ones or more.
 template <typename T>
 cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
                            const int* const elem[2], const int* const lv[2], const int* pre_lv,
                            int maxL, int lsplit, const int* pre_cs, int ir, int pn, int pw,
-                           const bool (&many)[2], GridBar* gb, int max_p, int grid_want, cudaStream_t st,
-                           int reserve = 0);
-// Whether P's element / reduction blocks are solved by a whole CUDA block each.
+                           const bool (&many)[2], bool most, GridBar* gb, int max_p,
+                           int grid_want, cudaStream_t st, int reserve = 0);
+// Whether P's element / reduction blocks are solved by several warps each.
 bool solve_wide(const DevProb& P, bool elem);
 template <typename T>
 size_t elem_factor_smem(const DevProb& P, bool full);

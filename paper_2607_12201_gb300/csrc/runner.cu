@@ -49,10 +49,11 @@ struct Plan {
   size_t smem_eval[2] = {0, 0};   // without / with derivatives
   size_t smem_f[2] = {0, 0}, smem_sweep = 0;
   int cap_f[2] = {1 << 30, 1 << 30};
-  int solve_pw = 0;             // rows of the largest block a CUDA block solves
+  int solve_pw = 0;             // rows of the largest block several warps solve
   int solve_pn = 0;             // ... that one warp solves
-  bool solve_many[2] = {false, false};   // more than two one-warp / CUDA-block elements
+  bool solve_many[2] = {false, false};   // more than two one-warp / wide elements
                                          // for each warp / CUDA block the device holds
+  bool solve_most = false;      // four wide ones or more
   int solve_want = 0;           // CUDA blocks that hold every element at once
   int rt_threads[2] = {0, 0};   // block size of the register-tiled element kernel
   size_t rt_smem[2] = {0, 0};   // its dynamic shared memory
@@ -282,6 +283,7 @@ struct Runner {
     // n_slabs: two per SM
     pl.solve_many[0] = items[0] > 2 * probs[slots[0]]->n_slabs * 8;
     pl.solve_many[1] = items[1] > 2 * probs[slots[0]]->n_slabs;
+    pl.solve_most = items[1] >= 4 * probs[slots[0]]->n_slabs;
     pl.off_cs_s = o; h[o] = 0;
     for (int k = 0; k < A; ++k) {
       const DevProb& Q = P(slots[k]);
@@ -479,7 +481,8 @@ struct Runner {
     const int* lv[2] = {pl.solve_lv(0), pl.solve_lv(1)};
     auto launch = prec == COLLO_PRECISION_MIXED ? launch_solve_b<float> : launch_solve_b<double>;
     e = launch(d_insts, pl.act(), pl.A, elem, lv, pl.pre_lv(), pl.maxL, pl.lsplit, pl.pre_cs_r(), ir,
-               pl.solve_pn, pl.solve_pw, pl.solve_many, gbar, pl.max_p, pl.solve_want, stream, reserve_sms);
+               pl.solve_pn, pl.solve_pw, pl.solve_many, pl.solve_most, gbar, pl.max_p, pl.solve_want, stream,
+               reserve_sms);
     COLLO_CUDA(e);
     return COLLO_OK;
   }

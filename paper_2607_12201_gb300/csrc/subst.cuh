@@ -1,5 +1,5 @@
-// Substitutions through the eliminated columns of a block, by a group of one or
-// eight warps.
+// Substitutions through the eliminated columns of a block, by a group of one, two,
+// four or eight warps.
 //
 // Bound: the chain of dependent columns, and the memory latency of the factor's
 // entries behind it (for many large blocks, their bandwidth).  Columns are taken
@@ -139,15 +139,23 @@ struct SubRing {
   int* err;                 // GridBar::err
 };
 
+// Groups of G of the block's eight warps.  A block's result does not depend on G > 1:
+// panels are those of the block's rows, a row of the forward substitution takes the
+// columns in their order, and a column's sum of the backward one is over the
+// lanes' strided rows and then the same tree, whichever warp has it.
+constexpr int SUB_WARPS = 8;
+template <int G>
+__device__ inline int group_index() { return (int)threadIdx.x / (32 * G); }
 template <int G>
 __device__ inline void group_sync() {
-  if constexpr (G > 1) __syncthreads();
-  else __syncwarp();
+  if constexpr (G == 1) __syncwarp();
+  else if constexpr (G == SUB_WARPS) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + group_index<G>()), "n"(32 * G) : "memory");
 }
 
-// Thread of the group: G = 1 a warp of the block, G > 1 the whole block.
+// Thread of the group.
 template <int G>
-__device__ inline int group_tid() { return G > 1 ? (int)threadIdx.x : (int)(threadIdx.x & 31); }
+__device__ inline int group_tid() { return (int)threadIdx.x % (32 * G); }
 
 // A group's memory for blocks of up to msz rows in `bytes` at p (16-byte
 // aligned): vector and sums, ring; bar: its SUB_STAGES barriers, initialised
@@ -177,14 +185,14 @@ __device__ inline SubMem<T, G> sub_carve(unsigned char* p, size_t bytes, int msz
 // carries the chain, where there are others.
 template <int G>
 constexpr int SUB_ASKING = G > 1 ? G - 1 : 1;
-// Initialises the barriers of n1 groups of one warp and, behind them, nG groups of G
-// (the whole block calls).
+// Initialises the barriers of n groups of G (all of a kernel's, then sub_ready; the
+// whole block calls).
 template <int G>
-__device__ inline void sub_init(unsigned long long* bar, int n1, int nG) {
-  const int t = threadIdx.x;
-  if (t < SUB_STAGES * (n1 + nG))
-    mbar_init((unsigned)__cvta_generic_to_shared(bar + t),
-              t < SUB_STAGES * n1 ? SUB_ASKING<1> : SUB_ASKING<G>);
+__device__ inline void sub_init(unsigned long long* bar, int n) {
+  if ((int)threadIdx.x < n * SUB_STAGES)
+    mbar_init((unsigned)__cvta_generic_to_shared(bar + threadIdx.x), SUB_ASKING<G>);
+}
+__device__ inline void sub_ready() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
@@ -207,7 +215,7 @@ __device__ inline void sub_ask(const SubRing& R, int slot, const FactorCols<T>& 
                                int ld) {
   constexpr int Q = 16 / sizeof(T);
   constexpr int NW = SUB_ASKING<G>;
-  const int w = G > 1 ? (int)(threadIdx.x >> 5) - 1 : 0, lane = threadIdx.x & 31;
+  const int w = G > 1 ? (group_tid<G>() >> 5) - 1 : 0, lane = threadIdx.x & 31;
   if (cp >= 0 && cp < L.cols && w >= 0) {
     const int K = min(pc, L.cols - cp), r0 = cp & ~(Q - 1);
     const int mine = w < K ? (K - w + NW - 1) / NW : 0;   // columns w, w + NW, ...
@@ -245,7 +253,10 @@ template <int G, typename T>
 __device__ inline void sub_start(SubRing& R, const FactorCols<T>& L, bool forward) {
   const int pc = sub_panel<T, G>(L.rows), ld = sub_ld(L.rows);
   R.slot_bytes = pc * ld * (int)sizeof(T);
-  R.stages = min(SUB_STAGES, R.bytes / R.slot_bytes);
+  R.stages = 1;
+#pragma unroll
+  for (int st = 2; st <= SUB_STAGES; ++st)
+    if (st * R.slot_bytes <= R.bytes) R.stages = st;
   R.slot = 0;
   const int first = forward ? 0 : (L.cols - 1) & ~(pc - 1), step = forward ? pc : -pc;
   for (int q = 0, cp = first; q < max(1, R.stages - 1); ++q, cp += step)
@@ -354,7 +365,7 @@ __device__ __noinline__ unsigned group_backward(T* x, T* sums, SubRing R, const 
         for (int c = 0; c < CW; ++c) acc[c] = fma(k0 + c < K ? s[c * ld] : T(0), xr, acc[c]);
       }
       const T s = warp_rows_sum<T, CW>(acc);
-      constexpr int SH = CW == 16 ? 1 : 3;   // lane l has column l >> SH
+      constexpr int SH = CW == 16 ? 1 : CW == 8 ? 2 : 3;   // lane l has column l >> SH
       if ((lane & ((1 << SH) - 1)) == 0) sums[k0 + (lane >> SH)] = s;
     }
     group_sync<G>();
