@@ -23,14 +23,20 @@
 // previous element's stage increments, a new inverse when the contraction is
 // slow.
 // Residual, update and stopping test are FP64; the FP32 inverse only decides
-// how fast the iteration contracts.
+// how fast the iteration contracts.  The short way's contraction is linear, and
+// what it leaves behind adds up along the chain: it goes on until the remainder,
+// from the slowest contraction seen with this inverse, is below SHORT_REST of the
+// largest state, or the correction is at rounding level.  Ending at 2e-16 and at the
+// contraction of the last step alone left the sweep of 27 species, 120 elements
+// 2.3e-13 from the 64-bit solution and that of 50 species, 400 elements 3.4e-14; now
+// 7e-16 and 1e-15, as with an LU in every iteration.
 //
 // Measured on a GB300 against Newton's method with an FP32 LU in every
 // iteration (one warp up to 32 unknowns, one block above): 10 species, 400
-// elements 18.4 -> 1.74 ms; 27 species, 415 elements 179 -> 2.95 ms (2.5
-// iterations and 0.03 inversions per element); per element at 50 species 1480 ->
-// 13 us, at 100 species 10.7 -> 0.83 ms.  On meshes so coarse that every element
-// goes the plain way: 27 species 563 -> 32 us, 100 species 14.5 -> 11.5 ms.
+// elements 18.4 -> 2.4 ms; 27 species, 415 elements 181 -> 4.0 ms (the remainder
+// above costs a third: 1.7 and 2.9 ms with the shorter stop); 50 species, 400 elements
+// 455 -> 6.8 ms.  On meshes so coarse that every element
+// goes the plain way: 27 species 563 -> 32 us an element, 100 species 14.5 -> 11.5 ms.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -43,6 +49,7 @@ namespace collo {
 constexpr int SWEEP_MAXIT = 30;
 constexpr float CHORD_RATE = 0.25f;   // contraction per iteration below which an inverse is kept
 constexpr float EASY_STEP = 0.05f;      // largest first correction of the short way, against max |Z|
+constexpr float SHORT_REST = 1e-18f;    // remainder at which the short way ends, against max |Z|
 constexpr int SWEEP_MAX_THREADS = 512;
 constexpr int SWEEP_REG_DIM = 192;    // largest K n whose inverse is held in registers
 
@@ -277,6 +284,7 @@ __device__ void sweep_one(const DevProb& P, double* __restrict__ x, int* __restr
   int my_z = -1, my_step = 0;   // register inverse: place in Z of this lane's sum, step[g_row]
   int nfail = 0;
   bool have = false;            // an inverse is held
+  float rate = 0.f;             // ... its slowest contraction so far
   int least = SWEEP_MAXIT, excess = 0;   // iterations since it was made (below)
   const int excess_max = 8 + dim / 6;
   int cur = 0;
@@ -361,6 +369,7 @@ __device__ void sweep_one(const DevProb& P, double* __restrict__ x, int* __restr
           have = true;
           made = true;
           if (attempt == 0) prev = INFINITY;   // the next correction is this inverse's first
+          rate = 0.f;
           least = SWEEP_MAXIT;
           excess = 0;
           sweep_bar<NW>();   // step[] is complete
@@ -385,8 +394,12 @@ __device__ void sweep_one(const DevProb& P, double* __restrict__ x, int* __restr
           double g = 0.0;
           if (g_on) {
             const double* Dk = D[g_k + 1];
-            for (int j = g_part; j < np; j += LPR)
-              g = fma(Dk[j], j == 0 ? z0[g_q] : Z[(j - 1) * zl + g_q], g);
+            // the products with D nearly cancel: all in one chain of multiply-adds
+            // (rounded apart by several threads they tripled the sweep's error)
+            if (g_part == 0) {
+              g = Dk[0] * z0[g_q];
+              for (int j = 1; j < np; ++j) g = fma(Dk[j], Z[(j - 1) * zl + g_q], g);
+            }
             const double* mo = s.mon + g_k * r;
             for (int e = g_e0 + g_part; e < g_e1; e += LPR) g = fma(-s.coef[e], mo[s.lst[e]], g);
           }
@@ -452,12 +465,14 @@ __device__ void sweep_one(const DevProb& P, double* __restrict__ x, int* __restr
         if (dmax >= 0x7f800000u) { have = false; break; }
         const float dz = __uint_as_float(dmax);
         const float sc = fmaxf(1.f, (float)__hiloint2double((int)zmax, 0));
+        // the contraction, while the correction is above the residual's rounding
+        if (attempt == 0 && prev < INFINITY && dz > 1e-14f * sc) rate = fmaxf(rate, dz / prev);
         if (dz <= 1e-12f * sc) {
-          // converged to the tolerance; the iteration's linear contraction rho
-          // leaves an error of about rho / (1 - rho) dz: go on until that is at
-          // rounding level too, or the correction no longer halves
+          // converged to the tolerance; a linear contraction leaves an error of about
+          // rate / (1 - rate) dz: the short way goes on until that is small too, or
+          // the correction is at rounding level or no longer halves
           if (attempt == 1 || dz <= 2e-16f * sc || dz > 0.5f * prev ||
-              (prev < INFINITY && dz * dz <= 2e-16f * sc * (prev - dz))) {
+              (rate > 0.f && rate * dz <= SHORT_REST * sc * (1.f - rate))) {
             ok = true;
             break;
           }
