@@ -369,7 +369,7 @@ __device__ void eval_reduce_one(const DevProb& P, const DevEval& E, double* out,
   if (block > 0) {
     const int q0 = 32 * (block - 1);
     const double v = column_sums(E.wtt_part, P.N, P.p, q0, sh);
-    if (tid < 32 && q0 + tid < P.p) E.wtt[q0 + tid] = v;
+    if ((tid & 31) == 0 && q0 + (tid >> 5) < P.p) E.wtt[q0 + (tid >> 5)] = v;
     return;
   }
   double a = 0.0, b = 0.0, c = 0.0;
@@ -379,9 +379,7 @@ __device__ void eval_reduce_one(const DevProb& P, const DevEval& E, double* out,
       b += E.part[i * 4 + 1];
       c = fmax(c, E.part[i * 4 + 2]);
     }
-  a = first_sum<RED_BS>(a, sh);
-  b = first_sum<RED_BS>(b, sh);
-  c = first_max<RED_BS>(c, sh);
+  first_sums(a, b, c, sh);
   if (tid == 0) {
     E.red[0] = a; E.red[1] = b; E.red[2] = c;
     if (out) { out[O_PHI] = a; out[O_C1] = b; out[O_CINF] = c; }
@@ -389,21 +387,21 @@ __device__ void eval_reduce_one(const DevProb& P, const DevEval& E, double* out,
 }
 
 __global__ void __launch_bounds__(TH_BS) k_eval_reduce(DevProb P, DevEval E) {
-  __shared__ double sh[32 * 33];
+  __shared__ double sh[TH_SH];
   eval_reduce_one(P, E, nullptr, blockIdx.x, sh);
 }
 
 // Reduction of collo_eval_noalloc: the partials in the fixed scratch, Phi
 // into the caller's output (out[0] = Phi).
 __global__ void __launch_bounds__(TH_BS) k_eval_reduce_noalloc(DevProb P, DevEval E, double* phi) {
-  __shared__ double sh[32 * 33];
+  __shared__ double sh[TH_SH];
   eval_reduce_one(P, E, nullptr, blockIdx.x, sh);
   if (blockIdx.x == 0 && threadIdx.x == 0) *phi = E.red[0];
 }
 
 __global__ void __launch_bounds__(TH_BS)
 k_eval_reduce_b(const DevInst* __restrict__ insts, const int* __restrict__ act) {
-  __shared__ double sh[32 * 33];
+  __shared__ double sh[TH_SH];
   const DevInst& I = insts[act[blockIdx.x]];
   if ((int)blockIdx.y >= theta_blocks(I.P.p)) return;
   eval_reduce_one(I.P, I.E, I.out, blockIdx.y, sh);
@@ -441,7 +439,7 @@ k_kkt_resid_theta(DevProb P, DevEval E, const double* __restrict__ sigma, double
                   const double* __restrict__ bc, double* __restrict__ rout,
                   const double* __restrict__ thpart, const double* __restrict__ npart,
                   const double* __restrict__ th_extra, double* __restrict__ out) {
-  __shared__ double sh[32 * 33];
+  __shared__ double sh[TH_SH];
   resid_theta_one(P, E, sigma, dw, vx, bx, bxs, bc, rout, thpart, npart, th_extra, out,
                   blockIdx.y, sh);
 }
@@ -449,7 +447,7 @@ k_kkt_resid_theta(DevProb P, DevEval E, const double* __restrict__ sigma, double
 __global__ void __launch_bounds__(TH_BS)
 k_kkt_resid_theta_b(const DevInst* __restrict__ insts, const int* __restrict__ act,
                     const InstParams* __restrict__ prm, int mode) {
-  __shared__ double sh[32 * 33];
+  __shared__ double sh[TH_SH];
   const int k = blockIdx.x;
   const DevInst& I = insts[act[k]];
   if ((int)blockIdx.y >= theta_blocks(I.P.p)) return;

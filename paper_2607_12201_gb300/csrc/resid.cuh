@@ -10,6 +10,8 @@ namespace collo {
 constexpr int EVAL_BS = 128;
 constexpr int RED_BS = 256;
 constexpr int TH_BS = 1024;   // threads of the per-instance reductions over elements
+// Doubles of shared memory they use: column_sums, and block_max3 behind it.
+constexpr int TH_SH = 32 * 33 + 3 * TH_BS / 32;
 
 // |v| as bits that order like the values, a value that is not a number as zero
 // (fmax passes over one).  Comparing them costs integer instructions; an FP64
@@ -44,10 +46,11 @@ __device__ inline void block_max3(unsigned long long& a, unsigned long long& b,
 }
 // Column sums of v[N][L] for the 32 columns from q0 on, by TH_BS threads: per
 // column 32 partial sums over i = l, l + 32, ... in that order, then a fixed tree;
-// the sum of column q0 + tid is valid on threads tid < 32.  A warp reads 32
+// warp w returns the sum of column q0 + w.  A warp reads 32
 // neighbouring columns of a row, so the loads are whole lines (one warp per column
 // read a sector per lane: 50 species, 2000 elements 225 us for all columns on one
-// SM, now a few us on p / 32 of them).  sh: 32 x 33 doubles.
+// SM, 37 us on p / 32 of them).  One barrier: the tree over a column's partial sums
+// is a warp's.  sh: TH_SH doubles, the first 32 x 33.
 __device__ inline double column_sums(const double* __restrict__ v, int N, int L, int q0,
                                      double* sh) {
   const int ql = threadIdx.x & 31, l = threadIdx.x >> 5, q = q0 + ql;
@@ -63,14 +66,9 @@ __device__ inline double column_sums(const double* __restrict__ v, int N, int L,
     }
   sh[l * 33 + ql] = y;
   __syncthreads();
+  y = sh[ql * 33 + l];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    if (l < o) {
-      y += sh[(l + o) * 33 + ql];
-      sh[l * 33 + ql] = y;
-    }
-    __syncthreads();
-  }
+  for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
   return y;
 }
 // Blocks of an instance's reductions: the scalars, and 32 columns each.
@@ -107,34 +105,33 @@ __device__ inline double block_max(double v, double* sh) {
   return r;
 }
 
-// The same over the first BS threads of a larger block (all its threads call).
-template <int BS>
-__device__ inline double first_sum(double v, double* sh) {
+// The sums of a and b and the maximum of c over the first RED_BS threads of a larger
+// block (all its threads call), in block_sum's order; valid on thread 0.  One
+// barrier: a lane of the first warp adds its column of the tree, then shuffles
+// (three trees in shared memory, nine barriers of 32 warps each: the reductions of a
+// two-species evaluation 12.4 -> 8.0 us).  sh: 3 RED_BS doubles.
+__device__ inline void first_sums(double& a, double& b, double& c, double* sh) {
   const int t = threadIdx.x;
-  if (t < BS) sh[t] = v;
+  if (t < RED_BS) { sh[t] = a; sh[RED_BS + t] = b; sh[2 * RED_BS + t] = c; }
   __syncthreads();
+  if (t >= 32) return;
+  auto tree = [&](const double* s, auto op) {
+    double v[RED_BS / 32];
 #pragma unroll
-  for (int s = BS / 2; s > 0; s >>= 1) {
-    if (t < s) sh[t] += sh[t + s];
-    __syncthreads();
-  }
-  double r = sh[0];
-  __syncthreads();
-  return r;
-}
-template <int BS>
-__device__ inline double first_max(double v, double* sh) {
-  const int t = threadIdx.x;
-  if (t < BS) sh[t] = v;
-  __syncthreads();
+    for (int k = 0; k < RED_BS / 32; ++k) v[k] = s[t + 32 * k];
 #pragma unroll
-  for (int s = BS / 2; s > 0; s >>= 1) {
-    if (t < s) sh[t] = fmax(sh[t], sh[t + s]);
-    __syncthreads();
-  }
-  double r = sh[0];
-  __syncthreads();
-  return r;
+    for (int h = RED_BS / 64; h > 0; h >>= 1)
+#pragma unroll
+      for (int k = 0; k < h; ++k) v[k] = op(v[k], v[k + h]);
+    double y = v[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) y = op(y, __shfl_xor_sync(0xffffffffu, y, o));
+    return y;
+  };
+  auto add = [](double x, double y) { return x + y; };
+  a = tree(sh, add);
+  b = tree(sh + RED_BS, add);
+  c = tree(sh + 2 * RED_BS, [](double x, double y) { return fmax(x, y); });
 }
 
 // Structured FP64 product y = K v of the regularised KKT matrix
@@ -315,17 +312,25 @@ __device__ inline void resid_theta_one(const DevProb& P, const DevEval& E,
     if (bx)
       for (int q = tid; q < p; q += TH_BS) mb = max_bits(mb, abs_bits(bx[nz + q]));
   } else {
-    const int q0 = 32 * (block - 1), q = q0 + tid;
+    const int q0 = 32 * (block - 1), q = q0 + (tid >> 5);
+    const bool mine = (tid & 31) == 0 && q < p;
+    // asked for before the sum
+    double w = 0.0, v = 0.0, ex = 0.0, b = 0.0;
+    if (mine) {
+      if (vx) { w = E.wtt[q] + (sigma ? sigma[nz + q] : 0.0) + dw; v = vx[nz + q]; }
+      if (th_extra) ex = th_extra[q];
+      if (bx) b = bx[nz + q];
+    }
     double y = column_sums(thpart, N, p, q0, sh);
-    if (tid < 32 && q < p) {
-      if (vx) y += (E.wtt[q] + (sigma ? sigma[nz + q] : 0.0) + dw) * vx[nz + q];
-      if (th_extra) y -= th_extra[q];
-      const double rr = (bx ? bxs * bx[nz + q] : 0.0) - y;
+    if (mine) {
+      if (vx) y += w * v;
+      if (th_extra) y -= ex;
+      const double rr = (bx ? bxs * b : 0.0) - y;
       if (rout) rout[nz + q] = rr;
       mx = abs_bits(rr);
     }
   }
-  block_max3<TH_BS>(mx, mc, mb, reinterpret_cast<unsigned long long*>(sh));
+  block_max3<TH_BS>(mx, mc, mb, reinterpret_cast<unsigned long long*>(sh + 32 * 33));
   if (tid == 0) {
     unsigned long long* o = reinterpret_cast<unsigned long long*>(out);
     atomicMax(o, mx);
