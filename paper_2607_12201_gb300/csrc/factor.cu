@@ -1902,8 +1902,16 @@ __device__ inline double sum_chunks4(const double* __restrict__ part, int G, int
 }
 
 constexpr int SBS = 256;
-// One block: S = (total of all contributions, schur_total) + diag(W_thth + sigma +
-// dw), FP64 LDL^T with 1x1 pivots, total inertia.  work: schur_doubles(p) doubles
+// Whether the block that factors the Schur complement also totals its entries
+// (schur_total): one entry of the lower triangle per thread at most.  The totals are
+// then one pass over the chunk sums; from two passes on, all blocks share them and a
+// grid barrier follows.  A factorization of two species, 50 elements 123.0 us with the
+// barrier, 122.1 without, 11 species (253 entries), 100 elements 220.1 and 216.7, 10
+// species, 400 elements equal.
+__host__ __device__ inline bool schur_totals_inside(int p) { return p * (p + 1) / 2 <= SBS; }
+// One block: S = (total of all contributions) + diag(W_thth + sigma + dw), FP64
+// LDL^T with 1x1 pivots, total inertia.  sums: the chunk sums (summed: their
+// totals, schur_total, in the first chunk's place).  work: schur_doubles(p) doubles
 // in dynamic shared memory, or S.S itself when that does not fit: the matrix,
 // lower triangle column-major (entry (r, c) at c ld + r, the layout of the
 // factor left in S.S), and three columns of multipliers.
@@ -1912,9 +1920,9 @@ constexpr int SBS = 256;
 // pivot while the other warps apply column k to the columns beyond: one barrier
 // per column, and the reciprocal is off the other warps' path.
 __device__ void schur_block(const DevProb& P, const int* __restrict__ inert,
-                            const double* __restrict__ total, const double* __restrict__ wtt,
-                            const double* __restrict__ sigma, double dw, const DevSchur& S,
-                            double* work) {
+                            const double* __restrict__ sums, bool summed,
+                            const double* __restrict__ wtt, const double* __restrict__ sigma,
+                            double dw, const DevSchur& S, double* work) {
   __shared__ long long cnt[3];
   __shared__ long long red[3][SBS];
   const int p = P.p, N = P.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1922,10 +1930,11 @@ __device__ void schur_block(const DevProb& P, const int* __restrict__ inert,
   const size_t nz = (size_t)N * P.np * P.n;
   double* A = work;
   double* lbuf = A + (size_t)p * ld;
-  for (int idx = tid; idx < p * p; idx += SBS) {
-    const int q = idx / p, q2 = idx - q * p;
-    if (q2 > q) continue;
-    double v = total[idx];
+  for (int t = tid; t < p * (p + 1) / 2; t += SBS) {
+    int q, q2;
+    tri_tile(t, q, q2);
+    const int idx = q * p + q2;
+    double v = summed ? sums[idx] : sum_chunks(sums, n_chunks(2 * N), p * p, idx);
     if (q == q2) v += wtt[q] + (sigma ? sigma[nz + q] : 0.0) + dw;
     A[(size_t)q2 * ld + q] = v;
   }
@@ -1990,7 +1999,7 @@ k_schur(DevProb P, const int* __restrict__ inert, const double* __restrict__ chu
         const double* __restrict__ wtt, const double* __restrict__ sigma, double dw,
         DevSchur S, int in_global) {
   extern __shared__ double sS[];
-  schur_block(P, inert, chunkS, wtt, sigma, dw, S, in_global ? S.S : sS);
+  schur_block(P, inert, chunkS, true, wtt, sigma, dw, S, in_global ? S.S : sS);
 }
 
 // ---- solves: one warp or a group of them per block -----------------------------------
@@ -2503,7 +2512,7 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
            const int* __restrict__ pre_elem, const int* __restrict__ pre_lv, int maxL,
            const int* __restrict__ pre_cs, const InstParams* __restrict__ prm,
            const int* __restrict__ flags, GridBar* gb, size_t smem_bytes, int bcr_full,
-           int slab_pb) {
+           int slab_pb, int totals) {
   extern __shared__ __align__(16) unsigned char smraw[];
   unsigned int ep = 0;
   // 1. element condensation: done by k_elem_factor_rt_b / k_elem_factor_big_b
@@ -2584,20 +2593,23 @@ k_factor_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A
   }
   grid_barrier(gb, ep);
   // ... their totals
-  for (int t = blockIdx.x * FBS + threadIdx.x; t < pre_cs[A]; t += gridDim.x * FBS) {
-    const int k = find_item(pre_cs, A, t);
-    const DevInst& I = insts[act[k]];
-    if (t - pre_cs[k] < I.P.p * I.P.p)
-      schur_total(inst_factor<T>(I).chunkS, I.P.N, I.P.p, t - pre_cs[k]);
+  if (totals) {
+    for (int t = blockIdx.x * FBS + threadIdx.x; t < pre_cs[A]; t += gridDim.x * FBS) {
+      const int k = find_item(pre_cs, A, t);
+      const DevInst& I = insts[act[k]];
+      if (t - pre_cs[k] < I.P.p * I.P.p && !schur_totals_inside(I.P.p))
+        schur_total(inst_factor<T>(I).chunkS, I.P.N, I.P.p, t - pre_cs[k]);
+    }
+    grid_barrier(gb, ep);
   }
-  grid_barrier(gb, ep);
   // 4. parameter Schur complement, one block per instance
   for (int k = blockIdx.x; k < A; k += gridDim.x) {
     const DevInst& I = insts[act[k]];
     const DevFactor<T>& F = inst_factor<T>(I);
     const size_t need = sizeof(double) * schur_doubles(I.P.p);
     double* sS = need <= smem_bytes ? reinterpret_cast<double*>(smraw) : I.S.S;
-    schur_block(I.P, F.inert, F.chunkS, I.E.wtt, I.sigma, prm[k].dw, I.S, sS);
+    schur_block(I.P, F.inert, F.chunkS, !schur_totals_inside(I.P.p), I.E.wtt, I.sigma, prm[k].dw, I.S,
+                sS);
     if (threadIdx.x == 0) {
       long long* o = reinterpret_cast<long long*>(I.out + O_INERT);
       o[0] = I.S.inertia[0]; o[1] = I.S.inertia[1]; o[2] = I.S.inertia[2];
@@ -2938,7 +2950,7 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
                             const int* pre_lv, int maxL, const int* pre_cs,
                             const InstParams* prm, const int* flags, GridBar* gb, size_t smem,
                             int grid_cap, int rt_threads, size_t rt_smem, int tot_elem,
-                            int big_grid, size_t big_smem, int bcr_tpt, int bcr_full, int parts,
+                            int big_grid, size_t big_smem, int bcr_tpt, int bcr_full, int max_p, int parts,
                             cudaStream_t st, int reserve) {
   if (A == 0) return cudaSuccess;
   if ((parts & 1) && rt_threads > 0 && tot_elem > 0) {
@@ -2982,8 +2994,9 @@ cudaError_t launch_factor_b(const DevInst* insts, const int* act, int A, const i
   int grid = coop_grid(kern, FBS, smem, grid_cap, reserve);
   if (grid < 1) return cudaErrorInvalidConfiguration;
   int slab_pb = sch.slab_pairs;
+  int totals = schur_totals_inside(max_p) ? 0 : 1;
   void* args[] = {(void*)&insts, (void*)&act, &A, (void*)&pre_elem, (void*)&pre_lv, &maxL,
-                  (void*)&pre_cs, (void*)&prm, (void*)&flags, &gb, &smem, &bcr_full, &slab_pb};
+                  (void*)&pre_cs, (void*)&prm, (void*)&flags, &gb, &smem, &bcr_full, &slab_pb, &totals};
   count_launch();
   return cudaLaunchCooperativeKernel((void*)kern, dim3(grid), dim3(FBS), args, smem, st);
 }
@@ -3023,11 +3036,11 @@ cudaError_t launch_solve_b(const DevInst* insts, const int* act, int A,
 template cudaError_t launch_factor_b<float>(const DevInst*, const int*, int, const int*,
                                             const int*, int, const int*, const InstParams*,
                                             const int*, GridBar*, size_t, int, int, size_t, int,
-                                            int, size_t, int, int, int, cudaStream_t, int);
+                                            int, size_t, int, int, int, int, cudaStream_t, int);
 template cudaError_t launch_factor_b<double>(const DevInst*, const int*, int, const int*,
                                              const int*, int, const int*, const InstParams*,
                                              const int*, GridBar*, size_t, int, int, size_t, int,
-                                             int, size_t, int, int, int, cudaStream_t, int);
+                                             int, size_t, int, int, int, int, cudaStream_t, int);
 int bcr_rt_tiles_of(const DevProb& P) { return bcr_rt_tiles(P.bext); }
 size_t elem_rt_stage_bytes(const DevProb& P, bool f32) {
   return f32 ? elem_stage_bytes<float>(P) : elem_stage_bytes<double>(P);

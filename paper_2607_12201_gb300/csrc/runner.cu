@@ -461,14 +461,14 @@ struct Runner {
                                  pl.pre_cs_s(), pl.d_prm, pl.flags(1), gbar, pl.smem_f[1],
                                  std::min(pl.cap_f[1], std::max(pl.tot_elem, pl.A)),
                                  pl.rt_threads[1], pl.rt_smem[1], pl.tot_elem, pl.big_grid[1],
-                                 pl.big_smem[1], pl.bcr_tpt, pl.bcr_full, parts, stream,
+                                 pl.big_smem[1], pl.bcr_tpt, pl.bcr_full, pl.max_p, parts, stream,
                                  reserve_sms);
     else
       e = launch_factor_b<double>(d_insts, pl.act(), pl.A, pl.pre_elem(), pl.pre_lv(), pl.maxL,
                                   pl.pre_cs_s(), pl.d_prm, pl.flags(0), gbar, pl.smem_f[0],
                                   std::min(pl.cap_f[0], std::max(pl.tot_elem, pl.A)),
                                   pl.rt_threads[0], pl.rt_smem[0], pl.tot_elem, pl.big_grid[0],
-                                  pl.big_smem[0], pl.bcr_tpt, pl.bcr_full, parts, stream,
+                                  pl.big_smem[0], pl.bcr_tpt, pl.bcr_full, pl.max_p, parts, stream,
                                   reserve_sms);
     COLLO_CUDA(e);
     return COLLO_OK;
