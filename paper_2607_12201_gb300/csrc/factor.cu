@@ -2677,6 +2677,16 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
       k = kn;
     }
   };
+  // a phase's wide and narrow blocks; a kind that no instance has is not looked for
+  // (a list's length is a read of the L2 on every level's path)
+  auto both = [&](const int* narrows, const int* wides, bool fwd, auto&& cols, auto&& one) {
+    if (pw > 0) {
+      list(wides, wg, nwg, wide, fwd, cols, one(wide));
+      sub_release();
+      __syncthreads();
+    }
+    if (pn > 0) list(narrows, gw, nw, narrow, fwd, cols, one(narrow));
+  };
   auto elems = [&](bool fwd) {
     auto cols = [&](const DevInst& I, int e) { return elem_cols(I.P, inst_factor<T>(I), e); };
     auto one = [&](auto& sm) {
@@ -2685,10 +2695,7 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
         else elem_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, e, sm, next);
       };
     };
-    list(sp.elem[1], wg, nwg, wide, fwd, cols, one(wide));
-    sub_release();
-    __syncthreads();
-    list(sp.elem[0], gw, nw, narrow, fwd, cols, one(narrow));
+    both(sp.elem[0], sp.elem[1], fwd, cols, one);
   };
   auto level = [&](int lv, bool fwd) {
     const size_t o = (size_t)lv * (A + 1);
@@ -2701,10 +2708,7 @@ k_solve_b(const DevInst* __restrict__ insts, const int* __restrict__ act, int A,
         else bcr_bwd_one(I.P, inst_factor<T>(I), I.S, ir ? I.kc : I.kb, 1 << lv, 0, bi, sm, next);
       };
     };
-    list(sp.lv[1] + o, wg, nwg, wide, fwd, cols, one(wide));
-    sub_release();
-    __syncthreads();
-    list(sp.lv[0] + o, gw, nw, narrow, fwd, cols, one(narrow));
+    both(sp.lv[0] + o, sp.lv[1] + o, fwd, cols, one);
   };
   // the levels from lsplit up of instance k, by this block
   auto top = [&](const DevInst& I, int k, int lv, bool fwd) {
