@@ -13,22 +13,6 @@
 
 namespace collo {
 
-cudaError_t launch_chunk_sums(const double* X, int C, int L, double* part, cudaStream_t st);
-
-
-__device__ inline double sum_chunks(const double* __restrict__ part, int G, int L, int l) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int g = 0;
-  for (; g + 3 < G; g += 4) {
-    a0 += part[(size_t)g * L + l];
-    a1 += part[(size_t)(g + 1) * L + l];
-    a2 += part[(size_t)(g + 2) * L + l];
-    a3 += part[(size_t)(g + 3) * L + l];
-  }
-  for (; g < G; ++g) a0 += part[(size_t)g * L + l];
-  return (a0 + a1) + (a2 + a3);
-}
-
 // Observation weights l_j(tau_m) (Lagrange basis on the element's
 // interpolation points) and the observation's element; one thread per
 // observation.

@@ -52,11 +52,6 @@ __device__ inline void cp_async_elem(T* dst, const T* src) {
 }
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-template <int N>
-__device__ inline void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // L columns of an eliminated block, unit lower, column-major: entry (row r,
 // column c), r > c, at p[c ld + r]; p 16-byte aligned, ld = factor_ld(rows).
 template <typename T>
