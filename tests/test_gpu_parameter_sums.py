@@ -1,6 +1,7 @@
 """The parameter block's right-hand side: sums over the chain's contributions by quads of
 lanes, at parameter counts that leave part of a warp idle and element counts whose number of
-partial sums (2 N up to 64) leaves a remainder to one lane."""
+partial sums (2 N up to 64) leaves a remainder to one lane; and the Schur complement's totals, by
+the block that factors it up to 22 parameters and by the grid above."""
 import numpy as np
 import pytest
 
@@ -22,7 +23,7 @@ def collo():
 
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("N", [1, 3, 17, 33])
-@pytest.mark.parametrize("p", [2, 3, 11, 21, 67])
+@pytest.mark.parametrize("p", [2, 3, 11, 21, 22, 23, 67])
 def test_solution_before_refinement(collo, p, N, mode):
     """FP64, no refinement.  A lost or doubled partial sum leaves a residual of the size of the
     parameter rows' right-hand side; rounding, with pivots that are not searched for, stays
