@@ -596,7 +596,7 @@ typedef struct collo_schedule {
   int solve_top_blocks;       /* the batched solve runs the reduction levels with
                                  at most this many blocks per instance in one CUDA
                                  block per instance (default 8; a block above 128
-                                 rows, which takes all eight warps, counts as
+                                 rows, which takes up to eight warps, counts as
                                  eight) */
   int solve_elems_per_block;  /* elements per 8-warp block of the solve's grid
                                  (default 8) */
